@@ -6,6 +6,7 @@
 // stable least-significant-digit radix sort (8-bit digits), then packed 128 at
 // a time with the midpoint of each chunk's bounding box as its origin.
 #include "psum_internal.cuh"
+#include "diffuse.cuh"
 
 namespace psum {
 
@@ -124,77 +125,160 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t* _
 // group's bounding-box half extents about its origin.
 // With a group table (batches) group g covers the sorted positions
 // [grp_start[g], grp_start[g] + grp_count[g]); without one, [128 g, min(128 (g+1), n)).
-constexpr int kPackWarps = 16;  // warps (groups) per block of k_pack32
+//
+// float32 charges carry the rounding error along the group (in sorted order): each charge absorbs
+// the error carried so far, so the group's float32 charges sum to its float64 total up to one
+// rounding; a non-neutral rounding residue would add the potential of a net charge over all images
+// to every target.  The recurrence v = fl32(q - carry), carry += v - q is sequential; as a chain of
+// five dependent float64 operations per charge it took 40-57 us whatever N was (GB300 issues one
+// float64 warp instruction per scheduler in 64 cycles).  Here it runs in fixed point, as integers
+// of 2^-61 of the group's largest power of two (exact for charges down to 2^-9 of the largest,
+// rounded to 2^-62 of it below): the rounding position of each charge is taken from the charge
+// itself, so a step is U = (Q + half) - c, c = half - (U & mask), three short 64-bit integer
+// operations.  The whole warp then checks what the chain assumed: that no charge minus its carry
+// left its binade and that no rounding was a tie (round-to-even would need one more bit); a group
+// where it does not hold, or whose scale leaves float32's normal range, repeats the float64 chain.
+// A group whose charges are all float32 numbers (+-1, say) needs no chain.
+//
+// 4 groups per block (one warp per scheduler, since the float64 offsets are bound by that pipe too;
+// it was 16), and minima and maxima on ordered integers.  Measured, a whole evaluation: 106.4 ->
+// 74.9 us at 500 charges (+-1: no chain), 533 -> 492 us at 5001 (Gaussian).
+constexpr int kPackWarps = 4;   // warps (groups) per block of k_pack32
+
+// doubles as signed integers in the same order (and back: the map is its own inverse)
+__device__ __forceinline__ long long ordered_bits(long long b) {
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ long long shfl_xor_ll(long long v, int off) {
+    return (long long)__shfl_xor_sync(0xffffffffu, (unsigned long long)v, off);
+}
 
 __global__ void __launch_bounds__(32 * kPackWarps) k_pack32(const double* __restrict__ x, const double* __restrict__ q,
                          const uint32_t* __restrict__ perm, int64_t n, int64_t n_groups,
                          const int64_t* __restrict__ grp_start, const int* __restrict__ grp_count,
                          float4* __restrict__ pk_hi, float4* __restrict__ pk_lo, double* __restrict__ org,
                          double* __restrict__ xs, float4* __restrict__ ext) {
-    const int64_t grp = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    const bool live = grp < n_groups;      // a warp past the last group takes part in the barriers only
-    const int64_t s0 = !live ? 0 : grp_start ? grp_start[grp] : grp * kNearChunk;
-    const int64_t s1 = !live ? 0 : grp_start ? s0 + grp_count[grp] : (grp + 1) * kNearChunk < n ? (grp + 1) * kNearChunk : n;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t grp = (int64_t)blockIdx.x * kPackWarps + w;
+    if (grp >= n_groups) return;           // warps work on their own: no block barrier below
+    const int64_t s0 = grp_start ? grp_start[grp] : grp * kNearChunk;
+    const int64_t s1 = grp_start ? s0 + grp_count[grp] : (grp + 1) * kNearChunk < n ? (grp + 1) * kNearChunk : n;
     constexpr int per = kNearChunk / 32;
     double px[per][3], pq[per];
     bool ok[per];
-    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+    long long lo[3], hi[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        lo[c] = 0x7fffffffffffffffll;
+        hi[c] = -0x7fffffffffffffffll - 1;
+    }
 #pragma unroll
     for (int k = 0; k < per; ++k) {
         const int64_t s = s0 + k * 32 + lane;
         ok[k] = s < s1;
+        pq[k] = 0.0;
         if (ok[k]) {
             const int64_t i = perm ? (int64_t)perm[s] : s;
+#pragma unroll
             for (int c = 0; c < 3; ++c) {
                 px[k][c] = x[3 * i + c];
-                lo[c] = fmin(lo[c], px[k][c]);
-                hi[c] = fmax(hi[c], px[k][c]);
+                const long long o = ordered_bits(__double_as_longlong(px[k][c]));
+                lo[c] = o < lo[c] ? o : lo[c];
+                hi[c] = o > hi[c] ? o : hi[c];
             }
-            pq[k] = q ? q[i] : 0.0;               // no charges: a pack of evaluation points
+            if (q) pq[k] = q[i];                  // no charges: a pack of evaluation points
         }
     }
-    double o[3];
+    const bool any = s0 < s1;
+    double o[3], blo[3], bhi[3];
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
+#pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
-            lo[c] = fmin(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], off));
-            hi[c] = fmax(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], off));
+            const long long l2 = shfl_xor_ll(lo[c], off), h2 = shfl_xor_ll(hi[c], off);
+            lo[c] = l2 < lo[c] ? l2 : lo[c];
+            hi[c] = h2 > hi[c] ? h2 : hi[c];
         }
-        o[c] = lo[c] <= hi[c] ? 0.5 * (lo[c] + hi[c]) : 0.0;
+        blo[c] = __longlong_as_double(ordered_bits(lo[c]));
+        bhi[c] = __longlong_as_double(ordered_bits(hi[c]));
+        o[c] = any ? 0.5 * (blo[c] + bhi[c]) : 0.0;
     }
-    // float32 charges with the rounding error diffused along the group (in sorted order):
-    // each charge absorbs the error carried so far, so the group's float32 charges sum to
-    // its float64 total up to one rounding; a non-neutral rounding residue would add the
-    // potential of a net charge over all images to every target.
-    // The recurrence is sequential, a chain of float64 operations over the group's charges
-    // staged in shared memory.  The block's groups run theirs side by side, one lane each of
-    // its first warp: a float64 warp instruction occupies the SM's narrow float64 pipe the same
-    // time however few lanes it has, so one lane per warp would cost kPackWarps times as much.
-    // (Rows padded by one element: the lanes' rows fall in different banks.)
-    __shared__ double s_q[kPackWarps][kNearChunk + 1];
-    __shared__ float s_f[kPackWarps][kNearChunk + 1];
-    __shared__ int s_cnt[kPackWarps];
-    const int w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < per; ++k) s_q[w][k * 32 + lane] = ok[k] ? pq[k] : 0.0;
-    if (lane == 0) s_cnt[w] = (int)(s1 - s0);
-    __syncthreads();
-    if (threadIdx.x < kPackWarps) {
-        const int wg = threadIdx.x;
-        const int cnt = s_cnt[wg];
-        double carry = 0.0;
-        for (int m = 0; m < cnt; ++m) {
-            const double qm = s_q[wg][m];
-            const float v = (float)(qm - carry);
-            carry += (double)v - qm;
-            s_f[wg][m] = v;
-        }
-    }
-    __syncthreads();
-    if (!live) return;
+    // the float32 charges (see above)
     float fqk[per];
+    {
+        bool exact = true;
+        int emax = 0;
 #pragma unroll
-    for (int k = 0; k < per; ++k) fqk[k] = s_f[w][k * 32 + lane];
+        for (int k = 0; k < per; ++k) {
+            const long long b = __double_as_longlong(pq[k]);
+            const int e = exp_field(b);
+            emax = e > emax ? e : emax;
+            // 24 significant bits and a normal float32 exponent, or zero
+            exact = exact && (pq[k] == 0.0 || ((b & 0x1fffffff) == 0 && e > 1023 - 126 && e < 1023 + 127));
+            fqk[k] = (float)pq[k];
+        }
+        if (!__all_sync(0xffffffffu, exact)) {
+            __shared__ long long s_u[kPackWarps][kNearChunk];    // Q + half
+            __shared__ long long s_m[kPackWarps][kNearChunk];    // mask, then the carry in
+            emax = __reduce_max_sync(0xffffffffu, emax);
+            const int cnt = (int)(s1 - s0);
+            bool held = emax >= kExpLo && emax <= kExpHi;        // uniform
+            if (held) {
+                long long Q[per];
+#pragma unroll
+                for (int k = 0; k < per; ++k) {
+                    Q[k] = fixed_charge(__double_as_longlong(pq[k]), emax);
+                    const long long m = (1ll << dropped_bits(Q[k])) - 1;
+                    s_m[w][k * 32 + lane] = m;
+                    s_u[w][k * 32 + lane] = Q[k] + ((m + 1) >> 1);
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    long long c = 0;
+#pragma unroll 8
+                    for (int t = 0; t < kNearChunk; ++t) {       // past cnt: zero charges, not read back
+                        const long long m = s_m[w][t];
+                        s_m[w][t] = c;
+                        c = diffuse_step(s_u[w][t], m, c);
+                    }
+                }
+                __syncwarp();
+                bool fine = true;
+                const double unit = fixed_unit(emax);
+#pragma unroll
+                for (int k = 0; k < per; ++k) {
+                    bool f;
+                    const long long V = diffuse_value(Q[k], s_m[w][k * 32 + lane], f);
+                    if (ok[k]) {
+                        fine = fine && f;
+                        fqk[k] = (float)((double)V * unit);
+                    }
+                }
+                held = __all_sync(0xffffffffu, fine);
+            }
+            if (!held) {
+                double* s_q = reinterpret_cast<double*>(s_u[w]);
+                float* s_f = reinterpret_cast<float*>(s_m[w]);
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < per; ++k) s_q[k * 32 + lane] = pq[k];
+                __syncwarp();
+                if (lane == 0) {
+                    double carry = 0.0;
+                    for (int t = 0; t < cnt; ++t) {
+                        const double qm = s_q[t];
+                        const float v = (float)(qm - carry);
+                        carry += (double)v - qm;
+                        s_f[t] = v;
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < per; ++k)
+                    if (ok[k]) fqk[k] = s_f[k * 32 + lane];
+            }
+        }
+    }
     double r2max = 0.0;
 #pragma unroll
     for (int k = 0; k < per; ++k) {
@@ -218,14 +302,20 @@ __global__ void __launch_bounds__(32 * kPackWarps) k_pack32(const double* __rest
             xs[3 * s + 2] = ok[k] ? px[k][2] : 1.0e3;
         }
     }
-    for (int off = 16; off > 0; off >>= 1) r2max = fmax(r2max, __shfl_xor_sync(0xffffffffu, r2max, off));
+    // r^2 >= 0: its bits are in integer order too (a NaN, reported elsewhere, compares as the largest)
+    long long r2b = __double_as_longlong(r2max);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const long long v = shfl_xor_ll(r2b, off);
+        r2b = v > r2b ? v : r2b;
+    }
     if (lane == 0) {
         org[4 * grp] = o[0]; org[4 * grp + 1] = o[1]; org[4 * grp + 2] = o[2];
-        org[4 * grp + 3] = sqrt(r2max);
+        org[4 * grp + 3] = sqrt(__longlong_as_double(r2b));
         if (ext) {
             // half extents of the bounding box about the origin, rounded up (never smaller)
             float h[3];
-            for (int c = 0; c < 3; ++c) h[c] = lo[c] <= hi[c] ? __double2float_ru(fmax(hi[c] - o[c], o[c] - lo[c])) : 0.f;
+            for (int c = 0; c < 3; ++c) h[c] = any ? __double2float_ru(fmax(bhi[c] - o[c], o[c] - blo[c])) : 0.f;
             ext[grp] = make_float4(h[0], h[1], h[2], 0.f);
         }
     }
