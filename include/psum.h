@@ -337,10 +337,10 @@ int psum_check_form(psum_plan_t plan, int *form);
  * PSUM_NUM_STAGES durations (milliseconds) of the last evaluation:
  *   [0] validation, spatial sort and packing
  *   [1] near-field sum at the charges (potential and gradient)
- *   [2] the charges' reduction, and what is left of the check-point sums and the box mean:
- *       those run on an internal stream of the lowest priority from the end of [0], beside
- *       the charge sum, and fill the SMs it releases as it finishes
- *   [3] right-hand side, least squares and C_1
+ *   [2] the charges' reduction
+ *   [3] what is left of the check-point sums, the least squares, the box mean and C_1: those
+ *       run on internal streams of the lowest priority from the end of [0] (the mean from its
+ *       start), beside the charge sum, and fill the SMs it releases as it finishes
  *   [4] far field, combination and write-back
  * Returns PSUM_ERR_ARG if profiling is off. */
 #define PSUM_NUM_STAGES 5

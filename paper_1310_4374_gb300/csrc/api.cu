@@ -56,6 +56,9 @@ __global__ void k_status_merge(const int* eval_status, int* plan_status) {
     if (*eval_status) atomicOr(plan_status, *eval_status);
 }
 
+// ints of an evaluation's flags: the status word and the pair launches' work-item counters
+constexpr int kFlags = 8;
+
 struct Layout {
     // FP32C
     uint32_t *ka, *va, *kb, *vb, *hist;
@@ -66,7 +69,7 @@ struct Layout {
     // FP64
     double4_32a* pk64;
     // common
-    double *part_n, *part_c, *phi_n, *grad_n, *phi_c, *val_part, *mean_part, *f;
+    double *part_n, *part_c, *phi_n, *grad_n, *phi_c, *val_part, *mean_part;
     int* eval_status;
     // backward
     double *far_phi, *far_grad, *w_part, *w, *u, *psi, *gpsi, *part_b;
@@ -114,6 +117,7 @@ NearSymLaunch sym_band_launch(const Layout& L, int64_t k, bool inject, int64_t d
     S.W = sym_sys_items(b);
     S.G = std::min(L.S.G, S.W);
     S.inject = inject ? 1 : 0;
+    S.zeroed = k == 0;               // queue_forward zeroes the counters once
     return S;
 }
 
@@ -251,14 +255,14 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
     L.nblk_mean = mean_blocks(N, pl.num_sms);
     L.val_part = b.take<double>(2 * (size_t)L.nblk_val);
     L.mean_part = b.take<double>((size_t)L.nblk_mean);
-    L.f = b.take<double>((size_t)pl.opt.M);
     // the status word and the pair launches' work-item counters
-    int* flags = b.take<int>(8);
+    int* flags = b.take<int>(kFlags);
     L.eval_status = flags;
     L.Ln.counter = flags + 1;
     L.Lc.counter = flags + 2;
     L.Ln.status = L.Lc.status = flags;
     L.Ln.n_status = L.Lc.n_status = 1;
+    L.Ln.zeroed = L.Lc.zeroed = true;   // queue_forward zeroes the flags once
     L.S.counter = flags + 1;
     L.S.status = flags;
     L.S.n_status = 1;
@@ -348,14 +352,17 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     const bool ff = o.precision == PSUM_FF;
     const int M = o.M, P = pl.P;
     if (h->profile) TRY(cudaEventRecord(h->ev[0], st));
+    // the status word and the work-item counters start at zero; every other buffer is written
+    // before it is read
+    TRY(cudaMemsetAsync(L.eval_status, 0, kFlags * sizeof(int), st));
     // the block's box mean needs only the caller's charges: on the second side stream (least
     // urgent priority) from the start, beside validation, sort and packing; the ball's mean
     // reads the sorted order and forks with the check sums below
     const bool zero_mean = o.mean_mode == PSUM_MEAN_ZERO;
     const bool early_mean = zero_mean && !(pl.Rb > 0.0);
+    if (early_mean || sep) TRY(cudaEventRecord(h->fork0, st));
     if (early_mean) {
         cudaStream_t s2 = h->side2;
-        TRY(cudaEventRecord(h->fork0, st));
         TRY(cudaStreamWaitEvent(s2, h->fork0, 0));
         const double H[3] = {0.5 * (2 * o.K[0] + 1) * o.d[0], 0.5 * (2 * o.K[1] + 1) * o.d[1],
                              0.5 * (2 * o.K[2] + 1) * o.d[2]};
@@ -363,43 +370,48 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
         TRY(cudaEventRecord(h->join2, s2));
         h->launches += 1;
     }
-    // the status word must start at zero; every other buffer is written before it is read
-    TRY(cudaMemsetAsync(L.eval_status, 0, sizeof(int), st));
-    TRY(launch_validate(x, q, N, o.d, L.val_part, L.nblk_val, L.eval_status, st));
-    h->launches += 2;
+    // separate evaluation points: validated, sorted and packed like the charges, without charges,
+    // beside them on the first side stream
+    const double* ex = sep ? y : x;              // evaluation points, caller order
+    const int* eperm = nullptr;
+    if (sep) {
+        cudaStream_t sp = h->side;
+        TRY(cudaStreamWaitEvent(sp, h->fork0, 0));
+        TRY(launch_prepare(y, nullptr, T, o.d, nullptr, reduce_blocks(T, pl.num_sms), L.eval_status,
+                           fp32 ? L.tkb : nullptr, sp));
+        if (fp32) {
+            TRY(launch_curve_order(T, L.tka, L.tva, L.tkb, L.tvb, L.thist, sp));
+            eperm = (const int*)L.tva;
+            TRY(launch_pack32(y, nullptr, L.tva, T, L.n_tiles * kTgt32, L.tpk32, L.tpk32lo, L.torg, sp));
+            h->launches += 1 + curve_order_launches(T) + 1;
+        } else {
+            TRY(launch_pack64(y, nullptr, T, L.n_pts, L.tpk64, sp));
+            h->launches += 2;
+        }
+        TRY(cudaEventRecord(h->join, sp));
+    }
     const int* perm = nullptr;
+    TRY(launch_prepare(x, q, N, o.d, L.val_part, L.nblk_val, L.eval_status, fp32 ? L.kb : nullptr, st));
     if (fp32) {
-        TRY(launch_curve_sort(x, N, o.d, L.ka, L.va, L.kb, L.vb, L.hist, st));
+        TRY(launch_curve_order(N, L.ka, L.va, L.kb, L.vb, L.hist, st));
         perm = (const int*)L.va;
         TRY(launch_pack32(x, q, L.va, N, L.n_src_groups, L.pk32, L.pk32lo, L.org, st, L.xs, L.ext));
-        h->launches += curve_sort_launches(N) + 1;
+        h->launches += 1 + curve_order_launches(N) + 1;
     } else {
         TRY(launch_pack64(x, q, N, L.n_src_pts, L.pk64, st));
-        h->launches += 1;
+        h->launches += 2;
     }
-    // separate evaluation points: validated, sorted and packed like the charges, without charges
-    const double* ex = sep ? y : x;              // evaluation points, caller order
-    const int* eperm = perm;
-    if (sep) {
-        TRY(launch_validate_points(y, T, o.d, L.nblk_val, L.eval_status, st));
-        h->launches += 1;
-        if (fp32) {
-            TRY(launch_curve_sort(y, T, o.d, L.tka, L.tva, L.tkb, L.tvb, L.thist, st));
-            eperm = (const int*)L.tva;
-            TRY(launch_pack32(y, nullptr, L.tva, T, L.n_tiles * kTgt32, L.tpk32, L.tpk32lo, L.torg, st));
-            h->launches += curve_sort_launches(T) + 1;
-        } else {
-            TRY(launch_pack64(y, nullptr, T, L.n_pts, L.tpk64, st));
-            h->launches += 1;
-        }
-    }
+    if (sep)
+        TRY(cudaStreamWaitEvent(st, h->join, 0));
+    else
+        eperm = perm;
     const float4* thi = sep ? L.tpk32 : L.pk32;
     const float4* tlo = sep ? L.tpk32lo : L.pk32lo;
     const double* tor = sep ? L.torg : L.org;
     const double4_32a* t64 = sep ? L.tpk64 : L.pk64;
     if (h->profile) TRY(cudaEventRecord(h->ev[1], st));
     // fork: the side stream (least urgent priority) waits for the packing, then takes the
-    // check-point sums, their reduction and the box mean while the charge kernel runs first
+    // check-point sums, their reduction, the fit and the constant while the charge kernel runs first
     TRY(cudaEventRecord(h->fork, st));
     if (L.sym) {
         // band by band: the pair kernel writes the band's slots, the reduction adds them to the
@@ -449,7 +461,6 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     const int tile = fp32 ? kTile32 : kTile64;
     TRY(launch_near_reduce(L.part_c, layers ? (int64_t)pl.lc_tiles * tile : pl.n_check, tile, 1, L.Lc, L.phi_c,
                            nullptr, sd));
-    TRY(cudaEventRecord(h->join, sd));
     // the ball's box mean on the second side stream, beside the check sums
     if (zero_mean && !early_mean) {
         cudaStream_t s2 = h->side2;
@@ -458,32 +469,31 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
         TRY(cudaEventRecord(h->join2, s2));
         h->launches += 1;
     }
+    // the fit and the constant follow the check sums and the mean, beside the charge kernel
+    TRY(launch_project(pl.d_pinv, P - 1, M, L.phi_c, layers ? pl.d_lc_pos : pl.d_check_pos, pl.d_C, sd, layers));
+    if (zero_mean) TRY(cudaStreamWaitEvent(sd, h->join2, 0));
+    TRY(launch_constant(pl.d_C, pl.d_Rbox, P, L.mean_part, L.nblk_mean, 1.0 / (o.d[0] * o.d[1] * o.d[2]),
+                        zero_mean ? 1 : 0, L.val_part, L.nblk_val, L.eval_status, sd));
+    TRY(cudaEventRecord(h->join, sd));
     if (L.sym)
         TRY(launch_sym_reduce(L.part_n, N, sym_band_launch(L, L.sym_bands - 1, false, h->debug_limit), L.phi_n,
                               L.grad_n, st, !fp32, L.sym_bands > 1));
     else
         TRY(launch_near_reduce(L.part_n, sep ? T : N, tile, 4, L.Ln, L.phi_n, L.grad_n, st));
     h->launches += 4;   // two near-field kernels, two reductions
-    // join: the fit needs the check sums and the mean
-    TRY(cudaStreamWaitEvent(st, h->join, 0));
-    if (zero_mean) TRY(cudaStreamWaitEvent(st, h->join2, 0));
     if (h->profile) TRY(cudaEventRecord(h->ev[3], st));
-    TRY(launch_project(pl.d_pinv, P - 1, M, L.phi_c, layers ? pl.d_lc_pos : pl.d_check_pos, L.f, pl.d_C, st,
-                       layers));
-    TRY(launch_constant(pl.d_C, pl.d_Rbox, P, L.mean_part, L.nblk_mean, 1.0 / (o.d[0] * o.d[1] * o.d[2]),
-                        zero_mean ? 1 : 0, st));
+    // join: the far field needs the coefficients
+    TRY(cudaStreamWaitEvent(st, h->join, 0));
     if (h->profile) TRY(cudaEventRecord(h->ev[4], st));
     const int64_t NE = sep ? T : N;
     if (o.basis == PSUM_BASIS_RBF)
         TRY(launch_far_rbf(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C, pl.d_rbf, pl.P - 1,
-                           L.eval_status, phi, grad, L.eval_status, st));
+                           L.eval_status, phi, grad, L.eval_status, pl.d_status, st));
     else
         TRY(launch_far_combine(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C, o.p, 1.0 / pl.R0,
                                pl.d_shtab64, o.precision == PSUM_FP32C ? pl.d_shtab32 : nullptr, L.eval_status,
-                               phi, grad, L.eval_status, st));
-    k_status_merge<<<1, 1, 0, st>>>(L.eval_status, pl.d_status);
-    TRY(cudaGetLastError());
-    h->launches += 5;   // right-hand side, projection, constant, far field, status merge
+                               phi, grad, L.eval_status, pl.d_status, st));
+    h->launches += 3;   // projection, constant, far field
     if (h->profile) TRY(cudaEventRecord(h->ev[5], st));
     return PSUM_OK;
 }
@@ -530,7 +540,7 @@ int backward_device(psum_plan_s* h, int64_t N, const double* x, const double* q,
         TRY(launch_curve_sort(x, N, o.d, L.ka, L.va, L.kb, L.vb, L.hist, st));
         perm = (const int*)L.va;
         TRY(launch_pack32(x, q, L.va, N, L.n_src_groups, L.pk32, L.pk32lo, L.org, st));
-        h->launches += curve_sort_launches(N) + 1;
+        h->launches += 1 + curve_order_launches(N) + 1;
     } else {
         TRY(launch_pack64(x, q, N, L.n_src_pts, L.pk64, st));
         h->launches += 1;

@@ -111,14 +111,7 @@ __global__ void __launch_bounds__(kSeg) k_bcurve_keys(const double* __restrict__
     const BatchDev& S = sys[b];
     const int64_t i = seg_start[seg] + threadIdx.x;
     if (i >= S.n0 + S.n) return;
-    uint32_t c[3];
-    for (int k = 0; k < 3; ++k) {
-        const double u = (x[3 * i + k] / S.d[k] + 0.5) * 256.0;
-        int v = (int)floor(u);
-        v = v < 0 ? 0 : (v > 255 ? 255 : v);
-        c[k] = (uint32_t)v;
-    }
-    keys[i] = (prefix ? (uint32_t)b << 24 : 0u) | hilbert_key24(c[0], c[1], c[2]);
+    keys[i] = (prefix ? (uint32_t)b << 24 : 0u) | curve_key(x + 3 * i, S.d);
     vals[i] = (uint32_t)i;
 }
 

@@ -35,50 +35,38 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
 
 constexpr int kRedThreads = 256;
 
-// Eq. 1: charges must sum to zero; positions must lie in [-d/2, d/2).
-__global__ void __launch_bounds__(kRedThreads) k_validate(const double* __restrict__ x, const double* __restrict__ q,
-                                                          int64_t n, double d0, double d1, double d2,
-                                                          double* __restrict__ partial, int* __restrict__ status) {
+// Eq. 1: charges must sum to zero; positions must lie in [-d/2, d/2).  Without charges (kCharges
+// false): evaluation points, inside the half-open box and finite.  `keys` (optional) receives the
+// points' places on the spatial curve, so that validation adds no launch before the sort.
+template <bool kCharges>
+__global__ void __launch_bounds__(kRedThreads) k_prepare(const double* __restrict__ x, const double* __restrict__ q,
+                                                         int64_t n, double d0, double d1, double d2,
+                                                         double* __restrict__ partial, int* __restrict__ status,
+                                                         uint32_t* __restrict__ keys) {
+    const double d[3] = {d0, d1, d2};
     double s = 0.0, sa = 0.0;
     int bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads) {
-        const double a = x[3 * i], b = x[3 * i + 1], c = x[3 * i + 2], qi = q[i];
+        const double a = x[3 * i], b = x[3 * i + 1], c = x[3 * i + 2];
         const bool in = (a >= -0.5 * d0) && (a < 0.5 * d0) && (b >= -0.5 * d1) && (b < 0.5 * d1) &&
                         (c >= -0.5 * d2) && (c < 0.5 * d2);
         if (!in) bad |= kStatOutOfBox;           // also catches NaN positions
-        if (!(fabs(qi) <= 1.7976931348623157e308)) bad |= kStatNonFinite;
-        s += qi;
-        sa += fabs(qi);
+        if (keys) keys[i] = curve_key(x + 3 * i, d);
+        if constexpr (kCharges) {
+            const double qi = q[i];
+            if (!(fabs(qi) <= 1.7976931348623157e308)) bad |= kStatNonFinite;
+            s += qi;
+            sa += fabs(qi);
+        }
     }
     if (bad) atomicOr(status, bad);
-    block_sum2<kRedThreads>(s, sa);
-    if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = s;
-        partial[2 * blockIdx.x + 1] = sa;
+    if constexpr (kCharges) {
+        block_sum2<kRedThreads>(s, sa);
+        if (threadIdx.x == 0) {
+            partial[2 * blockIdx.x] = s;
+            partial[2 * blockIdx.x + 1] = sa;
+        }
     }
-}
-
-// Evaluation points: inside the half-open box and finite, like the charges.
-__global__ void __launch_bounds__(kRedThreads) k_validate_points(const double* __restrict__ y, int64_t n, double d0,
-                                                                 double d1, double d2, int* __restrict__ status) {
-    int bad = 0;
-    for (int64_t i = (int64_t)blockIdx.x * kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads) {
-        const double a = y[3 * i], b = y[3 * i + 1], c = y[3 * i + 2];
-        const bool in = (a >= -0.5 * d0) && (a < 0.5 * d0) && (b >= -0.5 * d1) && (b < 0.5 * d1) &&
-                        (c >= -0.5 * d2) && (c < 0.5 * d2);
-        if (!in) bad |= kStatOutOfBox;
-    }
-    if (bad) atomicOr(status, bad);
-}
-
-__global__ void k_validate_finish(const double* __restrict__ partial, int nblk, int* __restrict__ status) {
-    double s = 0.0, sa = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += 32) { s += partial[2 * b]; sa += partial[2 * b + 1]; }
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_down_sync(0xffffffffu, s, o);
-        sa += __shfl_down_sync(0xffffffffu, sa, o);
-    }
-    if (threadIdx.x == 0 && !(fabs(s) <= 1e-12 * sa)) atomicOr(status, kStatNonNeutral);
 }
 
 // One (charge, term) pair per work item: sum_i q_i U(x_i) with U the regrouped corner sum
@@ -164,39 +152,57 @@ __global__ void __launch_bounds__(kRedThreads) k_box_mean_ball(const double* __r
 // ---------------------------------------------------------------------------
 constexpr int kProjThreads = 256;
 
-// f_l = phi_near(y~_l) - phi_near(y_l); with `layers` the check sums already hold the
-// difference (the two image layers at y_l), at packed position check_pos[l].
-__global__ void k_rhs(const double* __restrict__ phi_check, const int* __restrict__ check_pos, int M,
-                      int layers, double* __restrict__ f) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l < M) f[l] = layers ? phi_check[check_pos[l]] : phi_check[check_pos[M + l]] - phi_check[check_pos[l]];
-}
-
+// With `layers` the check sums already hold the difference (the two image layers at y_l), at
+// packed position check_pos[l].  Each row gathers f itself (it stays in cache): no launch for it.
 __global__ void __launch_bounds__(kProjThreads) k_project(const double* __restrict__ pinv, int rows, int M,
-                                                          const double* __restrict__ f, double* __restrict__ C) {
+                                                          const double* __restrict__ phi_check,
+                                                          const int* __restrict__ check_pos, int layers,
+                                                          double* __restrict__ C) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * (kProjThreads / 32) + w;
     if (row >= rows) return;
     const double* a = pinv + (int64_t)row * M;
     double s = 0.0;
-    for (int l = lane; l < M; l += 32) s = fma(a[l], f[l], s);
+#pragma unroll 4
+    for (int l = lane; l < M; l += 32) {
+        const double f = layers ? phi_check[check_pos[l]] : phi_check[check_pos[M + l]] - phi_check[check_pos[l]];
+        s = fma(a[l], f, s);
+    }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) C[1 + row] = s;
 }
 
-// Step 6 (Eq. pfx3 with phi_mean = 0): C_1 = -<phi_near> - sum_{t>=2} C_t R_t^(0).
-__global__ void k_constant(double* __restrict__ C, const double* __restrict__ Rbox, int P,
-                           const double* __restrict__ mean_partial, int nblk, double inv_V0, int zero_mean) {
-    double s = 0.0, m = 0.0;
+// Step 6 (Eq. pfx3 with phi_mean = 0): C_1 = -<phi_near> - sum_{t>=2} C_t R_t^(0); and the end of
+// the validation: the charges' total against their absolute sum (Eq. 1).
+__global__ void __launch_bounds__(kRedThreads) k_constant(double* __restrict__ C, const double* __restrict__ Rbox,
+                                                          int P, const double* __restrict__ mean_partial, int nblk,
+                                                          double inv_V0, int zero_mean,
+                                                          const double* __restrict__ val_partial, int nblk_val,
+                                                          int* __restrict__ status) {
+    double s = 0.0, m = 0.0, qs = 0.0, qa = 0.0;
     if (zero_mean) {
-        for (int t = 1 + threadIdx.x; t < P; t += 32) s = fma(C[t], Rbox[t], s);
-        for (int b = threadIdx.x; b < nblk; b += 32) m += mean_partial[b];
+        for (int t = 1 + threadIdx.x; t < P; t += kRedThreads) s = fma(C[t], Rbox[t], s);
+        for (int b = threadIdx.x; b < nblk; b += kRedThreads) m += mean_partial[b];
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_down_sync(0xffffffffu, s, o);
-        m += __shfl_down_sync(0xffffffffu, m, o);
+    for (int b = threadIdx.x; b < nblk_val; b += kRedThreads) {
+        qs += val_partial[2 * b];
+        qa += val_partial[2 * b + 1];
     }
+    block_sum2<kRedThreads>(s, m);
     if (threadIdx.x == 0) C[0] = zero_mean ? (-m * inv_V0 - s) : 0.0;
+    __syncthreads();                           // block_sum2's shared sums are free again
+    block_sum2<kRedThreads>(qs, qa);
+    if (threadIdx.x == 0 && !(fabs(qs) <= 1e-12 * qa)) atomicOr(status, kStatNonNeutral);
+}
+
+// The evaluation's status joins the plan's (psum_sync reads it): what was flagged before this
+// kernel by its first thread, what a thread finds itself at once.
+__device__ __forceinline__ void merge_status(const int* status, int* plan_status) {
+    if (blockIdx.x == 0 && threadIdx.x == 0 && *status) atomicOr(plan_status, *status);
+}
+__device__ __forceinline__ void flag_nonfinite(int* status, int* plan_status) {
+    atomicOr(status, kStatNonFinite);
+    atomicOr(plan_status, kStatNonFinite);
 }
 
 // ---------------------------------------------------------------------------
@@ -217,7 +223,8 @@ __global__ void __launch_bounds__(kFarThreads) k_far_combine(const double* __res
                                                              const T* __restrict__ tab,
                                                              const int* __restrict__ status,
                                                              double* __restrict__ phi, double* __restrict__ grad,
-                                                             int* __restrict__ status_out) {
+                                                             int* __restrict__ status_out, int* __restrict__ plan_status) {
+    merge_status(status, plan_status);
     extern __shared__ unsigned char s_raw[];
     const int P = (p + 1) * (p + 1);
     const int nt = sh_tab_size(p);
@@ -264,7 +271,7 @@ __global__ void __launch_bounds__(kFarThreads) k_far_combine(const double* __res
         finite = finite && fabs(g0) <= 1.7976931348623157e308 && fabs(g1) <= 1.7976931348623157e308 &&
                  fabs(g2) <= 1.7976931348623157e308;
     }
-    if (!finite) atomicOr(status_out, kStatNonFinite);
+    if (!finite) flag_nonfinite(status_out, plan_status);
 }
 
 // Steps 7-8 with the RBF basis of Eq. 5: phi_far(y) = C_1 + sum_t C_{t+1} / |y - x_t| and
@@ -283,7 +290,8 @@ __global__ void __launch_bounds__(kFarThreads) k_far_rbf(const double* __restric
                                                          const double* __restrict__ centres, int S,
                                                          const int* __restrict__ status,
                                                          double* __restrict__ phi, double* __restrict__ grad,
-                                                         int* __restrict__ status_out) {
+                                                         int* __restrict__ status_out, int* __restrict__ plan_status) {
+    merge_status(status, plan_status);
     __shared__ double4_32a s_c[kRbfBlock];
     const int64_t s = (int64_t)blockIdx.x * kFarThreads + threadIdx.x;
     const bool live = s < n;
@@ -330,7 +338,7 @@ __global__ void __launch_bounds__(kFarThreads) k_far_rbf(const double* __restric
         finite = finite && fabs(g0) <= 1.7976931348623157e308 && fabs(g1) <= 1.7976931348623157e308 &&
                  fabs(g2) <= 1.7976931348623157e308;
     }
-    if (!finite) atomicOr(status_out, kStatNonFinite);
+    if (!finite) flag_nonfinite(status_out, plan_status);
 }
 
 // ---------------------------------------------------------------------------
@@ -338,14 +346,14 @@ __global__ void __launch_bounds__(kFarThreads) k_far_rbf(const double* __restric
 // ---------------------------------------------------------------------------
 cudaError_t launch_far_rbf(const double* x, int64_t n, const int* perm, const double* phi_near,
                            const double* grad_near, const double* C, const double* centres, int S, const int* status,
-                           double* phi, double* grad, int* status_out, cudaStream_t st) {
+                           double* phi, double* grad, int* status_out, int* plan_status, cudaStream_t st) {
     const unsigned nb = (unsigned)((n + kFarThreads - 1) / kFarThreads);
     if (grad)
         k_far_rbf<true><<<nb, kFarThreads, 0, st>>>(x, n, perm, phi_near, grad_near, C, centres, S, status, phi,
-                                                    grad, status_out);
+                                                    grad, status_out, plan_status);
     else
         k_far_rbf<false><<<nb, kFarThreads, 0, st>>>(x, n, perm, phi_near, grad_near, C, centres, S, status, phi,
-                                                     grad, status_out);
+                                                     grad, status_out, plan_status);
     return cudaGetLastError();
 }
 
@@ -356,16 +364,12 @@ int reduce_blocks(int64_t n, int num_sms) {
     return nb < 1 ? 1 : (int)nb;
 }
 
-cudaError_t launch_validate_points(const double* y, int64_t n, const double d[3], int nblk, int* status,
-                                   cudaStream_t st) {
-    k_validate_points<<<nblk, kRedThreads, 0, st>>>(y, n, d[0], d[1], d[2], status);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_validate(const double* x, const double* q, int64_t n, const double d[3], double* partial,
-                            int nblk, int* status, cudaStream_t st) {
-    k_validate<<<nblk, kRedThreads, 0, st>>>(x, q, n, d[0], d[1], d[2], partial, status);
-    k_validate_finish<<<1, 32, 0, st>>>(partial, nblk, status);
+cudaError_t launch_prepare(const double* x, const double* q, int64_t n, const double d[3], double* partial, int nblk,
+                           int* status, uint32_t* keys, cudaStream_t st) {
+    if (q)
+        k_prepare<true><<<nblk, kRedThreads, 0, st>>>(x, q, n, d[0], d[1], d[2], partial, status, keys);
+    else
+        k_prepare<false><<<nblk, kRedThreads, 0, st>>>(x, q, n, d[0], d[1], d[2], partial, status, keys);
     return cudaGetLastError();
 }
 
@@ -390,33 +394,34 @@ cudaError_t launch_box_mean_ball(const double* x, const double* q, const uint32_
 }
 
 cudaError_t launch_project(const double* pinv, int rows, int M, const double* phi_check, const int* check_pos,
-                           double* f, double* C, cudaStream_t st, bool layers) {
-    k_rhs<<<(M + 255) / 256, 256, 0, st>>>(phi_check, check_pos, M, layers ? 1 : 0, f);
+                           double* C, cudaStream_t st, bool layers) {
     const int per = kProjThreads / 32;
-    k_project<<<(rows + per - 1) / per, kProjThreads, 0, st>>>(pinv, rows, M, f, C);
+    k_project<<<(rows + per - 1) / per, kProjThreads, 0, st>>>(pinv, rows, M, phi_check, check_pos, layers ? 1 : 0, C);
     return cudaGetLastError();
 }
 
 cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean_partial, int nblk,
-                            double inv_V0, int zero_mean, cudaStream_t st) {
-    k_constant<<<1, 32, 0, st>>>(C, Rbox, P, mean_partial, nblk, inv_V0, zero_mean);
+                            double inv_V0, int zero_mean, const double* val_partial, int nblk_val, int* status,
+                            cudaStream_t st) {
+    k_constant<<<1, kRedThreads, 0, st>>>(C, Rbox, P, mean_partial, nblk, inv_V0, zero_mean, val_partial, nblk_val,
+                                          status);
     return cudaGetLastError();
 }
 
 cudaError_t launch_far_combine(const double* x, int64_t n, const int* perm, const double* phi_near,
                                const double* grad_near, const double* C, int p, double inv_R0, const double* tab64,
                                const float* tab32, const int* status, double* phi, double* grad, int* status_out,
-                               cudaStream_t st) {
+                               int* plan_status, cudaStream_t st) {
     const int P = (p + 1) * (p + 1);
     const unsigned nb = (unsigned)((n + kFarThreads - 1) / kFarThreads);
     if (tab32) {
         const size_t smem = sizeof(float) * (P + sh_tab_size(p));
         k_far_combine<float><<<nb, kFarThreads, smem, st>>>(x, n, perm, phi_near, grad_near, C, p, inv_R0, tab32,
-                                                            status, phi, grad, status_out);
+                                                            status, phi, grad, status_out, plan_status);
     } else {
         const size_t smem = sizeof(double) * (P + sh_tab_size(p));
         k_far_combine<double><<<nb, kFarThreads, smem, st>>>(x, n, perm, phi_near, grad_near, C, p, inv_R0, tab64,
-                                                             status, phi, grad, status_out);
+                                                             status, phi, grad, status_out, plan_status);
     }
     return cudaGetLastError();
 }

@@ -43,7 +43,9 @@ constexpr int kNear32Variants = 2;
 int near64_occupancy_ctas();
 // sort.cu
 int sort_blocks(int64_t n);
-int curve_sort_launches(int64_t n);   // kernels launch_curve_sort queues for n points
+int curve_order_launches(int64_t n);   // kernels launch_curve_order queues for n points
+cudaError_t launch_curve_order(int64_t n, uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, uint32_t* hist,
+                               cudaStream_t st);
 cudaError_t launch_curve_sort(const double* x, int64_t n, const double d[3], uint32_t* ka, uint32_t* va,
                                uint32_t* kb, uint32_t* vb, uint32_t* hist, cudaStream_t st);
 cudaError_t launch_pack32(const double* x, const double* q, const uint32_t* perm, int64_t n, int64_t n_groups,
@@ -51,7 +53,7 @@ cudaError_t launch_pack32(const double* x, const double* q, const uint32_t* perm
                           float4* ext = nullptr);
 cudaError_t launch_pack64(const double* x, const double* q, int64_t n, int64_t n_pad, double4_32a* pk, cudaStream_t st);
 cudaError_t launch_radix_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, uint32_t* hist, int64_t n,
-                              int passes, cudaStream_t st);
+                              int passes, cudaStream_t st, uint32_t* spare = nullptr);
 cudaError_t launch_pack32_groups(const double* x, const double* q, const uint32_t* perm, int64_t n_groups,
                                  const int64_t* grp_start, const int* grp_count, float4* pk_hi, float4* pk_lo,
                                  double* org, cudaStream_t st, float4* ext = nullptr);
@@ -59,30 +61,31 @@ cudaError_t launch_pack64_groups(const double* x, const double* q, int64_t n_pts
                                  const int* grp_count, double4_32a* pk, cudaStream_t st);
 // far.cu
 int reduce_blocks(int64_t n, int num_sms);
-cudaError_t launch_validate_points(const double* y, int64_t n, const double d[3], int nblk, int* status,
-                                   cudaStream_t st);
-cudaError_t launch_validate(const double* x, const double* q, int64_t n, const double d[3], double* partial,
-                            int nblk, int* status, cudaStream_t st);
+// validation of the charges (q) or of evaluation points (q null), with their curve keys where
+// `keys` is given; launch_constant finishes the charges' neutrality test
+cudaError_t launch_prepare(const double* x, const double* q, int64_t n, const double d[3], double* partial, int nblk,
+                           int* status, uint32_t* keys, cudaStream_t st);
 int mean_blocks(int64_t n, int num_sms);   // grid of launch_box_mean for n charges
 cudaError_t launch_box_mean(const double* x, const double* q, int64_t n, const double H[3], double* partial,
                             int nblk, cudaStream_t st);
 // far field of the RBF basis (Eq. 5): phi = phi_near + C_1 + sum_t C_{t+1} / |y - x_t|, float64
 cudaError_t launch_far_rbf(const double* x, int64_t n, const int* perm, const double* phi_near,
                            const double* grad_near, const double* C, const double* centres, int S, const int* status,
-                           double* phi, double* grad, int* status_out, cudaStream_t st);
+                           double* phi, double* grad, int* status_out, int* plan_status, cudaStream_t st);
 // trimmed near set: sum over the kept images x + p (|x + p| <= Rb) of the single box's potential
 cudaError_t launch_box_mean_ball(const double* x, const double* q, const uint32_t* perm, int64_t n,
                                  const double d[3], const int K[3], double Rb, double* partial, int nblk,
                                  cudaStream_t st);
 cudaError_t launch_project(const double* pinv, int rows, int M, const double* phi_check, const int* check_pos,
-                           double* f, double* C, cudaStream_t st, bool layers = false);
+                           double* C, cudaStream_t st, bool layers = false);
 cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean_partial, int nblk,
-                            double inv_V0, int zero_mean, cudaStream_t st);
+                            double inv_V0, int zero_mean, const double* val_partial, int nblk_val, int* status,
+                            cudaStream_t st);
 // tab32 != nullptr: the far field in float (FP32C plans), else in double with tab64
 cudaError_t launch_far_combine(const double* x, int64_t n, const int* perm, const double* phi_near,
                                const double* grad_near, const double* C, int p, double inv_R0, const double* tab64,
                                const float* tab32, const int* status, double* phi, double* grad, int* status_out,
-                               cudaStream_t st);
+                               int* plan_status, cudaStream_t st);
 // backward.cu
 cudaError_t launch_moments(const double* x, const double* q, int64_t n, const double* C, int p, double inv_R0,
                            const double* tab, double* far_phi, double* far_grad, double* w_partial, int nblk,

@@ -719,7 +719,7 @@ cudaError_t launch_near32(bool grad, const float4* src_hi, const float4* src_lo,
     a.n_cls = n_cls;
     const size_t smem = near32_dyn_smem(L.max_img, Rb > 0.0, grad, n_cls);
     if (!L.counter) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaMemsetAsync(L.counter, 0, sizeof(int), st);
+    const cudaError_t e = L.zeroed ? cudaSuccess : cudaMemsetAsync(L.counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     const unsigned G = (unsigned)L.G;
     const auto kernel = near32_instance(grad, variant, Rb > 0.0, ff);
@@ -738,7 +738,7 @@ cudaError_t launch_near64(bool grad, const double4_32a* src, const double4_32a* 
     a.img_w = img_w; a.n_cls = n_cls;
     a.U = L.U; a.W = L.W; a.counter = L.counter; a.max_contrib = L.max_contrib; a.tab = L.tab;
     if (!L.counter) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaMemsetAsync(L.counter, 0, sizeof(int), st);
+    const cudaError_t e = L.zeroed ? cudaSuccess : cudaMemsetAsync(L.counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     if (grad)
         k_near64<true><<<(unsigned)L.G, kThreads64, 0, st>>>(a);

@@ -1097,7 +1097,7 @@ cudaError_t launch_near32s(const float4* pk_hi, const float4* pk_lo, const doubl
     a.tab = S.tab; a.W = S.W; a.max_ipg = S.max_ipg;
     a.counter = S.counter; a.status = S.status; a.n_status = S.n_status; a.inject = S.inject;
     a.limit = sym_limit(S);
-    const cudaError_t e = cudaMemsetAsync(S.counter, 0, sizeof(int), st);
+    const cudaError_t e = S.zeroed ? cudaSuccess : cudaMemsetAsync(S.counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     const size_t smem = near32s_dyn_smem(S.max_ipg);
     if (ff)
@@ -1149,7 +1149,7 @@ cudaError_t launch_near64s(const double4_32a* pk, const double* shifts, double* 
     Near64SymArgs a;
     a.pk = pk; a.shifts = shifts; a.partial = partial; a.tab = S.tab; a.W = S.W; a.counter = S.counter;
     a.status = S.status; a.n_status = S.n_status; a.limit = sym_limit(S);
-    const cudaError_t e = cudaMemsetAsync(S.counter, 0, sizeof(int), st);
+    const cudaError_t e = S.zeroed ? cudaSuccess : cudaMemsetAsync(S.counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     k_near64s<kNear64sMinBlocks><<<(unsigned)S.G, kThreads64, 0, st>>>(a);
     return cudaGetLastError();

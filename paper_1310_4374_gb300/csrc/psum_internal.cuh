@@ -69,6 +69,19 @@ __host__ __device__ __forceinline__ uint32_t hilbert_key24(uint32_t c0, uint32_t
     return (spread3_8(X[0]) << 2) | (spread3_8(X[1]) << 1) | spread3_8(X[2]);
 }
 
+// the key of a position in the box d (a position outside it, NaN included, maps into range: it is
+// reported by the validation)
+__device__ __forceinline__ uint32_t curve_key(const double* __restrict__ p, const double d[3]) {
+    uint32_t c[3];
+    for (int k = 0; k < 3; ++k) {
+        const double u = (p[k] / d[k] + 0.5) * 256.0;
+        int v = (int)floor(u);
+        v = v < 0 ? 0 : (v > 255 ? 255 : v);
+        c[k] = (uint32_t)v;
+    }
+    return hilbert_key24(c[0], c[1], c[2]);
+}
+
 // two-layer check points: flag in a group's class mask for a group of padding alone
 constexpr int kGroupEmpty = 1 << 30;
 
@@ -457,6 +470,7 @@ struct NearPlanLaunch {
     int64_t U, G;
     int64_t W;                    // work items
     int* counter = nullptr;       // device int, zeroed by the launcher before each launch
+    bool zeroed = false;          // ... unless the caller's own stream order has zeroed it already
     int* status = nullptr;        // device error words the pair kernel may flag (kStatTimeout)
     int n_status = 0;
     int inject = 0;               // test hook: arm the chunk-copy barrier for bytes that never come
@@ -542,6 +556,7 @@ struct NearSymLaunch {
     int max_ipg = 0;               // largest images per group (shared-memory sizing)
     size_t doubles = 0;            // partial buffer
     int* counter = nullptr;
+    bool zeroed = false;           // the caller has zeroed the counter (see NearPlanLaunch)
     int* status = nullptr;
     int n_status = 0;
     int inject = 0;

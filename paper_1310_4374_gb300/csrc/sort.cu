@@ -17,19 +17,11 @@ constexpr int kSortTile = kSortThreads * kSortPerThread;   // 2048 keys per bloc
 constexpr int kRadix = 256;
 
 __global__ void k_curve_keys(const double* __restrict__ x, int64_t n, double d0, double d1, double d2,
-                         uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+                             uint32_t* __restrict__ keys) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double dd[3] = {d0, d1, d2};
-    uint32_t c[3];
-    for (int k = 0; k < 3; ++k) {
-        double u = (x[3 * i + k] / dd[k] + 0.5) * 256.0;
-        int v = (int)floor(u);
-        v = v < 0 ? 0 : (v > 255 ? 255 : v);      // also maps NaN (validated elsewhere) into range
-        c[k] = (uint32_t)v;
-    }
-    keys[i] = hilbert_key24(c[0], c[1], c[2]);
-    vals[i] = (uint32_t)i;
+    const double d[3] = {d0, d1, d2};
+    keys[i] = curve_key(x + 3 * i, d);
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __restrict__ keys, int64_t n, int shift,
@@ -111,7 +103,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t* _
         __syncwarp();
         if (valid) {
             kout[pos] = key;
-            vout[pos] = vin[i];
+            vout[pos] = vin ? vin[i] : (uint32_t)i;     // no values: the input positions
         }
     }
 }
@@ -359,9 +351,10 @@ int sort_blocks(int64_t n) { return (int)((n + kSortTile - 1) / kSortTile); }
 
 // Stable LSD radix sort of (key, value) pairs, 8 bits per pass over `passes` passes,
 // ping-ponging (ka, va) -> (kb, vb) -> ...: the result ends in (ka, va) after an even
-// number of passes and in (kb, vb) after an odd one; hist is scratch.
+// number of passes and in (kb, vb) after an odd one; hist is scratch.  With va null the values are
+// the input positions, and the passes after the first ping-pong between vb and `spare`.
 cudaError_t launch_radix_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, uint32_t* hist, int64_t n,
-                              int passes, cudaStream_t st) {
+                              int passes, cudaStream_t st, uint32_t* spare) {
     const int nblk = sort_blocks(n);
     uint32_t *ki = ka, *vi = va, *ko = kb, *vo = vb;
     for (int pass = 0; pass < passes; ++pass) {
@@ -370,61 +363,82 @@ cudaError_t launch_radix_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t
         k_sort_scan<<<1, 1024, 0, st>>>(hist, (int64_t)kRadix * nblk);
         k_sort_scatter<<<nblk, kSortThreads, 0, st>>>(ki, vi, n, shift, hist, nblk, ko, vo);
         uint32_t* t = ki; ki = ko; ko = t;
-        t = vi; vi = vo; vo = t;
+        t = vi ? vi : spare;
+        vi = vo;
+        vo = t;
     }
     return cudaGetLastError();
 }
 
-// Small inputs in one block: the (key, index) pairs as 64-bit words in shared memory, a
-// bitonic sort, the same order as the stable radix sort (ties broken by the index), in one
-// launch instead of nine.
-constexpr int kSmallSort = 4096;
-constexpr int kSmallSortThreads = 1024;
+// Small inputs by counting: a point's place is the number of points before it in (key, index)
+// order, the order of the stable radix sort.  A block ranks 32 points, one per lane; its 16 warps
+// count over every 16th block of four keys, which all lanes read as one 16-byte broadcast, and the
+// warps' counts are added in shared memory.  n^2 compares at two instructions each stay below the
+// radix sort's nine dependent launches (about 65 us at any size up to 1e5) until some 3e4 points;
+// measured in a whole evaluation against the sorts it replaces: see kRankMax.
+constexpr int kRankWarps = 16;
+constexpr int kRankPoints = 32;
 
-__global__ void __launch_bounds__(kSmallSortThreads) k_sort_small(const uint32_t* __restrict__ kin,
-                                                                  const uint32_t* __restrict__ vin, int n,
-                                                                  uint32_t* __restrict__ kout,
-                                                                  uint32_t* __restrict__ vout) {
-    __shared__ unsigned long long w[kSmallSort];
-    int m = 1;
-    while (m < n) m <<= 1;
-    for (int i = threadIdx.x; i < m; i += kSmallSortThreads)
-        w[i] = i < n ? ((unsigned long long)kin[i] << 32) | vin[i] : ~0ull;
+__global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const uint32_t* __restrict__ keys, int n,
+                                                                uint32_t* __restrict__ perm) {
+    __shared__ int s_cnt[kRankWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * kRankPoints, i = i0 + lane;
+    const uint32_t key = i < n ? keys[i] : 0u;
+    const uint4* k4 = reinterpret_cast<const uint4*>(keys);   // the key buffer starts on 256 bytes
+    const int n4 = n >> 2, own = i0 >> 2;                     // whole blocks of four; the block's own eight
+    int c = 0;
+    // points before the block's own: an equal key counts; after them: it does not
+#pragma unroll 8
+    for (int j = w; j < own; j += kRankWarps) {
+        const uint4 k = k4[j];
+        c += (k.x <= key) + (k.y <= key) + (k.z <= key) + (k.w <= key);
+    }
+#pragma unroll 8
+    for (int j = own + kRankPoints / 4 + w; j < n4; j += kRankWarps) {
+        const uint4 k = k4[j];
+        c += (k.x < key) + (k.y < key) + (k.z < key) + (k.w < key);
+    }
+    if (w == 0)
+        for (int j = i0; j < i0 + kRankPoints && j < n; ++j) c += keys[j] < key || (keys[j] == key && j < i);
+    // keys past the last whole block of four, unless they are the block's own
+    if (w == 1 && (n4 << 2) >= i0 + kRankPoints)
+        for (int j = n4 << 2; j < n; ++j) c += keys[j] < key;
+    s_cnt[w][lane] = c;
     __syncthreads();
-    for (int k = 2; k <= m; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < m; i += kSmallSortThreads) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const unsigned long long a = w[i], b = w[p];
-                    const bool up = (i & k) == 0;
-                    if ((a > b) == up) {
-                        w[i] = b;
-                        w[p] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    for (int i = threadIdx.x; i < n; i += kSmallSortThreads) {
-        kout[i] = (uint32_t)(w[i] >> 32);
-        vout[i] = (uint32_t)(w[i] & 0xffffffffu);
+    if (w == 0 && i < n) {
+        int r = 0;
+#pragma unroll
+        for (int k = 0; k < kRankWarps; ++k) r += s_cnt[k][lane];
+        perm[r] = (uint32_t)i;
     }
 }
 
-int curve_sort_launches(int64_t n) { return n <= kSmallSort ? 2 : 1 + 3 * 3; }
+// Where counting gives way to the radix sort.
+#ifndef PSUM_RANK_MAX
+#define PSUM_RANK_MAX 24576
+#endif
+constexpr int64_t kRankMax = PSUM_RANK_MAX;
 
-// Hilbert order of the points: 24-bit keys, written to (kb, vb) and sorted (3 radix passes,
-// or one block for small inputs) so that the sorted keys and the permutation end in (ka, va).
+int curve_order_launches(int64_t n) { return n <= kRankMax ? 1 : 3 * 3; }
+
+// The stable order of n points by their 24-bit keys (in kb, which is overwritten): the permutation
+// ends in va.
+cudaError_t launch_curve_order(int64_t n, uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, uint32_t* hist,
+                               cudaStream_t st) {
+    if (n <= kRankMax) {
+        k_rank_order<<<(unsigned)((n + kRankPoints - 1) / kRankPoints), 32 * kRankWarps, 0, st>>>(kb, (int)n, va);
+        return cudaGetLastError();
+    }
+    return launch_radix_sort(kb, nullptr, ka, va, hist, n, 3, st, vb);
+}
+
+// Keys and order of the points (callers whose keys do not come with the validation).
 cudaError_t launch_curve_sort(const double* x, int64_t n, const double d[3], uint32_t* ka, uint32_t* va,
                                uint32_t* kb, uint32_t* vb, uint32_t* hist, cudaStream_t st) {
     const int bs = 256;
-    k_curve_keys<<<(unsigned)((n + bs - 1) / bs), bs, 0, st>>>(x, n, d[0], d[1], d[2], kb, vb);
-    if (n <= kSmallSort) {
-        k_sort_small<<<1, kSmallSortThreads, 0, st>>>(kb, vb, (int)n, ka, va);
-        return cudaGetLastError();
-    }
-    return launch_radix_sort(kb, vb, ka, va, hist, n, 3, st);
+    k_curve_keys<<<(unsigned)((n + bs - 1) / bs), bs, 0, st>>>(x, n, d[0], d[1], d[2], kb);
+    return launch_curve_order(n, ka, va, kb, vb, hist, st);
 }
 
 cudaError_t launch_pack32(const double* x, const double* q, const uint32_t* perm, int64_t n, int64_t n_groups,
