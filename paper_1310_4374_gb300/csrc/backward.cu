@@ -162,10 +162,18 @@ __global__ void __launch_bounds__(kEnThreads) k_energy_partial(const double* __r
     }
 }
 
-__global__ void k_energy_finish(const double* __restrict__ partial, int nblk, double* __restrict__ E) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+// the partial sums in a fixed order: each thread every 256th, then the block as above
+__global__ void __launch_bounds__(kEnThreads) k_energy_finish(const double* __restrict__ partial, int nblk,
+                                                              double* __restrict__ E) {
+    __shared__ double sh[kEnThreads / 32];
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += kEnThreads) s += partial[b];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int b = 0; b < nblk; ++b) t += partial[b];
+        for (int w = 0; w < kEnThreads / 32; ++w) t += sh[w];
         *E = 0.5 * t;
     }
 }
@@ -223,7 +231,7 @@ cudaError_t launch_backward_combine(int64_t n, const int* perm, const double* q,
 cudaError_t launch_energy(const double* q, const double* phi, int64_t n, double* partial, int nblk, double* E,
                           cudaStream_t st) {
     k_energy_partial<<<nblk, kEnThreads, 0, st>>>(q, phi, n, partial);
-    k_energy_finish<<<1, 32, 0, st>>>(partial, nblk, E);
+    k_energy_finish<<<1, kEnThreads, 0, st>>>(partial, nblk, E);
     return cudaGetLastError();
 }
 

@@ -41,7 +41,7 @@ struct BatchDev {
     int p, P, M, zero_mean;
     int layers;               // the check sums are the two-layer differences at the M points
     int seg0, nseg;
-    double d[3], H[3];
+    double d[3], inv_d256[3], H[3];
     double inv_V0, inv_R0;
 };
 
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kSeg) k_bcurve_keys(const double* __restrict__
     const BatchDev& S = sys[b];
     const int64_t i = seg_start[seg] + threadIdx.x;
     if (i >= S.n0 + S.n) return;
-    keys[i] = (prefix ? (uint32_t)b << 24 : 0u) | curve_key(x + 3 * i, S.d);
+    keys[i] = (prefix ? (uint32_t)b << 24 : 0u) | curve_key(x + 3 * i, S.d, S.inv_d256);
     vals[i] = (uint32_t)i;
 }
 
@@ -696,6 +696,7 @@ int psum_batch_create(const psum_plan_t* plans, int B, const int64_t* offsets, p
         S.nseg = (int)((n + kSeg - 1) / kSeg);
         for (int k = 0; k < 3; ++k) {
             S.d[k] = pl.opt.d[k];
+            S.inv_d256[k] = 256.0 / pl.opt.d[k];
             S.H[k] = 0.5 * (2 * pl.opt.K[k] + 1) * pl.opt.d[k];
         }
         S.inv_V0 = 1.0 / (pl.opt.d[0] * pl.opt.d[1] * pl.opt.d[2]);

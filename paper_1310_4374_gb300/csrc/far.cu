@@ -5,7 +5,8 @@
 //   the far field and its gradient at the charges and the final sum (steps 7-8,
 //   Eqs. 1.6-1.9).
 // All of it runs in float64.
-#include "psum_internal.cuh"
+#include "launch.cuh"
+#include "diffuse.cuh"
 #include "mean.cuh"
 
 namespace psum {
@@ -38,30 +39,40 @@ constexpr int kRedThreads = 256;
 // Eq. 1: charges must sum to zero; positions must lie in [-d/2, d/2).  Without charges (kCharges
 // false): evaluation points, inside the half-open box and finite.  `keys` (optional) receives the
 // points' places on the spatial curve, so that validation adds no launch before the sort.
+// The range test runs on ordered integers and the blocks are small: the float64 pipe of an SM is two
+// lanes wide, so a few large blocks would queue on a few SMs' pipes.
+constexpr int kPrepThreads = 64;
+
 template <bool kCharges>
-__global__ void __launch_bounds__(kRedThreads) k_prepare(const double* __restrict__ x, const double* __restrict__ q,
-                                                         int64_t n, double d0, double d1, double d2,
-                                                         double* __restrict__ partial, int* __restrict__ status,
-                                                         uint32_t* __restrict__ keys) {
-    const double d[3] = {d0, d1, d2};
+__global__ void __launch_bounds__(kPrepThreads) k_prepare(const double* __restrict__ x, const double* __restrict__ q,
+                                                          int64_t n, CurveBox box, double* __restrict__ partial,
+                                                          int* __restrict__ status, uint32_t* __restrict__ keys) {
+    long long lo[3], hi[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        lo[c] = ordered_bits(__double_as_longlong(-0.5 * box.d[c]));
+        hi[c] = ordered_bits(__double_as_longlong(0.5 * box.d[c]));
+    }
     double s = 0.0, sa = 0.0;
     int bad = 0;
-    for (int64_t i = (int64_t)blockIdx.x * kRedThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kRedThreads) {
-        const double a = x[3 * i], b = x[3 * i + 1], c = x[3 * i + 2];
-        const bool in = (a >= -0.5 * d0) && (a < 0.5 * d0) && (b >= -0.5 * d1) && (b < 0.5 * d1) &&
-                        (c >= -0.5 * d2) && (c < 0.5 * d2);
-        if (!in) bad |= kStatOutOfBox;           // also catches NaN positions
-        if (keys) keys[i] = curve_key(x + 3 * i, d);
+    for (int64_t i = (int64_t)blockIdx.x * kPrepThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kPrepThreads) {
+        const double p[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const long long b = ordered_bits(__double_as_longlong(p[c]));
+            if (!(b >= lo[c] && b < hi[c])) bad |= kStatOutOfBox;      // NaN positions too
+        }
+        if (keys) keys[i] = stored_key(p, box);
         if constexpr (kCharges) {
             const double qi = q[i];
-            if (!(fabs(qi) <= 1.7976931348623157e308)) bad |= kStatNonFinite;
+            if (exp_field(__double_as_longlong(qi)) == 0x7ff) bad |= kStatNonFinite;
             s += qi;
             sa += fabs(qi);
         }
     }
     if (bad) atomicOr(status, bad);
     if constexpr (kCharges) {
-        block_sum2<kRedThreads>(s, sa);
+        block_sum2<kPrepThreads>(s, sa);
         if (threadIdx.x == 0) {
             partial[2 * blockIdx.x] = s;
             partial[2 * blockIdx.x + 1] = sa;
@@ -358,8 +369,8 @@ cudaError_t launch_far_rbf(const double* x, int64_t n, const int* perm, const do
 }
 
 int reduce_blocks(int64_t n, int num_sms) {
-    int64_t nb = (n + kRedThreads - 1) / kRedThreads;
-    const int64_t cap = 4LL * num_sms;
+    int64_t nb = (n + kPrepThreads - 1) / kPrepThreads;
+    const int64_t cap = 16LL * num_sms;
     if (nb > cap) nb = cap;
     return nb < 1 ? 1 : (int)nb;
 }
@@ -367,9 +378,9 @@ int reduce_blocks(int64_t n, int num_sms) {
 cudaError_t launch_prepare(const double* x, const double* q, int64_t n, const double d[3], double* partial, int nblk,
                            int* status, uint32_t* keys, cudaStream_t st) {
     if (q)
-        k_prepare<true><<<nblk, kRedThreads, 0, st>>>(x, q, n, d[0], d[1], d[2], partial, status, keys);
+        k_prepare<true><<<nblk, kPrepThreads, 0, st>>>(x, q, n, curve_box(d, n), partial, status, keys);
     else
-        k_prepare<false><<<nblk, kRedThreads, 0, st>>>(x, q, n, d[0], d[1], d[2], partial, status, keys);
+        k_prepare<false><<<nblk, kPrepThreads, 0, st>>>(x, q, n, curve_box(d, n), partial, status, keys);
     return cudaGetLastError();
 }
 

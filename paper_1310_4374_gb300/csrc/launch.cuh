@@ -42,6 +42,21 @@ int near32s_occupancy_ctas(int img_per_g, bool ff = false, bool refine = false);
 constexpr int kNear32Variants = 2;
 int near64_occupancy_ctas();
 // sort.cu
+// The box as the keys need it, and how they are stored: as float32 numbers where the points are
+// ordered by counting (up to kRankMax of them; k_rank_order), as integers for the radix sort.  At
+// kRankMax points counting takes about half of the radix sort's nine launches.
+struct CurveBox {
+    double d[3], inv[3];
+    int as_float;
+};
+constexpr int64_t kRankMax = 24576;
+inline CurveBox curve_box(const double d[3], int64_t n) {
+    return CurveBox{{d[0], d[1], d[2]}, {256.0 / d[0], 256.0 / d[1], 256.0 / d[2]}, n <= kRankMax ? 1 : 0};
+}
+__device__ __forceinline__ uint32_t stored_key(const double* p, const CurveBox& box) {
+    const uint32_t k = curve_key(p, box.d, box.inv);
+    return box.as_float ? __float_as_uint((float)k) : k;
+}
 int sort_blocks(int64_t n);
 int curve_order_launches(int64_t n);   // kernels launch_curve_order queues for n points
 cudaError_t launch_curve_order(int64_t n, uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, uint32_t* hist,

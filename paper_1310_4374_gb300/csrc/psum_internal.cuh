@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <string.h>
+
 #include <cmath>
 #include <vector>
 
@@ -69,17 +71,32 @@ __host__ __device__ __forceinline__ uint32_t hilbert_key24(uint32_t c0, uint32_t
     return (spread3_8(X[0]) << 2) | (spread3_8(X[1]) << 1) | spread3_8(X[2]);
 }
 
-// the key of a position in the box d (a position outside it, NaN included, maps into range: it is
-// reported by the validation)
-__device__ __forceinline__ uint32_t curve_key(const double* __restrict__ p, const double d[3]) {
-    uint32_t c[3];
-    for (int k = 0; k < 3; ++k) {
-        const double u = (p[k] / d[k] + 0.5) * 256.0;
-        int v = (int)floor(u);
-        v = v < 0 ? 0 : (v > 255 ? 255 : v);
-        c[k] = (uint32_t)v;
-    }
-    return hilbert_key24(c[0], c[1], c[2]);
+// A double's bits as a signed integer in the same order (its own inverse): comparisons, minima and
+// maxima that need not go through the float64 pipe.  -0 sorts below +0, a NaN beyond the infinity of
+// its sign.
+__host__ __device__ __forceinline__ long long ordered_bits(long long b) {
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
+// The cells of a position along the curve's 256^3 grid, floor((x / d + 1/2) 256) in float64.  The
+// division alone is some twenty float64 operations; the cell is read off one multiply-add by 256/d
+// and one addition that leaves the result's fixed point (22 fraction bits) in the low word.  Both
+// forms agree to 2^-43 of a cell, so only a position within 2^-20 of a cell's face takes the
+// division.  A position outside the box, NaN included, maps into range: the validation reports it.
+__host__ __device__ __forceinline__ uint32_t curve_cell(double x, double d, double inv_d256) {
+    const double t = fma(x, inv_d256, 128.0) + 1610612736.0;      // 1.5 * 2^30: unit 2^-22 in the last place
+    long long b;
+    memcpy(&b, &t, sizeof b);
+    const uint32_t v = (uint32_t)b;
+    const uint32_t f = v & 0x3fffffu;
+    if (f - 4u < 0x3ffff8u) return (v >> 22) & 255u;
+    const double u = (x / d + 0.5) * 256.0;
+    const int c = (int)floor(u);
+    return (uint32_t)(c < 0 ? 0 : (c > 255 ? 255 : c));
+}
+__host__ __device__ __forceinline__ uint32_t curve_key(const double* p, const double d[3], const double inv[3]) {
+    return hilbert_key24(curve_cell(p[0], d[0], inv[0]), curve_cell(p[1], d[1], inv[1]),
+                         curve_cell(p[2], d[2], inv[2]));
 }
 
 // two-layer check points: flag in a group's class mask for a group of padding alone

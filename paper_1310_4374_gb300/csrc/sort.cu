@@ -5,7 +5,7 @@
 // ordered along the Hilbert curve of a 256^3 grid over the box (hilbert_key24) by a
 // stable least-significant-digit radix sort (8-bit digits), then packed 128 at
 // a time with the midpoint of each chunk's bounding box as its origin.
-#include "psum_internal.cuh"
+#include "launch.cuh"
 #include "diffuse.cuh"
 
 namespace psum {
@@ -16,12 +16,9 @@ constexpr int kSortPerThread = 8;
 constexpr int kSortTile = kSortThreads * kSortPerThread;   // 2048 keys per block
 constexpr int kRadix = 256;
 
-__global__ void k_curve_keys(const double* __restrict__ x, int64_t n, double d0, double d1, double d2,
-                             uint32_t* __restrict__ keys) {
+__global__ void k_curve_keys(const double* __restrict__ x, int64_t n, CurveBox box, uint32_t* __restrict__ keys) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double d[3] = {d0, d1, d2};
-    keys[i] = curve_key(x + 3 * i, d);
+    if (i < n) keys[i] = stored_key(x + 3 * i, box);
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __restrict__ keys, int64_t n, int shift,
@@ -108,7 +105,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t* _
     }
 }
 
-// One warp per group of kNearChunk sorted positions: the bounding-box midpoint is the
+// One block per group of kNearChunk sorted positions: the bounding-box midpoint is the
 // float64 origin, stored with the group radius (largest distance of a point from it);
 // each point's offset from the origin is split into a float32 hi part and the float32
 // rounding remainder lo, packed two float4 each: (x,x,y,y),(z,z,q,q) and (xl,xl,yl,yl),(zl,zl,ql,ql)
@@ -132,184 +129,169 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t* _
 // where it does not hold, or whose scale leaves float32's normal range, repeats the float64 chain.
 // A group whose charges are all float32 numbers (+-1, say) needs no chain.
 //
-// 4 groups per block (one warp per scheduler, since the float64 offsets are bound by that pipe too;
-// it was 16), and minima and maxima on ordered integers.  Measured, a whole evaluation: 106.4 ->
-// 74.9 us at 500 charges (+-1: no chain), 533 -> 492 us at 5001 (Gaussian).
-constexpr int kPackWarps = 4;   // warps (groups) per block of k_pack32
-
-// doubles as signed integers in the same order (and back: the map is its own inverse)
-__device__ __forceinline__ long long ordered_bits(long long b) {
-    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
+// A block of 128 threads packs one group, a point per thread: the offsets are some twenty operations
+// a point on the float64 pipe, which the four schedulers of an SM then share (a warp per group took
+// four times as long at small sizes).  Minima and maxima go over ordered integers.  Measured, a whole
+// evaluation: 106.4 -> 74.9 us at 500 charges (+-1: no chain), 533 -> 492 us at 5001 (Gaussian).
 __device__ __forceinline__ long long shfl_xor_ll(long long v, int off) {
     return (long long)__shfl_xor_sync(0xffffffffu, (unsigned long long)v, off);
 }
 
-__global__ void __launch_bounds__(32 * kPackWarps) k_pack32(const double* __restrict__ x, const double* __restrict__ q,
-                         const uint32_t* __restrict__ perm, int64_t n, int64_t n_groups,
+constexpr int kPackThreads = kNearChunk;
+
+__global__ void __launch_bounds__(kPackThreads) k_pack32(const double* __restrict__ x, const double* __restrict__ q,
+                         const uint32_t* __restrict__ perm, int64_t n,
                          const int64_t* __restrict__ grp_start, const int* __restrict__ grp_count,
                          float4* __restrict__ pk_hi, float4* __restrict__ pk_lo, double* __restrict__ org,
                          double* __restrict__ xs, float4* __restrict__ ext) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t grp = (int64_t)blockIdx.x * kPackWarps + w;
-    if (grp >= n_groups) return;           // warps work on their own: no block barrier below
+    constexpr int kWarps = kPackThreads / 32;
+    __shared__ long long s_box[kWarps][7];          // lows, highs, then r^2
+    __shared__ int s_emax[kWarps];
+    __shared__ long long s_u[kNearChunk];           // Q + half
+    __shared__ long long s_m[kNearChunk];           // mask, then the carry in
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int64_t grp = blockIdx.x;
     const int64_t s0 = grp_start ? grp_start[grp] : grp * kNearChunk;
     const int64_t s1 = grp_start ? s0 + grp_count[grp] : (grp + 1) * kNearChunk < n ? (grp + 1) * kNearChunk : n;
-    constexpr int per = kNearChunk / 32;
-    double px[per][3], pq[per];
-    bool ok[per];
+    const int cnt = s1 > s0 ? (int)(s1 - s0) : 0;
+    const bool ok = tid < cnt;
+    double px[3] = {0.0, 0.0, 0.0}, pq = 0.0;
     long long lo[3], hi[3];
+    if (ok) {
+        const int64_t i = perm ? (int64_t)perm[s0 + tid] : s0 + tid;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        lo[c] = 0x7fffffffffffffffll;
-        hi[c] = -0x7fffffffffffffffll - 1;
+        for (int c = 0; c < 3; ++c) px[c] = x[3 * i + c];
+        if (q) pq = q[i];                           // no charges: a pack of evaluation points
     }
 #pragma unroll
-    for (int k = 0; k < per; ++k) {
-        const int64_t s = s0 + k * 32 + lane;
-        ok[k] = s < s1;
-        pq[k] = 0.0;
-        if (ok[k]) {
-            const int64_t i = perm ? (int64_t)perm[s] : s;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                px[k][c] = x[3 * i + c];
-                const long long o = ordered_bits(__double_as_longlong(px[k][c]));
-                lo[c] = o < lo[c] ? o : lo[c];
-                hi[c] = o > hi[c] ? o : hi[c];
-            }
-            if (q) pq[k] = q[i];                  // no charges: a pack of evaluation points
-        }
-    }
-    const bool any = s0 < s1;
-    double o[3], blo[3], bhi[3];
-#pragma unroll
     for (int c = 0; c < 3; ++c) {
+        const long long o = ordered_bits(__double_as_longlong(px[c]));
+        lo[c] = ok ? o : 0x7fffffffffffffffll;
+        hi[c] = ok ? o : -0x7fffffffffffffffll - 1;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             const long long l2 = shfl_xor_ll(lo[c], off), h2 = shfl_xor_ll(hi[c], off);
             lo[c] = l2 < lo[c] ? l2 : lo[c];
             hi[c] = h2 > hi[c] ? h2 : hi[c];
         }
+        if (lane == 0) {
+            s_box[w][c] = lo[c];
+            s_box[w][3 + c] = hi[c];
+        }
+    }
+    const long long qb = __double_as_longlong(pq);
+    const int e = exp_field(qb);
+    {
+        const int em = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) s_emax[w] = em;
+    }
+    // 24 significant bits and a normal float32 exponent, or zero
+    const bool exact = pq == 0.0 || ((qb & 0x1fffffff) == 0 && e > 1023 - 126 && e < 1023 + 127);
+    const bool chain = !__syncthreads_and(exact);   // also: s_box and s_emax are written
+    double o[3], blo[3], bhi[3];
+    int emax = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        lo[c] = s_box[0][c];
+        hi[c] = s_box[0][3 + c];
+#pragma unroll
+        for (int k = 1; k < kWarps; ++k) {
+            lo[c] = s_box[k][c] < lo[c] ? s_box[k][c] : lo[c];
+            hi[c] = s_box[k][3 + c] > hi[c] ? s_box[k][3 + c] : hi[c];
+        }
         blo[c] = __longlong_as_double(ordered_bits(lo[c]));
         bhi[c] = __longlong_as_double(ordered_bits(hi[c]));
-        o[c] = any ? 0.5 * (blo[c] + bhi[c]) : 0.0;
+        o[c] = cnt > 0 ? 0.5 * (blo[c] + bhi[c]) : 0.0;
     }
-    // the float32 charges (see above)
-    float fqk[per];
-    {
-        bool exact = true;
-        int emax = 0;
 #pragma unroll
-        for (int k = 0; k < per; ++k) {
-            const long long b = __double_as_longlong(pq[k]);
-            const int e = exp_field(b);
-            emax = e > emax ? e : emax;
-            // 24 significant bits and a normal float32 exponent, or zero
-            exact = exact && (pq[k] == 0.0 || ((b & 0x1fffffff) == 0 && e > 1023 - 126 && e < 1023 + 127));
-            fqk[k] = (float)pq[k];
-        }
-        if (!__all_sync(0xffffffffu, exact)) {
-            __shared__ long long s_u[kPackWarps][kNearChunk];    // Q + half
-            __shared__ long long s_m[kPackWarps][kNearChunk];    // mask, then the carry in
-            emax = __reduce_max_sync(0xffffffffu, emax);
-            const int cnt = (int)(s1 - s0);
-            bool held = emax >= kExpLo && emax <= kExpHi;        // uniform
-            if (held) {
-                long long Q[per];
-#pragma unroll
-                for (int k = 0; k < per; ++k) {
-                    Q[k] = fixed_charge(__double_as_longlong(pq[k]), emax);
-                    const long long m = (1ll << dropped_bits(Q[k])) - 1;
-                    s_m[w][k * 32 + lane] = m;
-                    s_u[w][k * 32 + lane] = Q[k] + ((m + 1) >> 1);
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    long long c = 0;
+    for (int k = 0; k < kWarps; ++k) emax = s_emax[k] > emax ? s_emax[k] : emax;
+    // the float32 charge (see above)
+    float fq = (float)pq;
+    if (chain) {
+        bool held = emax >= kExpLo && emax <= kExpHi;        // uniform
+        if (held) {
+            const long long Q = fixed_charge(qb, emax);
+            {
+                const long long m = (1ll << dropped_bits(Q)) - 1;
+                s_m[tid] = m;
+                s_u[tid] = Q + ((m + 1) >> 1);
+            }
+            __syncthreads();
+            if (tid == 0) {
+                long long c = 0;
 #pragma unroll 8
-                    for (int t = 0; t < kNearChunk; ++t) {       // past cnt: zero charges, not read back
-                        const long long m = s_m[w][t];
-                        s_m[w][t] = c;
-                        c = diffuse_step(s_u[w][t], m, c);
-                    }
+                for (int t = 0; t < kNearChunk; ++t) {       // past cnt: zero charges, not read back
+                    const long long m = s_m[t];
+                    s_m[t] = c;
+                    c = diffuse_step(s_u[t], m, c);
                 }
-                __syncwarp();
-                bool fine = true;
-                const double unit = fixed_unit(emax);
-#pragma unroll
-                for (int k = 0; k < per; ++k) {
-                    bool f;
-                    const long long V = diffuse_value(Q[k], s_m[w][k * 32 + lane], f);
-                    if (ok[k]) {
-                        fine = fine && f;
-                        fqk[k] = (float)((double)V * unit);
-                    }
-                }
-                held = __all_sync(0xffffffffu, fine);
             }
-            if (!held) {
-                double* s_q = reinterpret_cast<double*>(s_u[w]);
-                float* s_f = reinterpret_cast<float*>(s_m[w]);
-                __syncwarp();
-#pragma unroll
-                for (int k = 0; k < per; ++k) s_q[k * 32 + lane] = pq[k];
-                __syncwarp();
-                if (lane == 0) {
-                    double carry = 0.0;
-                    for (int t = 0; t < cnt; ++t) {
-                        const double qm = s_q[t];
-                        const float v = (float)(qm - carry);
-                        carry += (double)v - qm;
-                        s_f[t] = v;
-                    }
+            __syncthreads();
+            bool fine;
+            const long long V = diffuse_value(Q, s_m[tid], fine);
+            fq = (float)((double)V * fixed_unit(emax));
+            held = __syncthreads_and(fine || !ok);
+        }
+        if (!held) {
+            double* s_q = reinterpret_cast<double*>(s_u);
+            float* s_f = reinterpret_cast<float*>(s_m);
+            s_q[tid] = pq;
+            __syncthreads();
+            if (tid == 0) {
+                double carry = 0.0;
+                for (int t = 0; t < cnt; ++t) {
+                    const double qm = s_q[t];
+                    const float v = (float)(qm - carry);
+                    carry += (double)v - qm;
+                    s_f[t] = v;
                 }
-                __syncwarp();
-#pragma unroll
-                for (int k = 0; k < per; ++k)
-                    if (ok[k]) fqk[k] = s_f[k * 32 + lane];
             }
+            __syncthreads();
+            fq = s_f[tid];
         }
     }
-    double r2max = 0.0;
-#pragma unroll
-    for (int k = 0; k < per; ++k) {
-        const int64_t s = grp * kNearChunk + k * 32 + lane;
-        float fx = 1.0e3f, fy = 1.0e3f, fz = 1.0e3f, fq = 0.f, lx = 0.f, ly = 0.f, lz = 0.f, lq = 0.f;
-        if (ok[k]) {
-            const double rx = px[k][0] - o[0], ry = px[k][1] - o[1], rz = px[k][2] - o[2];
-            r2max = fmax(r2max, rx * rx + ry * ry + rz * rz);
+    double r2 = 0.0;
+    const int64_t s = grp * kNearChunk + tid;
+    {
+        float fx = 1.0e3f, fy = 1.0e3f, fz = 1.0e3f, fc = 0.f, lx = 0.f, ly = 0.f, lz = 0.f, lq = 0.f;
+        if (ok) {
+            const double rx = px[0] - o[0], ry = px[1] - o[1], rz = px[2] - o[2];
+            r2 = rx * rx + ry * ry + rz * rz;
             fx = (float)rx; fy = (float)ry; fz = (float)rz;
             lx = (float)(rx - (double)fx); ly = (float)(ry - (double)fy); lz = (float)(rz - (double)fz);
-            fq = fqk[k];
-            lq = (float)(pq[k] - (double)fq);     // the charge's float-float remainder (FF pair sums)
+            fc = fq;
+            lq = (float)(pq - (double)fq);        // the charge's float-float remainder (FF pair sums)
         }
         pk_hi[2 * s] = make_float4(fx, fx, fy, fy);
-        pk_hi[2 * s + 1] = make_float4(fz, fz, fq, fq);
+        pk_hi[2 * s + 1] = make_float4(fz, fz, fc, fc);
         pk_lo[2 * s] = make_float4(lx, lx, ly, ly);
         pk_lo[2 * s + 1] = make_float4(lz, lz, lq, lq);
-        if (xs) {
-            xs[3 * s] = ok[k] ? px[k][0] : 1.0e3;
-            xs[3 * s + 1] = ok[k] ? px[k][1] : 1.0e3;
-            xs[3 * s + 2] = ok[k] ? px[k][2] : 1.0e3;
-        }
     }
-    // r^2 >= 0: its bits are in integer order too (a NaN, reported elsewhere, compares as the largest)
-    long long r2b = __double_as_longlong(r2max);
+    if (xs) {
+        xs[3 * s] = ok ? px[0] : 1.0e3;
+        xs[3 * s + 1] = ok ? px[1] : 1.0e3;
+        xs[3 * s + 2] = ok ? px[2] : 1.0e3;
+    }
+    // r^2 >= 0: its bits are in integer order too (a NaN, reported elsewhere, counts as 0)
+    long long r2b = r2 >= 0.0 ? __double_as_longlong(r2) : 0ll;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         const long long v = shfl_xor_ll(r2b, off);
         r2b = v > r2b ? v : r2b;
     }
-    if (lane == 0) {
+    if (lane == 0) s_box[w][6] = r2b;
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+        for (int k = 1; k < kWarps; ++k) r2b = s_box[k][6] > r2b ? s_box[k][6] : r2b;
         org[4 * grp] = o[0]; org[4 * grp + 1] = o[1]; org[4 * grp + 2] = o[2];
         org[4 * grp + 3] = sqrt(__longlong_as_double(r2b));
-        if (ext) {
-            // half extents of the bounding box about the origin, rounded up (never smaller)
-            float h[3];
-            for (int c = 0; c < 3; ++c) h[c] = any ? __double2float_ru(fmax(bhi[c] - o[c], o[c] - blo[c])) : 0.f;
-            ext[grp] = make_float4(h[0], h[1], h[2], 0.f);
-        }
+    }
+    if (ext && tid == 32) {
+        // half extents of the bounding box about the origin, rounded up (never smaller)
+        float h[3];
+        for (int c = 0; c < 3; ++c) h[c] = cnt > 0 ? __double2float_ru(fmax(bhi[c] - o[c], o[c] - blo[c])) : 0.f;
+        ext[grp] = make_float4(h[0], h[1], h[2], 0.f);
     }
 }
 
@@ -373,32 +355,42 @@ cudaError_t launch_radix_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t
 // Small inputs by counting: a point's place is the number of points before it in (key, index)
 // order, the order of the stable radix sort.  A block ranks 32 points, one per lane; its 16 warps
 // count over every 16th block of four keys, which all lanes read as one 16-byte broadcast, and the
-// warps' counts are added in shared memory.  n^2 compares at two instructions each stay below the
-// radix sort's nine dependent launches (about 65 us at any size up to 1e5) until some 3e4 points;
-// measured in a whole evaluation against the sorts it replaces: see kRankMax.
+// warps' counts are added in shared memory.  The keys are stored as float32 numbers (24 bits,
+// exact), so that a compare is a saturating subtraction, min(max(key - other, 0), 1), and its count
+// another addition: two operations on the full-rate pipe, where integer compares and counts took
+// seven cycles (20 000 points 76 us).  n^2 compares then stay below the radix sort's nine dependent
+// launches (about 65 us at any size up to 1e5) until kRankMax points.
 constexpr int kRankWarps = 16;
 constexpr int kRankPoints = 32;
 
-__global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const uint32_t* __restrict__ keys, int n,
+__global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const float* __restrict__ keys, int n,
                                                                 uint32_t* __restrict__ perm) {
     __shared__ int s_cnt[kRankWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i0 = blockIdx.x * kRankPoints, i = i0 + lane;
-    const uint32_t key = i < n ? keys[i] : 0u;
-    const uint4* k4 = reinterpret_cast<const uint4*>(keys);   // the key buffer starts on 256 bytes
+    const float key = i < n ? keys[i] : 0.f;
+    const float4* k4 = reinterpret_cast<const float4*>(keys); // the key buffer starts on 256 bytes
     const int n4 = n >> 2, own = i0 >> 2;                     // whole blocks of four; the block's own eight
-    int c = 0;
+    float c0 = 0.f, c1 = 0.f;                                 // counts below 2^24: exact
     // points before the block's own: an equal key counts; after them: it does not
+    const float key1 = key + 1.f;
 #pragma unroll 8
     for (int j = w; j < own; j += kRankWarps) {
-        const uint4 k = k4[j];
-        c += (k.x <= key) + (k.y <= key) + (k.z <= key) + (k.w <= key);
+        const float4 k = k4[j];
+        c0 += __saturatef(key1 - k.x);
+        c1 += __saturatef(key1 - k.y);
+        c0 += __saturatef(key1 - k.z);
+        c1 += __saturatef(key1 - k.w);
     }
 #pragma unroll 8
     for (int j = own + kRankPoints / 4 + w; j < n4; j += kRankWarps) {
-        const uint4 k = k4[j];
-        c += (k.x < key) + (k.y < key) + (k.z < key) + (k.w < key);
+        const float4 k = k4[j];
+        c0 += __saturatef(key - k.x);
+        c1 += __saturatef(key - k.y);
+        c0 += __saturatef(key - k.z);
+        c1 += __saturatef(key - k.w);
     }
+    int c = (int)(c0 + c1);
     if (w == 0)
         for (int j = i0; j < i0 + kRankPoints && j < n; ++j) c += keys[j] < key || (keys[j] == key && j < i);
     // keys past the last whole block of four, unless they are the block's own
@@ -414,20 +406,15 @@ __global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const uint32_t* 
     }
 }
 
-// Where counting gives way to the radix sort.
-#ifndef PSUM_RANK_MAX
-#define PSUM_RANK_MAX 24576
-#endif
-constexpr int64_t kRankMax = PSUM_RANK_MAX;
-
 int curve_order_launches(int64_t n) { return n <= kRankMax ? 1 : 3 * 3; }
 
-// The stable order of n points by their 24-bit keys (in kb, which is overwritten): the permutation
-// ends in va.
+// The stable order of n points by their keys as stored_key wrote them to kb (which is overwritten):
+// the permutation ends in va.
 cudaError_t launch_curve_order(int64_t n, uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, uint32_t* hist,
                                cudaStream_t st) {
     if (n <= kRankMax) {
-        k_rank_order<<<(unsigned)((n + kRankPoints - 1) / kRankPoints), 32 * kRankWarps, 0, st>>>(kb, (int)n, va);
+        k_rank_order<<<(unsigned)((n + kRankPoints - 1) / kRankPoints), 32 * kRankWarps, 0, st>>>((const float*)kb, (int)n,
+                                                                                                va);
         return cudaGetLastError();
     }
     return launch_radix_sort(kb, nullptr, ka, va, hist, n, 3, st, vb);
@@ -437,25 +424,21 @@ cudaError_t launch_curve_order(int64_t n, uint32_t* ka, uint32_t* va, uint32_t* 
 cudaError_t launch_curve_sort(const double* x, int64_t n, const double d[3], uint32_t* ka, uint32_t* va,
                                uint32_t* kb, uint32_t* vb, uint32_t* hist, cudaStream_t st) {
     const int bs = 256;
-    k_curve_keys<<<(unsigned)((n + bs - 1) / bs), bs, 0, st>>>(x, n, d[0], d[1], d[2], kb);
+    k_curve_keys<<<(unsigned)((n + bs - 1) / bs), bs, 0, st>>>(x, n, curve_box(d, n), kb);
     return launch_curve_order(n, ka, va, kb, vb, hist, st);
 }
 
 cudaError_t launch_pack32(const double* x, const double* q, const uint32_t* perm, int64_t n, int64_t n_groups,
                           float4* pk_hi, float4* pk_lo, double* org, cudaStream_t st, double* xs, float4* ext) {
-    const int warps = kPackWarps;
-    k_pack32<<<(unsigned)((n_groups + warps - 1) / warps), 32 * warps, 0, st>>>(x, q, perm, n, n_groups, nullptr,
-                                                                                  nullptr, pk_hi, pk_lo, org, xs, ext);
+    k_pack32<<<(unsigned)n_groups, kPackThreads, 0, st>>>(x, q, perm, n, nullptr, nullptr, pk_hi, pk_lo, org, xs, ext);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pack32_groups(const double* x, const double* q, const uint32_t* perm, int64_t n_groups,
                                  const int64_t* grp_start, const int* grp_count, float4* pk_hi, float4* pk_lo,
                                  double* org, cudaStream_t st, float4* ext) {
-    const int warps = kPackWarps;
-    k_pack32<<<(unsigned)((n_groups + warps - 1) / warps), 32 * warps, 0, st>>>(x, q, perm, 0, n_groups, grp_start,
-                                                                                  grp_count, pk_hi, pk_lo, org,
-                                                                                  nullptr, ext);
+    k_pack32<<<(unsigned)n_groups, kPackThreads, 0, st>>>(x, q, perm, 0, grp_start, grp_count, pk_hi, pk_lo, org,
+                                                          nullptr, ext);
     return cudaGetLastError();
 }
 
