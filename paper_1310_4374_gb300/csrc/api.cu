@@ -76,6 +76,7 @@ struct Layout {
     float4* chk_src32;
     float4* chk_src32lo;   // float-float plans: lo parts of the check points as sources
     double4_32a* chk_src64;
+    double4_32a* C4;       // the given coefficients with the gradient's
     NearPlanLaunch Lb;
     int nblk_mom;
     NearPlanLaunch Ln, Lc;
@@ -270,6 +271,7 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
     L.chk_src32 = nullptr;
     L.chk_src32lo = nullptr;
     L.chk_src64 = nullptr;
+    L.C4 = nullptr;
     L.nblk_mom = 0;
     if (backward) {
         // the check points as sources: the two-layer sets (float32 packing with layers) or the 2M points
@@ -285,7 +287,9 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
         L.Lb.counter = flags + 3;
         L.Lb.status = flags;
         L.Lb.n_status = 1;
-        L.nblk_mom = moments_blocks(N);
+        L.Lb.zeroed = true;                 // backward_device zeroes the flags
+        L.nblk_mom = moments_blocks(N, pl.opt.p, pl.num_sms);
+        L.C4 = b.take<double4_32a>((size_t)pl.P);
         L.far_phi = b.take<double>((size_t)N);
         L.far_grad = b.take<double>(3 * (size_t)N);
         L.w_part = b.take<double>((size_t)L.nblk_mom * pl.P);
@@ -350,6 +354,7 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     const psum_opts& o = pl.opt;
     const bool fp32 = o.precision != PSUM_FP64;       // float32 packing (FP32C and FF)
     const bool ff = o.precision == PSUM_FF;
+    const bool far64 = o.basis == PSUM_BASIS_SPHERICAL && o.precision != PSUM_FP32C;
     const int M = o.M, P = pl.P;
     if (h->profile) TRY(cudaEventRecord(h->ev[0], st));
     // the status word and the work-item counters start at zero; every other buffer is written
@@ -473,7 +478,8 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     TRY(launch_project(pl.d_pinv, P - 1, M, L.phi_c, layers ? pl.d_lc_pos : pl.d_check_pos, pl.d_C, sd, layers));
     if (zero_mean) TRY(cudaStreamWaitEvent(sd, h->join2, 0));
     TRY(launch_constant(pl.d_C, pl.d_Rbox, P, L.mean_part, L.nblk_mean, 1.0 / (o.d[0] * o.d[1] * o.d[2]),
-                        zero_mean ? 1 : 0, L.val_part, L.nblk_val, L.eval_status, sd));
+                        zero_mean ? 1 : 0, L.val_part, L.nblk_val, L.eval_status, sd, far64 ? pl.d_C4 : nullptr,
+                        pl.d_gradtab, o.p));
     TRY(cudaEventRecord(h->join, sd));
     if (L.sym)
         TRY(launch_sym_reduce(L.part_n, N, sym_band_launch(L, L.sym_bands - 1, false, h->debug_limit), L.phi_n,
@@ -489,10 +495,12 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     if (o.basis == PSUM_BASIS_RBF)
         TRY(launch_far_rbf(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C, pl.d_rbf, pl.P - 1,
                            L.eval_status, phi, grad, L.eval_status, pl.d_status, st));
+    else if (far64)
+        TRY(launch_far64(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C4, o.p, 1.0 / pl.R0, pl.d_shtab64,
+                         L.eval_status, phi, grad, L.eval_status, pl.d_status, st));
     else
         TRY(launch_far_combine(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C, o.p, 1.0 / pl.R0,
-                               pl.d_shtab64, o.precision == PSUM_FP32C ? pl.d_shtab32 : nullptr, L.eval_status,
-                               phi, grad, L.eval_status, pl.d_status, st));
+                               pl.d_shtab32, L.eval_status, phi, grad, L.eval_status, pl.d_status, st));
     h->launches += 3;   // projection, constant, far field
     if (h->profile) TRY(cudaEventRecord(h->ev[5], st));
     return PSUM_OK;
@@ -533,8 +541,29 @@ int backward_device(psum_plan_s* h, int64_t N, const double* x, const double* q,
     const bool fp32 = o.precision != PSUM_FP64;       // float32 packing (FP32C and FF)
     const bool ff = o.precision == PSUM_FF;
     const int M = o.M, P = pl.P;
-    if (moments_smem(o.p) > 48 * 1024) TRY(set_moments_smem(moments_smem(o.p)));
-    TRY(cudaMemsetAsync(L.eval_status, 0, sizeof(int), st));
+    TRY(cudaMemsetAsync(L.eval_status, 0, kFlags * sizeof(int), st));
+    // on the side stream, beside the sort and the packing: moments w and the far field at the
+    // charges; u = (A^+)^T w; the check points as sources with charges from u
+    cudaStream_t sd = h->side;
+    TRY(cudaEventRecord(h->fork, st));
+    TRY(cudaStreamWaitEvent(sd, h->fork, 0));
+    TRY(launch_moments(x, q, N, C, L.C4, o.p, 1.0 / pl.R0, pl.d_shtab64, pl.d_gradtab, L.far_phi, L.far_grad, L.w_part,
+                       L.nblk_mom, L.w, sd));
+    TRY(launch_adjoint(pl.d_pinv, P - 1, M, L.w, L.u, sd));
+    const size_t n_bk = (size_t)pl.bk_chunks * kNearChunk;
+    const size_t n_chk_pts = (size_t)pl.n_check_tiles * (fp32 ? kTile32 : kTile64);
+    if (fp32 && pl.bk_chunks > 0) {
+        const float4* bk = (const float4*)pl.d_bk_pk;
+        TRY(launch_check_sources32(bk, bk + 2 * n_bk, pl.d_bk_slot, (int64_t)n_bk, M, L.u, L.chk_src32, L.chk_src32lo,
+                                   sd, true));
+    } else if (fp32) {
+        const float4* chk = (const float4*)pl.d_check_tgt;
+        TRY(launch_check_sources32(chk, chk + 2 * n_chk_pts, pl.d_check_inv, (int64_t)n_chk_pts, M, L.u,
+                                   L.chk_src32, L.chk_src32lo, sd));
+    } else {
+        TRY(launch_check_sources64((const double4_32a*)pl.d_check_tgt, (int64_t)n_chk_pts, M, L.u, L.chk_src64, sd));
+    }
+    TRY(cudaEventRecord(h->join, sd));
     const int* perm = nullptr;
     if (fp32) {
         TRY(launch_curve_sort(x, N, o.d, L.ka, L.va, L.kb, L.vb, L.hist, st));
@@ -545,39 +574,28 @@ int backward_device(psum_plan_s* h, int64_t N, const double* x, const double* q,
         TRY(launch_pack64(x, q, N, L.n_src_pts, L.pk64, st));
         h->launches += 1;
     }
-    // moments w and the far field at the charges; u = (A^+)^T w
-    TRY(launch_moments(x, q, N, C, o.p, 1.0 / pl.R0, pl.d_shtab64, L.far_phi, L.far_grad, L.w_part,
-                       L.nblk_mom, L.w, st));
-    TRY(launch_adjoint(pl.d_pinv, P - 1, M, L.w, L.u, st));
-    h->launches += 3;
+    h->launches += 4 + (o.p <= kMomColDegree ? 1 : 0);
+    TRY(cudaStreamWaitEvent(st, h->join, 0));
     // psi and grad psi at the charges: the check points as sources
     const int tile = fp32 ? kTile32 : kTile64;
     if (fp32 && pl.bk_chunks > 0) {
         // two-layer check sources: each chunk with its (class, side) image list
-        const size_t n_bk = (size_t)pl.bk_chunks * kNearChunk;
         const float4* bk = (const float4*)pl.d_bk_pk;
-        TRY(launch_check_sources32(bk, bk + 2 * n_bk, pl.d_bk_slot, (int64_t)n_bk, M, L.u, L.chk_src32, L.chk_src32lo,
-                                   st, true));
         TRY(launch_near32(true, L.chk_src32, ff ? L.chk_src32lo : bk + 2 * n_bk, pl.d_bk_org, L.pk32, L.pk32lo, L.org,
                           pl.d_bk_shifts, L.part_b, L.Lb, st, 0, nullptr, 0.0, ff, nullptr, nullptr, 1, nullptr,
                           pl.d_bk_img0, pl.d_bk_nimg));
     } else if (fp32) {
-        const size_t n_chk_pts = (size_t)pl.n_check_tiles * kTile32;
         const float4* chk = (const float4*)pl.d_check_tgt;
-        TRY(launch_check_sources32(chk, chk + 2 * n_chk_pts, pl.d_check_inv, (int64_t)n_chk_pts, M, L.u,
-                                   L.chk_src32, L.chk_src32lo, st));
         TRY(launch_near32(true, L.chk_src32, ff ? L.chk_src32lo : chk + 2 * n_chk_pts, pl.d_check_org, L.pk32,
                           L.pk32lo, L.org, pl.d_shifts, L.part_b, L.Lb, st, 0, nullptr, 0.0, ff));
     } else {
-        const size_t n_chk_pts = (size_t)pl.n_check_tiles * kTile64;
-        TRY(launch_check_sources64((const double4_32a*)pl.d_check_tgt, (int64_t)n_chk_pts, M, L.u, L.chk_src64, st));
         TRY(launch_near64(true, L.chk_src64, L.pk64, pl.d_shifts, L.part_b, L.Lb, st));
     }
     TRY(launch_near_reduce(L.part_b, N, tile, 4, L.Lb, L.psi, L.gpsi, st));
     TRY(launch_backward_combine(N, perm, q, phi, grad, L.far_phi, L.far_grad, L.psi, L.gpsi, gE, dEdq, dEdx, st));
     k_status_merge<<<1, 1, 0, st>>>(L.eval_status, pl.d_status);
     TRY(cudaGetLastError());
-    h->launches += 5;
+    h->launches += 4;   // pair sum, reduction, combination, status merge
     return PSUM_OK;
 }
 

@@ -10,13 +10,14 @@
 // as the forward sum: 2M charges (+u at y~, -u at y) with the near block's images, or, as the
 // right-hand side's two image layers, M points twice (+u_l with the upper layer's images, -u_l
 // with the lower's; float32 packing with plans that take the layers).
-#include "psum_internal.cuh"
+#include "harmonics.cuh"
 
 namespace psum {
 
 constexpr int kMomThreads = 128;
 
-// phi_far (with C_1) and grad phi_far at every charge, and per-block partial moments.
+// phi_far (with C_1) and grad phi_far at every charge, and per-block partial moments: degrees above
+// kMomColDegree.
 __global__ void __launch_bounds__(kMomThreads) k_moments(const double* __restrict__ x, const double* __restrict__ q,
                                                          int64_t n, const double* __restrict__ C, int p,
                                                          double inv_R0, const double* __restrict__ tab,
@@ -67,22 +68,119 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const double* __restric
     }
 }
 
-__global__ void k_moments_reduce(const double* __restrict__ w_partial, int nblk, int P, double* __restrict__ w) {
+// The same with the columns of the expansion shared out to the warps of a block of 32 charges
+// (harmonics.cuh).  Each warp leaves its terms' values in shared memory, and a thread per term sums
+// them over the charges, q in the multiply-add: one float64 warp operation per term where a shuffle
+// reduction of every term took five and carrying the gradient 27 (2000 charges, degree 8: 89 us).
+// A block takes every gridDim.x'th group of 32 charges and keeps its terms' sums in registers.
+// Degrees up to kMomColDegree, whose values fit the shared memory of an SM; k_moments above.
+constexpr int kMomOwn = 3;               // terms per thread: (p+1)^2 / (32 harmonic_warps(p)) < p/16 + 1
+constexpr int kMomPad = 33;
+
+__global__ void k_moments_columns(const double* __restrict__ x, const double* __restrict__ q, int64_t n,
+                                  const double4_32a* __restrict__ C4, int p, double inv_R0,
+                                  const double* __restrict__ tab, double* __restrict__ far_phi,
+                                  double* __restrict__ far_grad, double* __restrict__ w_partial) {
+    extern __shared__ double4_32a s_C4[];
+    const int P = (p + 1) * (p + 1), nt = sh_tab_size(p), W = blockDim.x / 32;
+    double* s_red = (double*)(s_C4 + P);              // [W][4][32]
+    double* s_tab = s_red + W * 4 * 32;
+    double* s_q = s_tab + nt;                         // [32]
+    double* s_v = s_q + 32;                           // [P][kMomPad]
+    for (int t = threadIdx.x; t < P; t += blockDim.x) s_C4[t] = C4[t];
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) s_tab[t] = tab[t];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double acc[kMomOwn] = {};
+    for (int64_t g = blockIdx.x; g * 32 < n; g += gridDim.x) {
+        const int64_t i = g * 32 + lane;
+        const bool live = i < n;
+        const double ux = live ? x[3 * i] * inv_R0 : 0.0, uy = live ? x[3 * i + 1] * inv_R0 : 0.0,
+                     uz = live ? x[3 * i + 2] * inv_R0 : 0.0;
+        __syncthreads();                              // tables in; the last group's values are used up
+        if (w == 0) s_q[lane] = live ? q[i] : 0.0;
+        double f = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+        harmonic_columns(ux, uy, uz, p, w, s_tab, [&](int t, double v) {
+            const double4_32a c = s_C4[t];
+            f = fma(c.x, v, f);
+            gx = fma(c.y, v, gx);
+            gy = fma(c.z, v, gy);
+            gz = fma(c.w, v, gz);
+            s_v[t * kMomPad + lane] = v;
+        });
+        s_red[(w * 4) * 32 + lane] = f;
+        s_red[(w * 4 + 1) * 32 + lane] = gx;
+        s_red[(w * 4 + 2) * 32 + lane] = gy;
+        s_red[(w * 4 + 3) * 32 + lane] = gz;
+        __syncthreads();
+        for (int c = w; c < 4 && live; c += W) {
+            double v = s_red[c * 32 + lane];
+            for (int k = 1; k < W; ++k) v += s_red[(k * 4 + c) * 32 + lane];
+            if (c == 0)
+                far_phi[i] = v;
+            else
+                far_grad[3 * i + c - 1] = v * inv_R0;
+        }
+#pragma unroll
+        for (int o = 0; o < kMomOwn; ++o) {
+            const int t = threadIdx.x + o * blockDim.x;
+            if (t < P) {
+                double s = 0.0;
+#pragma unroll 8
+                for (int j = 0; j < 32; ++j) s = fma(s_q[j], s_v[t * kMomPad + j], s);
+                acc[o] += s;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 0; o < kMomOwn; ++o) {
+        const int t = threadIdx.x + o * blockDim.x;
+        if (t < P) w_partial[(int64_t)blockIdx.x * P + t] = acc[o];
+    }
+}
+
+// the coefficients with those of the gradient (harmonics.cuh)
+__global__ void k_grad_coeffs(const double* __restrict__ C, const double* __restrict__ gt, int p,
+                              double4_32a* __restrict__ C4) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= P) return;
+    if (t >= (p + 1) * (p + 1)) return;
+    double4_32a c = make_double4_32a(C[t], 0.0, 0.0, 0.0);
+    grad_coeffs(C, gt, p, t, c.y, c.z, c.w);
+    C4[t] = c;
+}
+
+// Sums over rows with a lane per column: the warps take every kColWarps'th row and are added in a
+// fixed order (one thread per column walked 100 to 300 rows one after another).
+constexpr int kColWarps = 8;
+template <class Row>
+__device__ __forceinline__ double column_sum(int rows, Row&& row) {
+    __shared__ double s_part[kColWarps][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += w_partial[(int64_t)b * P + t];
-    w[t] = s;
+#pragma unroll 4
+    for (int r = w; r < rows; r += kColWarps) s = row(r, s);
+    s_part[w][lane] = s;
+    __syncthreads();
+    s = s_part[0][lane];
+#pragma unroll
+    for (int k = 1; k < kColWarps; ++k) s += s_part[k][lane];
+    return s;
+}
+
+__global__ void __launch_bounds__(32 * kColWarps) k_moments_reduce(const double* __restrict__ w_partial, int nblk, int P,
+                                                                  double* __restrict__ w) {
+    const int t = blockIdx.x * 32 + (threadIdx.x & 31);
+    const double s = column_sum(nblk, [&](int b, double a) { return t < P ? a + w_partial[(int64_t)b * P + t] : 0.0; });
+    if (threadIdx.x < 32 && t < P) w[t] = s;
 }
 
 // u = (A^+)^T w over the non-constant moments t = 2..P.
-__global__ void k_adjoint(const double* __restrict__ pinv, int rows, int M, const double* __restrict__ w,
-                          double* __restrict__ u) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= M) return;
-    double s = 0.0;
-    for (int r = 0; r < rows; ++r) s = fma(pinv[(int64_t)r * M + l], w[1 + r], s);
-    u[l] = s;
+__global__ void __launch_bounds__(32 * kColWarps) k_adjoint(const double* __restrict__ pinv, int rows, int M,
+                                                           const double* __restrict__ w, double* __restrict__ u) {
+    const int l = blockIdx.x * 32 + (threadIdx.x & 31);
+    const double s = column_sum(rows, [&](int r, double a) {
+        return l < M ? fma(pinv[(int64_t)r * M + l], w[1 + r], a) : 0.0;
+    });
+    if (threadIdx.x < 32 && l < M) u[l] = s;
 }
 
 // The check points as sources of psi with charges from u (packed positions from the plan).
@@ -179,30 +277,46 @@ __global__ void __launch_bounds__(kEnThreads) k_energy_finish(const double* __re
 }
 
 // ---------------------------------------------------------------------------
-size_t moments_smem(int p);
+size_t moments_smem(int p) {
+    const size_t P = (size_t)(p + 1) * (p + 1);
+    if (p <= kMomColDegree)
+        return sizeof(double4_32a) * P +
+               sizeof(double) * (harmonic_warps(p) * 128 + sh_tab_size(p) + 32 + P * kMomPad);
+    return sizeof(double) * (P * (1 + kMomThreads / 32) + sh_tab_size(p));
+}
 
-cudaError_t launch_moments(const double* x, const double* q, int64_t n, const double* C, int p, double inv_R0,
-                           const double* tab, double* far_phi, double* far_grad, double* w_partial, int nblk,
-                           double* w, cudaStream_t st) {
+// blocks of the moments' launch: resident ones (two an SM up to degree 16) that share the charges, or
+// one per kMomThreads charges
+int moments_blocks(int64_t n, int p, int num_sms) {
+    if (p > kMomColDegree) return (int)((n + kMomThreads - 1) / kMomThreads);
+    const int64_t nb = (n + 31) / 32, cap = 2LL * num_sms;
+    return (int)(nb < cap ? nb : cap);
+}
+
+cudaError_t launch_moments(const double* x, const double* q, int64_t n, const double* C, double4_32a* C4, int p,
+                           double inv_R0, const double* tab, const double* grad_tab, double* far_phi, double* far_grad,
+                           double* w_partial, int nblk, double* w, cudaStream_t st) {
     const int P = (p + 1) * (p + 1);
     const size_t smem = moments_smem(p);
-    k_moments<<<nblk, kMomThreads, smem, st>>>(x, q, n, C, p, inv_R0, tab, far_phi, far_grad, w_partial);
-    k_moments_reduce<<<(P + 127) / 128, 128, 0, st>>>(w_partial, nblk, P, w);
+    const bool cols = p <= kMomColDegree;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cols ? cudaFuncSetAttribute(k_moments_columns, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                                   : cudaFuncSetAttribute(k_moments, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    if (cols) {
+        k_grad_coeffs<<<(P + 127) / 128, 128, 0, st>>>(C, grad_tab, p, C4);
+        k_moments_columns<<<nblk, 32 * harmonic_warps(p), smem, st>>>(x, q, n, C4, p, inv_R0, tab, far_phi, far_grad,
+                                                                     w_partial);
+    } else {
+        k_moments<<<nblk, kMomThreads, smem, st>>>(x, q, n, C, p, inv_R0, tab, far_phi, far_grad, w_partial);
+    }
+    k_moments_reduce<<<(P + 31) / 32, 32 * kColWarps, 0, st>>>(w_partial, nblk, P, w);
     return cudaGetLastError();
 }
 
-cudaError_t set_moments_smem(size_t bytes) {
-    return cudaFuncSetAttribute(k_moments, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-int moments_blocks(int64_t n) { return (int)((n + kMomThreads - 1) / kMomThreads); }
-
-size_t moments_smem(int p) {
-    return sizeof(double) * ((p + 1) * (p + 1) * (1 + kMomThreads / 32) + sh_tab_size(p));
-}
-
 cudaError_t launch_adjoint(const double* pinv, int rows, int M, const double* w, double* u, cudaStream_t st) {
-    k_adjoint<<<(M + 127) / 128, 128, 0, st>>>(pinv, rows, M, w, u);
+    k_adjoint<<<(M + 31) / 32, 32 * kColWarps, 0, st>>>(pinv, rows, M, w, u);
     return cudaGetLastError();
 }
 

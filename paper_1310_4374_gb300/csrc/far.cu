@@ -7,6 +7,7 @@
 // All of it runs in float64.
 #include "launch.cuh"
 #include "diffuse.cuh"
+#include "harmonics.cuh"
 #include "mean.cuh"
 
 namespace psum {
@@ -189,8 +190,16 @@ __global__ void __launch_bounds__(kRedThreads) k_constant(double* __restrict__ C
                                                           int P, const double* __restrict__ mean_partial, int nblk,
                                                           double inv_V0, int zero_mean,
                                                           const double* __restrict__ val_partial, int nblk_val,
-                                                          int* __restrict__ status) {
+                                                          int* __restrict__ status, double4_32a* __restrict__ C4,
+                                                          const double* __restrict__ gt, int p) {
     double s = 0.0, m = 0.0, qs = 0.0, qa = 0.0;
+    if (C4)                                    // the coefficients with the gradient's (C_1 below)
+        for (int t = threadIdx.x; t < P; t += kRedThreads) {
+            double4_32a c = make_double4_32a(C[t], 0.0, 0.0, 0.0);
+            grad_coeffs(C, gt, p, t, c.y, c.z, c.w);
+            if (t) C4[t] = c;
+            else C4[0].y = c.y, C4[0].z = c.z, C4[0].w = c.w;
+        }
     if (zero_mean) {
         for (int t = 1 + threadIdx.x; t < P; t += kRedThreads) s = fma(C[t], Rbox[t], s);
         for (int b = threadIdx.x; b < nblk; b += kRedThreads) m += mean_partial[b];
@@ -200,7 +209,10 @@ __global__ void __launch_bounds__(kRedThreads) k_constant(double* __restrict__ C
         qa += val_partial[2 * b + 1];
     }
     block_sum2<kRedThreads>(s, m);
-    if (threadIdx.x == 0) C[0] = zero_mean ? (-m * inv_V0 - s) : 0.0;
+    if (threadIdx.x == 0) {
+        C[0] = zero_mean ? (-m * inv_V0 - s) : 0.0;
+        if (C4) C4[0].x = C[0];
+    }
     __syncthreads();                           // block_sum2's shared sums are free again
     block_sum2<kRedThreads>(qs, qa);
     if (threadIdx.x == 0 && !(fabs(qs) <= 1e-12 * qa)) atomicOr(status, kStatNonNeutral);
@@ -223,15 +235,14 @@ __device__ __forceinline__ void flag_nonfinite(int* status, int* plan_status) {
 // ---------------------------------------------------------------------------
 constexpr int kFarThreads = 128;
 
-// T = double for FP64 plans; T = float for FP32C plans, whose far field is a smooth,
-// slowly varying part of phi (its float32 evaluation errors sit well below the pair sum's)
-template <class T>
+// FP32C plans: in float32, a smooth, slowly varying part of phi (its float32 evaluation errors sit
+// well below the pair sum's)
 __global__ void __launch_bounds__(kFarThreads) k_far_combine(const double* __restrict__ x, int64_t n,
                                                              const int* __restrict__ perm,
                                                              const double* __restrict__ phi_near,
                                                              const double* __restrict__ grad_near,
                                                              const double* __restrict__ C, int p, double inv_R0,
-                                                             const T* __restrict__ tab,
+                                                             const float* __restrict__ tab,
                                                              const int* __restrict__ status,
                                                              double* __restrict__ phi, double* __restrict__ grad,
                                                              int* __restrict__ status_out, int* __restrict__ plan_status) {
@@ -239,6 +250,7 @@ __global__ void __launch_bounds__(kFarThreads) k_far_combine(const double* __res
     extern __shared__ unsigned char s_raw[];
     const int P = (p + 1) * (p + 1);
     const int nt = sh_tab_size(p);
+    using T = float;
     T* s_C = (T*)s_raw;
     T* s_tab = s_C + P;
     for (int t = threadIdx.x; t < P; t += kFarThreads) s_C[t] = (T)C[t];
@@ -283,6 +295,62 @@ __global__ void __launch_bounds__(kFarThreads) k_far_combine(const double* __res
                  fabs(g2) <= 1.7976931348623157e308;
     }
     if (!finite) flag_nonfinite(status_out, plan_status);
+}
+
+// FP64 and FF plans: in float64, the columns of the expansion shared out to the warps of a block of
+// 32 points (harmonics.cuh); C4 holds each coefficient with the gradient's.  One thread per point
+// with the gradient carried through the recurrence kept the float64 pipes of a few SMs busy for
+// 61 us at 1000 charges and degree 8 (a float64 warp instruction takes a scheduler 64 cycles);
+// this takes about a quarter of the operations and spreads them over four times the schedulers.
+template <bool kGrad>
+__global__ void k_far64(const double* __restrict__ x, int64_t n, const int* __restrict__ perm,
+                        const double* __restrict__ phi_near, const double* __restrict__ grad_near,
+                        const double4_32a* __restrict__ C4, int p, double inv_R0, const double* __restrict__ tab,
+                        const int* __restrict__ status, double* __restrict__ phi, double* __restrict__ grad,
+                        int* __restrict__ status_out, int* __restrict__ plan_status) {
+    merge_status(status, plan_status);
+    extern __shared__ double4_32a s_C4[];
+    const int P = (p + 1) * (p + 1), nt = sh_tab_size(p), W = blockDim.x / 32;
+    double* s_red = (double*)(s_C4 + P);              // [W][4][32]
+    double* s_tab = s_red + W * 4 * 32;
+    for (int t = threadIdx.x; t < P; t += blockDim.x) s_C4[t] = C4[t];
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) s_tab[t] = tab[t];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t s = (int64_t)blockIdx.x * 32 + lane;
+    const bool live = s < n;
+    const int64_t i = live ? (perm ? (int64_t)perm[s] : s) : 0;
+    const double ux = x[3 * i] * inv_R0, uy = x[3 * i + 1] * inv_R0, uz = x[3 * i + 2] * inv_R0;
+    __syncthreads();
+    double f = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+    harmonic_columns(ux, uy, uz, p, w, s_tab, [&](int t, double v) {
+        const double4_32a c = s_C4[t];
+        f = fma(c.x, v, f);
+        if (kGrad) {
+            gx = fma(c.y, v, gx);
+            gy = fma(c.z, v, gy);
+            gz = fma(c.w, v, gz);
+        }
+    });
+    s_red[(w * 4) * 32 + lane] = f;
+    if (kGrad) {
+        s_red[(w * 4 + 1) * 32 + lane] = gx;
+        s_red[(w * 4 + 2) * 32 + lane] = gy;
+        s_red[(w * 4 + 3) * 32 + lane] = gz;
+    }
+    __syncthreads();
+    // warp 0 finishes the potential, the next ones a field component each (a fixed order of warps)
+    for (int c = w; c < (kGrad ? 4 : 1) && live; c += W) {
+        double v = s_red[c * 32 + lane];
+        for (int k = 1; k < W; ++k) v += s_red[(k * 4 + c) * 32 + lane];
+        const bool failed = (*status & (kStatNonNeutral | kStatOutOfBox | kStatNonFinite | kStatTimeout | kStatBounds)) != 0;
+        const double r = failed ? __longlong_as_double(0x7ff8000000000000ll)
+                                : c == 0 ? phi_near[s] + v : grad_near[3 * s + c - 1] + v * inv_R0;
+        if (c == 0)
+            phi[i] = r;
+        else
+            grad[3 * i + c - 1] = r;
+        if (!failed && !(fabs(r) <= 1.7976931348623157e308)) flag_nonfinite(status_out, plan_status);
+    }
 }
 
 // Steps 7-8 with the RBF basis of Eq. 5: phi_far(y) = C_1 + sum_t C_{t+1} / |y - x_t| and
@@ -413,27 +481,35 @@ cudaError_t launch_project(const double* pinv, int rows, int M, const double* ph
 
 cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean_partial, int nblk,
                             double inv_V0, int zero_mean, const double* val_partial, int nblk_val, int* status,
-                            cudaStream_t st) {
+                            cudaStream_t st, double4_32a* C4, const double* grad_tab, int p) {
     k_constant<<<1, kRedThreads, 0, st>>>(C, Rbox, P, mean_partial, nblk, inv_V0, zero_mean, val_partial, nblk_val,
-                                          status);
+                                          status, C4, grad_tab, p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_far_combine(const double* x, int64_t n, const int* perm, const double* phi_near,
-                               const double* grad_near, const double* C, int p, double inv_R0, const double* tab64,
-                               const float* tab32, const int* status, double* phi, double* grad, int* status_out,
-                               int* plan_status, cudaStream_t st) {
+                               const double* grad_near, const double* C, int p, double inv_R0, const float* tab32,
+                               const int* status, double* phi, double* grad, int* status_out, int* plan_status,
+                               cudaStream_t st) {
     const int P = (p + 1) * (p + 1);
     const unsigned nb = (unsigned)((n + kFarThreads - 1) / kFarThreads);
-    if (tab32) {
-        const size_t smem = sizeof(float) * (P + sh_tab_size(p));
-        k_far_combine<float><<<nb, kFarThreads, smem, st>>>(x, n, perm, phi_near, grad_near, C, p, inv_R0, tab32,
-                                                            status, phi, grad, status_out, plan_status);
-    } else {
-        const size_t smem = sizeof(double) * (P + sh_tab_size(p));
-        k_far_combine<double><<<nb, kFarThreads, smem, st>>>(x, n, perm, phi_near, grad_near, C, p, inv_R0, tab64,
-                                                             status, phi, grad, status_out, plan_status);
+    k_far_combine<<<nb, kFarThreads, sizeof(float) * (P + sh_tab_size(p)), st>>>(
+        x, n, perm, phi_near, grad_near, C, p, inv_R0, tab32, status, phi, grad, status_out, plan_status);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_far64(const double* x, int64_t n, const int* perm, const double* phi_near, const double* grad_near,
+                         const double4_32a* C4, int p, double inv_R0, const double* tab64, const int* status,
+                         double* phi, double* grad, int* status_out, int* plan_status, cudaStream_t st) {
+    const int W = harmonic_warps(p);
+    const size_t smem = sizeof(double4_32a) * (size_t)(p + 1) * (p + 1) + sizeof(double) * (W * 128 + sh_tab_size(p));
+    const auto kernel = grad ? k_far64<true> : k_far64<false>;
+    if (smem > 48 * 1024) {              // high degrees
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
     }
+    kernel<<<(unsigned)((n + 31) / 32), 32 * W, smem, st>>>(x, n, perm, phi_near, grad_near, C4, p, inv_R0, tab64, status,
+                                                           phi, grad, status_out, plan_status);
     return cudaGetLastError();
 }
 

@@ -49,7 +49,8 @@ struct CurveBox {
     double d[3], inv[3];
     int as_float;
 };
-constexpr int64_t kRankMax = 24576;
+constexpr int64_t kRankSms = 152;                // SMs of the chip
+constexpr int64_t kRankMax = 5 * 32 * kRankSms;  // up to five points a lane, one block an SM
 inline CurveBox curve_box(const double d[3], int64_t n) {
     return CurveBox{{d[0], d[1], d[2]}, {256.0 / d[0], 256.0 / d[1], 256.0 / d[2]}, n <= kRankMax ? 1 : 0};
 }
@@ -95,18 +96,23 @@ cudaError_t launch_project(const double* pinv, int rows, int M, const double* ph
                            double* C, cudaStream_t st, bool layers = false);
 cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean_partial, int nblk,
                             double inv_V0, int zero_mean, const double* val_partial, int nblk_val, int* status,
-                            cudaStream_t st);
-// tab32 != nullptr: the far field in float (FP32C plans), else in double with tab64
+                            cudaStream_t st, double4_32a* C4 = nullptr, const double* grad_tab = nullptr, int p = 0);
+// the far field and the sum: in float32 (FP32C plans), or in float64 from the coefficients with the
+// gradient's that launch_constant has formed
 cudaError_t launch_far_combine(const double* x, int64_t n, const int* perm, const double* phi_near,
-                               const double* grad_near, const double* C, int p, double inv_R0, const double* tab64,
-                               const float* tab32, const int* status, double* phi, double* grad, int* status_out,
-                               int* plan_status, cudaStream_t st);
+                               const double* grad_near, const double* C, int p, double inv_R0, const float* tab32,
+                               const int* status, double* phi, double* grad, int* status_out, int* plan_status,
+                               cudaStream_t st);
+cudaError_t launch_far64(const double* x, int64_t n, const int* perm, const double* phi_near, const double* grad_near,
+                         const double4_32a* C4, int p, double inv_R0, const double* tab64, const int* status,
+                         double* phi, double* grad, int* status_out, int* plan_status, cudaStream_t st);
 // backward.cu
-cudaError_t launch_moments(const double* x, const double* q, int64_t n, const double* C, int p, double inv_R0,
-                           const double* tab, double* far_phi, double* far_grad, double* w_partial, int nblk,
-                           double* w, cudaStream_t st);
-int moments_blocks(int64_t n);
-size_t moments_smem(int p);
+// the moments w (P) of the charges and the far field of the coefficients C at them; C4: P scratch
+cudaError_t launch_moments(const double* x, const double* q, int64_t n, const double* C, double4_32a* C4, int p,
+                           double inv_R0, const double* tab, const double* grad_tab, double* far_phi, double* far_grad,
+                           double* w_partial, int nblk, double* w, cudaStream_t st);
+int moments_blocks(int64_t n, int p, int num_sms);
+constexpr int kMomColDegree = 25;   // the moments by columns up to this degree (backward.cu)
 cudaError_t launch_adjoint(const double* pinv, int rows, int M, const double* w, double* u, cudaStream_t st);
 cudaError_t launch_check_sources32(const float4* chk_hi, const float4* chk_lo, const int* inv, int64_t n_pts, int M,
                                    const double* u, float4* out_hi, float4* out_lo, cudaStream_t st,
@@ -119,6 +125,5 @@ cudaError_t launch_backward_combine(int64_t n, const int* perm, const double* q,
                                     double* dEdx, cudaStream_t st);
 cudaError_t launch_energy(const double* q, const double* phi, int64_t n, double* partial, int nblk, double* E,
                           cudaStream_t st);
-cudaError_t set_moments_smem(size_t bytes);
 }  // namespace psum
 

@@ -241,29 +241,30 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
                 for (int im = im_lo + tid; im < im_hi; im += kThreads32)
                     s_near[im] = (s_near[im] & kUnitWeighted) ? (s_near[im] & ~kUnitWeighted) : kUnitOutside;
             } else
-            for (int im = im_lo + tid; im < im_hi; im += kThreads32) {
+            // a thread per (image, target group): four groups one after another in one warp kept a
+            // float64 pipe busy for 6000 cycles a chunk, more than a unit's pair loop
+            for (int e = im_lo * kTgt32 + tid; e < im_hi * kTgt32; e += kThreads32) {
+                const int im = e / kTgt32, k = e % kTgt32;
                 const int img0 = a.chunk_img0 ? a.chunk_img0[chunk] : shift0;
                 const double* sh = a.shifts + 3 * (img0 + im);
+                const double* to = a.tgt_org + 4 * (cur_tile * kTgt32 + k);
                 int nr = 0;
                 bool weighted = false;
-                for (int k = 0; k < kTgt32; ++k) {
-                    const double* to = a.tgt_org + 4 * (cur_tile * kTgt32 + k);
-                    const double* shk = sh;
-                    if constexpr (!kGrad) {
-                        const float wk = a.img_w ? a.img_w[shift0 + im] : 1.f;
-                        s_w[im * kTgt32 + k] = wk;
-                        weighted = weighted || wk != 0.f;
-                    }
-                    // offset of the target-group origin from the shifted chunk origin, as hi + lo
-                    const double D0 = (to[0] - so[0]) - shk[0], D1 = (to[1] - so[1]) - shk[1],
-                                 D2 = (to[2] - so[2]) - shk[2];
-                    float* dl = s_delta + 6 * (im * kTgt32 + k);
-                    dl[0] = (float)D0; dl[1] = (float)D1; dl[2] = (float)D2;
-                    dl[3] = (float)(D0 - (double)dl[0]); dl[4] = (float)(D1 - (double)dl[1]);
-                    dl[5] = (float)(D2 - (double)dl[2]);
-                    const double reach = kNearFactor * (to[3] + so[3]);
-                    if (D0 * D0 + D1 * D1 + D2 * D2 <= reach * reach) nr |= k < 2 ? kUnitNear0 : kUnitNear1;
+                if constexpr (!kGrad) {
+                    const float wk = a.img_w ? a.img_w[shift0 + im] : 1.f;
+                    s_w[e] = wk;
+                    weighted = wk != 0.f;
                 }
+                // offset of the target-group origin from the shifted chunk origin, as hi + lo
+                const double D0 = (to[0] - so[0]) - sh[0], D1 = (to[1] - so[1]) - sh[1],
+                             D2 = (to[2] - so[2]) - sh[2];
+                float* dl = s_delta + 6 * e;
+                dl[0] = (float)D0; dl[1] = (float)D1; dl[2] = (float)D2;
+                dl[3] = (float)(D0 - (double)dl[0]); dl[4] = (float)(D1 - (double)dl[1]);
+                dl[5] = (float)(D2 - (double)dl[2]);
+                const double reach = kNearFactor * (to[3] + so[3]);
+                if (D0 * D0 + D1 * D1 + D2 * D2 <= reach * reach) nr |= k < 2 ? kUnitNear0 : kUnitNear1;
+                nr = quad_or(nr);
                 if (kTrim) {
                     // the chunk's bounding sphere against the ball, with a margin: the exact
                     // per-source test decides everything near the sphere
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
                 }
                 if (!kGrad && !weighted) nr = kUnitOutside;   // padding image of every group: skip
                 if (a.chunk_nimg && im >= a.chunk_nimg[chunk]) nr = kUnitOutside;   // past the chunk's list
-                s_near[im] = nr;
+                if (k == 0) s_near[im] = nr;
             }
             const long long limit = a.inject ? (1LL << 12) : kCopySpinLimit;
             if (tid == 0 && !mbar_wait(&s_bar, phase, limit)) s_fail = 1;

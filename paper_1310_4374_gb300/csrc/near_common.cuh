@@ -100,6 +100,13 @@ __device__ __forceinline__ int shift_sign(const double* sh) {
                         : sh[1] != 0.0 ? (sh[1] > 0.0 ? 1 : -1) : sh[2] != 0.0 ? (sh[2] > 0.0 ? 1 : -1) : 0;
 }
 
+// the OR over four neighbouring lanes (all four active)
+__device__ __forceinline__ int quad_or(int v) {
+    const unsigned m = __activemask();
+    v |= __shfl_xor_sync(m, v, 1);
+    return v | __shfl_xor_sync(m, v, 2);
+}
+
 // |x + p|^2 <= Rb^2 with the rounding of a plain left-to-right evaluation (no contraction),
 // the same decision for a source at the boundary as a straightforward float64 evaluation
 __device__ __forceinline__ bool in_ball(double x0, double x1, double x2, const double* p, double Rb) {

@@ -16,6 +16,7 @@
 #include <numeric>
 #include <vector>
 
+#include "harmonics.cuh"
 #include "launch.cuh"
 #include "mean.cuh"
 
@@ -606,6 +607,12 @@ int build_plan(const psum_opts& o, Plan& pl) {
         std::vector<float> tabf(tab.begin(), tab.end());
         if ((s2 = upload(&pl.d_shtab64, tab.data(), tab.size()))) return s2;
         if ((s2 = upload(&pl.d_shtab32, tabf.data(), tabf.size()))) return s2;
+        if (!rbf) {
+            std::vector<double> gt(grad_tab_size(p));
+            grad_tab_fill(p, gt.data());
+            if ((s2 = upload(&pl.d_gradtab, gt.data(), gt.size()))) return s2;
+            PSUM_CUDA_TRY(cudaMalloc((void**)&pl.d_C4, sizeof(double4_32a) * pl.P));
+        }
     }
     PSUM_CUDA_TRY(cudaMalloc((void**)&pl.d_C, sizeof(double) * pl.P));
     PSUM_CUDA_TRY(cudaMemset(pl.d_C, 0, sizeof(double) * pl.P));
@@ -640,6 +647,8 @@ void free_plan_device(Plan& pl) {
     cudaFree(pl.d_rbf);
     cudaFree(pl.d_shtab64);
     cudaFree(pl.d_shtab32);
+    cudaFree(pl.d_gradtab);
+    cudaFree(pl.d_C4);
     cudaFree(pl.d_C);
     cudaFree(pl.d_status);
     if (pl.h_status) cudaFreeHost(pl.h_status);

@@ -353,56 +353,77 @@ cudaError_t launch_radix_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t
 }
 
 // Small inputs by counting: a point's place is the number of points before it in (key, index)
-// order, the order of the stable radix sort.  A block ranks 32 points, one per lane; its 16 warps
-// count over every 16th block of four keys, which all lanes read as one 16-byte broadcast, and the
-// warps' counts are added in shared memory.  The keys are stored as float32 numbers (24 bits,
+// order, the order of the stable radix sort.  A block ranks 32 kPer points, kPer per lane; its 16
+// warps count over every 16th block of four keys, which all lanes read as one 16-byte broadcast, and
+// the warps' counts are added in shared memory.  The keys are stored as float32 numbers (24 bits,
 // exact), so that a compare is a saturating subtraction, min(max(key - other, 0), 1), and its count
 // another addition: two operations on the full-rate pipe, where integer compares and counts took
-// seven cycles (20 000 points 76 us).  n^2 compares then stay below the radix sort's nine dependent
-// launches (about 65 us at any size up to 1e5) until kRankMax points.
+// seven cycles.  n^2 compares then stay below the radix sort's nine dependent launches (about 65 us
+// at any size up to 1e5) until kRankMax points.
+// A broadcast fills 32 lanes' registers, four cycles of an SM's load path for 16 bytes: with one
+// point per lane that path bounds the kernel (20 000 points: 55 us).  A lane takes as many points as
+// bring the launch to one block an SM or fewer: 157 blocks on 152 SMs take the time of two rounds
+// (20 000 points with four per lane: 51 us).
 constexpr int kRankWarps = 16;
-constexpr int kRankPoints = 32;
 
+template <int kPer>
 __global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const float* __restrict__ keys, int n,
                                                                 uint32_t* __restrict__ perm) {
-    __shared__ int s_cnt[kRankWarps][32];
+    constexpr int kPoints = 32 * kPer;
+    __shared__ int s_cnt[kRankWarps][kPoints];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i0 = blockIdx.x * kRankPoints, i = i0 + lane;
-    const float key = i < n ? keys[i] : 0.f;
+    const int i0 = blockIdx.x * kPoints;
     const float4* k4 = reinterpret_cast<const float4*>(keys); // the key buffer starts on 256 bytes
-    const int n4 = n >> 2, own = i0 >> 2;                     // whole blocks of four; the block's own eight
-    float c0 = 0.f, c1 = 0.f;                                 // counts below 2^24: exact
+    const int n4 = n >> 2, own = i0 >> 2;                     // whole blocks of four; the block's own
+    float key[kPer], key1[kPer], c0[kPer], c1[kPer];          // counts below 2^24: exact
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+        const int i = i0 + 32 * r + lane;
+        key[r] = i < n ? keys[i] : 0.f;
+        key1[r] = key[r] + 1.f;
+        c0[r] = c1[r] = 0.f;
+    }
     // points before the block's own: an equal key counts; after them: it does not
-    const float key1 = key + 1.f;
-#pragma unroll 8
+#pragma unroll 4
     for (int j = w; j < own; j += kRankWarps) {
         const float4 k = k4[j];
-        c0 += __saturatef(key1 - k.x);
-        c1 += __saturatef(key1 - k.y);
-        c0 += __saturatef(key1 - k.z);
-        c1 += __saturatef(key1 - k.w);
+#pragma unroll
+        for (int r = 0; r < kPer; ++r) {
+            c0[r] += __saturatef(key1[r] - k.x);
+            c1[r] += __saturatef(key1[r] - k.y);
+            c0[r] += __saturatef(key1[r] - k.z);
+            c1[r] += __saturatef(key1[r] - k.w);
+        }
     }
-#pragma unroll 8
-    for (int j = own + kRankPoints / 4 + w; j < n4; j += kRankWarps) {
+#pragma unroll 4
+    for (int j = own + kPoints / 4 + w; j < n4; j += kRankWarps) {
         const float4 k = k4[j];
-        c0 += __saturatef(key - k.x);
-        c1 += __saturatef(key - k.y);
-        c0 += __saturatef(key - k.z);
-        c1 += __saturatef(key - k.w);
+#pragma unroll
+        for (int r = 0; r < kPer; ++r) {
+            c0[r] += __saturatef(key[r] - k.x);
+            c1[r] += __saturatef(key[r] - k.y);
+            c0[r] += __saturatef(key[r] - k.z);
+            c1[r] += __saturatef(key[r] - k.w);
+        }
     }
-    int c = (int)(c0 + c1);
-    if (w == 0)
-        for (int j = i0; j < i0 + kRankPoints && j < n; ++j) c += keys[j] < key || (keys[j] == key && j < i);
-    // keys past the last whole block of four, unless they are the block's own
-    if (w == 1 && (n4 << 2) >= i0 + kRankPoints)
-        for (int j = n4 << 2; j < n; ++j) c += keys[j] < key;
-    s_cnt[w][lane] = c;
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+        const int i = i0 + 32 * r + lane;
+        int c = (int)(c0[r] + c1[r]);
+        // the block's own points, each warp a share of them
+        for (int j = i0 + w; j < i0 + kPoints && j < n; j += kRankWarps) c += keys[j] < key[r] || (keys[j] == key[r] && j < i);
+        // keys past the last whole block of four, unless they are the block's own
+        if (w == 0 && (n4 << 2) >= i0 + kPoints)
+            for (int j = n4 << 2; j < n; ++j) c += keys[j] < key[r];
+        s_cnt[w][32 * r + lane] = c;
+    }
     __syncthreads();
-    if (w == 0 && i < n) {
+    if (w < kPer) {
+        const int i = i0 + 32 * w + lane;
         int r = 0;
 #pragma unroll
-        for (int k = 0; k < kRankWarps; ++k) r += s_cnt[k][lane];
-        perm[r] = (uint32_t)i;
+        for (int k = 0; k < kRankWarps; ++k) r += s_cnt[k][32 * w + lane];
+        if (i < n) perm[r] = (uint32_t)i;
     }
 }
 
@@ -413,8 +434,12 @@ int curve_order_launches(int64_t n) { return n <= kRankMax ? 1 : 3 * 3; }
 cudaError_t launch_curve_order(int64_t n, uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, uint32_t* hist,
                                cudaStream_t st) {
     if (n <= kRankMax) {
-        k_rank_order<<<(unsigned)((n + kRankPoints - 1) / kRankPoints), 32 * kRankWarps, 0, st>>>((const float*)kb, (int)n,
-                                                                                                va);
+        const int per = (int)((n + 32 * kRankSms - 1) / (32 * kRankSms));
+        const unsigned nb = (unsigned)((n + 32 * per - 1) / (32 * per));
+        const float* keys = (const float*)kb;
+        const auto kernel = per == 1 ? k_rank_order<1> : per == 2 ? k_rank_order<2> : per == 3 ? k_rank_order<3>
+                                     : per == 4 ? k_rank_order<4> : k_rank_order<5>;
+        kernel<<<nb, 32 * kRankWarps, 0, st>>>(keys, (int)n, va);
         return cudaGetLastError();
     }
     return launch_radix_sort(kb, nullptr, ka, va, hist, n, 3, st, vb);

@@ -25,7 +25,7 @@ def _run(precision, x, q):
         pc.close()
 
 
-@pytest.mark.parametrize("N", [2, 3, 31, 33, 127, 513, 4099, 24576, 24577])
+@pytest.mark.parametrize("N", [2, 3, 31, 33, 127, 513, 4099, 4865, 9729, 14593, 24320, 24321])
 @pytest.mark.parametrize("one_cell", [False, True])
 def test_order_keeps_every_charge(N, one_cell):
     rng = np.random.default_rng(N)
