@@ -69,7 +69,7 @@ struct Layout {
     // FP64
     double4_32a* pk64;
     // common
-    double *part_n, *part_c, *phi_n, *grad_n, *phi_c, *val_part, *mean_part;
+    double *part_n, *part_c, *phi_n, *grad_n, *phi_c, *val_part, *mean_part, *mean;
     int* eval_status;
     // backward
     double *far_phi, *far_grad, *w_part, *w, *u, *psi, *gpsi, *part_b;
@@ -256,6 +256,7 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
     L.nblk_mean = mean_blocks(N, pl.num_sms);
     L.val_part = b.take<double>(2 * (size_t)L.nblk_val);
     L.mean_part = b.take<double>((size_t)L.nblk_mean);
+    L.mean = b.take<double>(1);
     // the status word and the pair launches' work-item counters
     int* flags = b.take<int>(kFlags);
     L.eval_status = flags;
@@ -354,7 +355,6 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     const psum_opts& o = pl.opt;
     const bool fp32 = o.precision != PSUM_FP64;       // float32 packing (FP32C and FF)
     const bool ff = o.precision == PSUM_FF;
-    const bool far64 = o.basis == PSUM_BASIS_SPHERICAL && o.precision != PSUM_FP32C;
     const int M = o.M, P = pl.P;
     if (h->profile) TRY(cudaEventRecord(h->ev[0], st));
     // the status word and the work-item counters start at zero; every other buffer is written
@@ -365,14 +365,13 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     // reads the sorted order and forks with the check sums below
     const bool zero_mean = o.mean_mode == PSUM_MEAN_ZERO;
     const bool early_mean = zero_mean && !(pl.Rb > 0.0);
+    cudaStream_t s2 = h->side2;
     if (early_mean || sep) TRY(cudaEventRecord(h->fork0, st));
     if (early_mean) {
-        cudaStream_t s2 = h->side2;
         TRY(cudaStreamWaitEvent(s2, h->fork0, 0));
         const double H[3] = {0.5 * (2 * o.K[0] + 1) * o.d[0], 0.5 * (2 * o.K[1] + 1) * o.d[1],
                              0.5 * (2 * o.K[2] + 1) * o.d[2]};
         TRY(launch_box_mean(x, q, N, H, L.mean_part, L.nblk_mean, s2));
-        TRY(cudaEventRecord(h->join2, s2));
         h->launches += 1;
     }
     // separate evaluation points: validated, sorted and packed like the charges, without charges,
@@ -397,6 +396,18 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     }
     const int* perm = nullptr;
     TRY(launch_prepare(x, q, N, o.d, L.val_part, L.nblk_val, L.eval_status, fp32 ? L.kb : nullptr, st));
+    // the mean's total and the neutrality test on the second side stream, ahead of the pair sums
+    // (which leave no room on the SMs until they end)
+    auto queue_totals = [&]() {
+        const cudaError_t e = launch_totals(L.mean_part, zero_mean ? L.nblk_mean : 0, 1.0 / (o.d[0] * o.d[1] * o.d[2]),
+                                            L.val_part, L.nblk_val, L.eval_status, L.mean, s2);
+        return e != cudaSuccess ? e : cudaEventRecord(h->join2, s2);
+    };
+    if (early_mean || !zero_mean) {
+        TRY(cudaEventRecord(h->fork0, st));
+        TRY(cudaStreamWaitEvent(s2, h->fork0, 0));
+        TRY(queue_totals());
+    }
     if (fp32) {
         TRY(launch_curve_order(N, L.ka, L.va, L.kb, L.vb, L.hist, st));
         perm = (const int*)L.va;
@@ -466,42 +477,67 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
     const int tile = fp32 ? kTile32 : kTile64;
     TRY(launch_near_reduce(L.part_c, layers ? (int64_t)pl.lc_tiles * tile : pl.n_check, tile, 1, L.Lc, L.phi_c,
                            nullptr, sd));
-    // the ball's box mean on the second side stream, beside the check sums
+    // the fit follows the check sums; the ball's mean forks here, onto the second side stream
+    TRY(launch_project(pl.d_pinv, P - 1, M, L.phi_c, layers ? pl.d_lc_pos : pl.d_check_pos, pl.d_C, sd, layers));
     if (zero_mean && !early_mean) {
-        cudaStream_t s2 = h->side2;
         TRY(cudaStreamWaitEvent(s2, h->fork, 0));
         TRY(launch_box_mean_ball(x, q, fp32 ? L.va : nullptr, N, o.d, o.K, pl.Rb, L.mean_part, L.nblk_mean, s2));
-        TRY(cudaEventRecord(h->join2, s2));
+        TRY(queue_totals());
         h->launches += 1;
     }
-    // the fit and the constant follow the check sums and the mean, beside the charge kernel
-    TRY(launch_project(pl.d_pinv, P - 1, M, L.phi_c, layers ? pl.d_lc_pos : pl.d_check_pos, pl.d_C, sd, layers));
-    if (zero_mean) TRY(cudaStreamWaitEvent(sd, h->join2, 0));
-    TRY(launch_constant(pl.d_C, pl.d_Rbox, P, L.mean_part, L.nblk_mean, 1.0 / (o.d[0] * o.d[1] * o.d[2]),
-                        zero_mean ? 1 : 0, L.val_part, L.nblk_val, L.eval_status, sd, far64 ? pl.d_C4 : nullptr,
-                        pl.d_gradtab, o.p));
+    const bool rbf = o.basis == PSUM_BASIS_RBF;
+    if (rbf) {
+        TRY(cudaStreamWaitEvent(sd, h->join2, 0));
+        TRY(launch_constant(pl.d_C, pl.d_Rbox, P, L.mean, zero_mean ? 1 : 0, sd));
+        h->launches += 1;
+    }
     TRY(cudaEventRecord(h->join, sd));
-    if (L.sym)
-        TRY(launch_sym_reduce(L.part_n, N, sym_band_launch(L, L.sym_bands - 1, false, h->debug_limit), L.phi_n,
-                              L.grad_n, st, !fp32, L.sym_bands > 1));
-    else
-        TRY(launch_near_reduce(L.part_n, sep ? T : N, tile, 4, L.Ln, L.phi_n, L.grad_n, st));
-    h->launches += 4;   // two near-field kernels, two reductions
+    // the RBF far field reads reduced sums; the other far fields add up the slots themselves
+    const NearSymLaunch last = L.sym ? sym_band_launch(L, L.sym_bands - 1, false, h->debug_limit) : NearSymLaunch{};
+    if (rbf) {
+        if (L.sym)
+            TRY(launch_sym_reduce(L.part_n, N, last, L.phi_n, L.grad_n, st, !fp32, L.sym_bands > 1));
+        else
+            TRY(launch_near_reduce(L.part_n, sep ? T : N, tile, 4, L.Ln, L.phi_n, L.grad_n, st));
+        h->launches += 1;
+    }
+    h->launches += 3;   // two near-field kernels, the check sums' reduction
     if (h->profile) TRY(cudaEventRecord(h->ev[3], st));
-    // join: the far field needs the coefficients
+    // join: the far field needs the coefficients and the mean
     TRY(cudaStreamWaitEvent(st, h->join, 0));
+    TRY(cudaStreamWaitEvent(st, h->join2, 0));
     if (h->profile) TRY(cudaEventRecord(h->ev[4], st));
     const int64_t NE = sep ? T : N;
-    if (o.basis == PSUM_BASIS_RBF)
+    if (rbf) {
         TRY(launch_far_rbf(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C, pl.d_rbf, pl.P - 1,
                            L.eval_status, phi, grad, L.eval_status, pl.d_status, st));
-    else if (far64)
-        TRY(launch_far64(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C4, o.p, 1.0 / pl.R0, pl.d_shtab64,
-                         L.eval_status, phi, grad, L.eval_status, pl.d_status, st));
-    else
-        TRY(launch_far_combine(ex, NE, eperm, L.phi_n, grad ? L.grad_n : nullptr, pl.d_C, o.p, 1.0 / pl.R0,
-                               pl.d_shtab32, L.eval_status, phi, grad, L.eval_status, pl.d_status, st));
-    h->launches += 3;   // projection, constant, far field
+    } else {
+        NearSlots a{};
+        a.partial = L.part_n;
+        a.sym = L.sym ? 1 : 0;
+        a.tile = tile;
+        a.near = L.Ln.tab.one;
+        a.U = L.Ln.U;
+        a.W = L.Ln.W;
+        a.max_contrib = L.Ln.max_contrib;
+        if (L.sym) {
+            a.symsys = last.tab.one;
+            a.limit = sym_limit(last);
+            if (L.sym_bands > 1) {
+                a.phi_acc = L.phi_n;
+                a.grad_acc = L.grad_n;
+            }
+        } else {
+            a.limit = L.n_tiles * L.Ln.max_contrib * 4 * tile;
+        }
+        a.status = L.eval_status;
+        FarArgs f{ex, NE, eperm, pl.d_C, pl.d_Rbox, L.mean, zero_mean ? 1 : 0, o.p, 1.0 / pl.R0, phi, grad, pl.d_status};
+        if (o.precision == PSUM_FP32C)
+            TRY(launch_sum_far32(f, a, pl.d_shtab32, st));
+        else
+            TRY(launch_sum_far64(f, a, pl.d_shtab64, pl.d_gradtab, st));
+    }
+    h->launches += 3;   // projection, totals, far field
     if (h->profile) TRY(cudaEventRecord(h->ev[5], st));
     return PSUM_OK;
 }

@@ -184,38 +184,40 @@ __global__ void __launch_bounds__(kProjThreads) k_project(const double* __restri
     if (lane == 0) C[1 + row] = s;
 }
 
-// Step 6 (Eq. pfx3 with phi_mean = 0): C_1 = -<phi_near> - sum_{t>=2} C_t R_t^(0); and the end of
-// the validation: the charges' total against their absolute sum (Eq. 1).
-__global__ void __launch_bounds__(kRedThreads) k_constant(double* __restrict__ C, const double* __restrict__ Rbox,
-                                                          int P, const double* __restrict__ mean_partial, int nblk,
-                                                          double inv_V0, int zero_mean,
-                                                          const double* __restrict__ val_partial, int nblk_val,
-                                                          int* __restrict__ status, double4_32a* __restrict__ C4,
-                                                          const double* __restrict__ gt, int p) {
-    double s = 0.0, m = 0.0, qs = 0.0, qa = 0.0;
-    if (C4)                                    // the coefficients with the gradient's (C_1 below)
-        for (int t = threadIdx.x; t < P; t += kRedThreads) {
-            double4_32a c = make_double4_32a(C[t], 0.0, 0.0, 0.0);
-            grad_coeffs(C, gt, p, t, c.y, c.z, c.w);
-            if (t) C4[t] = c;
-            else C4[0].y = c.y, C4[0].z = c.z, C4[0].w = c.w;
-        }
-    if (zero_mean) {
-        for (int t = 1 + threadIdx.x; t < P; t += kRedThreads) s = fma(C[t], Rbox[t], s);
-        for (int b = threadIdx.x; b < nblk; b += kRedThreads) m += mean_partial[b];
-    }
+// The box mean of phi_near (Eq. pfx4) from its partial sums, and the end of the validation: the
+// charges' total against their absolute sum (Eq. 1).
+__global__ void __launch_bounds__(kRedThreads) k_totals(const double* __restrict__ mean_partial, int nblk,
+                                                        double inv_V0, const double* __restrict__ val_partial,
+                                                        int nblk_val, int* __restrict__ status,
+                                                        double* __restrict__ mean) {
+    double m = 0.0, dummy = 0.0, qs = 0.0, qa = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += kRedThreads) m += mean_partial[b];
     for (int b = threadIdx.x; b < nblk_val; b += kRedThreads) {
         qs += val_partial[2 * b];
         qa += val_partial[2 * b + 1];
     }
-    block_sum2<kRedThreads>(s, m);
-    if (threadIdx.x == 0) {
-        C[0] = zero_mean ? (-m * inv_V0 - s) : 0.0;
-        if (C4) C4[0].x = C[0];
-    }
+    block_sum2<kRedThreads>(m, dummy);
+    if (threadIdx.x == 0) *mean = m * inv_V0;
     __syncthreads();                           // block_sum2's shared sums are free again
     block_sum2<kRedThreads>(qs, qa);
     if (threadIdx.x == 0 && !(fabs(qs) <= 1e-12 * qa)) atomicOr(status, kStatNonNeutral);
+}
+
+// Step 6 (Eq. pfx3 with phi_mean = 0): C_1 = -<phi_near> - sum_{t>=2} C_t R_t^(0), by one warp; every
+// lane returns it.
+__device__ __forceinline__ double constant_term(const double* __restrict__ C, const double* __restrict__ Rbox, int P,
+                                                const double* __restrict__ mean, int zero_mean) {
+    if (!zero_mean) return 0.0;
+    double s = 0.0;
+#pragma unroll 4
+    for (int t = 1 + (threadIdx.x & 31); t < P; t += 32) s = fma(C[t], Rbox[t], s);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return -*mean - s;
+}
+__global__ void k_constant(double* __restrict__ C, const double* __restrict__ Rbox, int P,
+                           const double* __restrict__ mean, int zero_mean) {
+    const double c = constant_term(C, Rbox, P, mean, zero_mean);
+    if (threadIdx.x == 0) C[0] = c;
 }
 
 // The evaluation's status joins the plan's (psum_sync reads it): what was flagged before this
@@ -235,121 +237,191 @@ __device__ __forceinline__ void flag_nonfinite(int* status, int* plan_status) {
 // ---------------------------------------------------------------------------
 constexpr int kFarThreads = 128;
 
-// FP32C plans: in float32, a smooth, slowly varying part of phi (its float32 evaluation errors sit
-// well below the pair sum's)
-__global__ void __launch_bounds__(kFarThreads) k_far_combine(const double* __restrict__ x, int64_t n,
-                                                             const int* __restrict__ perm,
-                                                             const double* __restrict__ phi_near,
-                                                             const double* __restrict__ grad_near,
-                                                             const double* __restrict__ C, int p, double inv_R0,
-                                                             const float* __restrict__ tab,
-                                                             const int* __restrict__ status,
-                                                             double* __restrict__ phi, double* __restrict__ grad,
-                                                             int* __restrict__ status_out, int* __restrict__ plan_status) {
-    merge_status(status, plan_status);
-    extern __shared__ unsigned char s_raw[];
-    const int P = (p + 1) * (p + 1);
-    const int nt = sh_tab_size(p);
-    using T = float;
-    T* s_C = (T*)s_raw;
-    T* s_tab = s_C + P;
-    for (int t = threadIdx.x; t < P; t += kFarThreads) s_C[t] = (T)C[t];
-    for (int t = threadIdx.x; t < nt; t += kFarThreads) s_tab[t] = tab[t];
-    __syncthreads();
-    const int64_t s = (int64_t)blockIdx.x * kFarThreads + threadIdx.x;
-    if (s >= n) return;
-    const int64_t i = perm ? (int64_t)perm[s] : s;
-    const bool failed = (*status & (kStatNonNeutral | kStatOutOfBox | kStatNonFinite | kStatTimeout | kStatBounds)) != 0;
-    if (failed) {
-        phi[i] = __longlong_as_double(0x7ff8000000000000ll);
-        if (grad) grad[3 * i] = grad[3 * i + 1] = grad[3 * i + 2] = __longlong_as_double(0x7ff8000000000000ll);
-        return;
+//
+// The kernels also add up the pair sums' partial slots (NearSlots): a block of 32 points has eight
+// warps for the slots (every eighth each, combined in a fixed order) beside those that evaluate the
+// expansion, so neither a reduction launch nor its latency stands before the far field, and C_1 is
+// formed by each block for itself (the first one stores it).  As launches of their own the reduction
+// and the constant took 5 to 12 us each on the way of a small evaluation.
+struct SlotRow {
+    int64_t r1, e1, r2, n;      // entries [0, e1) sit at r1 + e, the others at r2 + e - e1
+};
+
+// A point's slots: the work items that touch its tile (one-sided kernels), or the tile's row of the
+// symmetric kernels' last band (see k_sym_reduce).
+__device__ __forceinline__ SlotRow slot_row(const NearSlots& a, int64_t tile) {
+    if (!a.sym) {
+        const int64_t upt = a.near.n_chunks * a.near.n_img, first = tile * upt;
+        const int64_t n = sk_owner(first + upt - 1, a.U, a.W) - sk_owner(first, a.U, a.W) + 1;
+        return SlotRow{tile * a.max_contrib, n, 0, n};
     }
-    const T ux = (T)(x[3 * i] * inv_R0), uy = (T)(x[3 * i + 1] * inv_R0), uz = (T)(x[3 * i + 2] * inv_R0);
-    T f = 0, gx = 0, gy = 0, gz = 0;
-    if (grad) {
-        sh_visit_tab<true>(ux, uy, uz, p, s_tab, [&](int nn, int mm, T v, T vx, T vy, T vz) {
-            const T c = s_C[sh_index(nn, mm)];
-            f = fma(c, v, f);
-            gx = fma(c, vx, gx);
-            gy = fma(c, vy, gy);
-            gz = fma(c, vz, gz);
-        });
-    } else {
-        sh_visit_tab<false>(ux, uy, uz, p, s_tab, [&](int nn, int mm, T v, T, T, T) {
-            f = fma(s_C[sh_index(nn, mm)], v, f);
-        });
-    }
-    // the t = 1 term of the sum is C_1 R^_0^0 = C_1: included by the visitor
-    const double ph = phi_near[s] + (double)f;
-    phi[i] = ph;
-    bool finite = fabs(ph) <= 1.7976931348623157e308;
-    if (grad) {
-        const double g0 = grad_near[3 * s] + (double)gx * inv_R0;
-        const double g1 = grad_near[3 * s + 1] + (double)gy * inv_R0;
-        const double g2 = grad_near[3 * s + 2] + (double)gz * inv_R0;
-        grad[3 * i] = g0;
-        grad[3 * i + 1] = g1;
-        grad[3 * i + 2] = g2;
-        finite = finite && fabs(g0) <= 1.7976931348623157e308 && fabs(g1) <= 1.7976931348623157e308 &&
-                 fabs(g2) <= 1.7976931348623157e308;
-    }
-    if (!finite) flag_nonfinite(status_out, plan_status);
+    const SymSys& S = a.symsys;
+    if (tile < S.a0) return SlotRow{0, 0, 0, 0};
+    const int64_t bw = S.a1 - S.a0, n_out = tile < S.a1 ? S.n_tiles - S.a1 : 0;
+    return SlotRow{sym_slot(S, tile, S.a0) * S.n_g, bw * S.n_g, n_out > 0 ? sym_slot(S, tile, S.a1) * S.n_g : 0,
+                   (bw + n_out) * S.n_g};
 }
 
-// FP64 and FF plans: in float64, the columns of the expansion shared out to the warps of a block of
-// 32 points (harmonics.cuh); C4 holds each coefficient with the gradient's.  One thread per point
-// with the gradient carried through the recurrence kept the float64 pipes of a few SMs busy for
-// 61 us at 1000 charges and degree 8 (a float64 warp instruction takes a scheduler 64 cycles);
-// this takes about a quarter of the operations and spreads them over four times the schedulers.
+// Warp w's share of the sums of packed point i: potential, then field components with kGrad.
 template <bool kGrad>
-__global__ void k_far64(const double* __restrict__ x, int64_t n, const int* __restrict__ perm,
-                        const double* __restrict__ phi_near, const double* __restrict__ grad_near,
-                        const double4_32a* __restrict__ C4, int p, double inv_R0, const double* __restrict__ tab,
-                        const int* __restrict__ status, double* __restrict__ phi, double* __restrict__ grad,
-                        int* __restrict__ status_out, int* __restrict__ plan_status) {
-    merge_status(status, plan_status);
-    extern __shared__ double4_32a s_C4[];
-    const int P = (p + 1) * (p + 1), nt = sh_tab_size(p), W = blockDim.x / 32;
-    double* s_red = (double*)(s_C4 + P);              // [W][4][32]
-    double* s_tab = s_red + W * 4 * 32;
-    for (int t = threadIdx.x; t < P; t += blockDim.x) s_C4[t] = C4[t];
-    for (int t = threadIdx.x; t < nt; t += blockDim.x) s_tab[t] = tab[t];
+__device__ __forceinline__ void slot_sums(const NearSlots& a, int64_t i, int w, double (&acc)[4]) {
+    const int64_t tile = i / a.tile;
+    const SlotRow r = slot_row(a, tile);
+    const double* base = a.partial + (i - tile * a.tile);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] = 0.0;
+#pragma unroll 4
+    for (int64_t k = w; k < r.n; k += kSlotWarps) {
+        const int64_t off = (k < r.e1 ? r.r1 + k : r.r2 + (k - r.e1)) * 4 * a.tile;
+        if (!debug_in_range(off, 4 * a.tile, a.limit, a.status, 1)) continue;
+#pragma unroll
+        for (int c = 0; c < (kGrad ? 4 : 1); ++c) acc[c] += base[off + c * a.tile];
+    }
+}
+
+// One output of one point (c = 0: the potential, 1..3: the field) from the slot sums of the eight
+// warps, the earlier bands' sums and the far field's value.
+__device__ __forceinline__ void write_point(const NearSlots& a, const double* s_part, int lane, int64_t s, int64_t i,
+                                            int c, double far, bool failed, double* phi, double* grad, int* status,
+                                            int* plan_status) {
+    double v = s_part[c * 32 + lane];
+#pragma unroll
+    for (int w = 1; w < kSlotWarps; ++w) v += s_part[(w * 4 + c) * 32 + lane];
+    if (a.phi_acc) v = (c == 0 ? a.phi_acc[s] : a.grad_acc[3 * s + c - 1]) + v;
+    const double r = failed ? __longlong_as_double(0x7ff8000000000000ll) : v + far;
+    if (c == 0)
+        phi[i] = r;
+    else
+        grad[3 * i + c - 1] = r;
+    if (!failed && !(fabs(r) <= 1.7976931348623157e308)) {
+        atomicOr(status, kStatNonFinite);
+        atomicOr(plan_status, kStatNonFinite);
+    }
+}
+constexpr int kStatFailed = kStatNonNeutral | kStatOutOfBox | kStatNonFinite | kStatTimeout | kStatBounds;
+
+// FP32C plans: the far field in float32, a smooth, slowly varying part of phi (its float32
+// evaluation errors sit well below the pair sum's), by the block's ninth warp.
+template <bool kGrad>
+__global__ void __launch_bounds__(32 * (kSlotWarps + 1)) k_sum_far32(FarArgs f, NearSlots a,
+                                                                     const float* __restrict__ tab) {
+    merge_status(a.status, f.plan_status);
+    extern __shared__ unsigned char s_raw[];
+    const int p = f.p, P = (p + 1) * (p + 1), nt = sh_tab_size(p);
+    double* s_part = (double*)s_raw;                   // [8][4][32], then the far field's [4][32]
+    double* s_far = s_part + kSlotWarps * 4 * 32;
+    float* s_C = (float*)(s_far + 4 * 32);
+    float* s_tab = s_C + P;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t s = (int64_t)blockIdx.x * 32 + lane;
-    const bool live = s < n;
-    const int64_t i = live ? (perm ? (int64_t)perm[s] : s) : 0;
-    const double ux = x[3 * i] * inv_R0, uy = x[3 * i + 1] * inv_R0, uz = x[3 * i + 2] * inv_R0;
-    __syncthreads();
-    double f = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
-    harmonic_columns(ux, uy, uz, p, w, s_tab, [&](int t, double v) {
-        const double4_32a c = s_C4[t];
-        f = fma(c.x, v, f);
+    const bool live = s < f.n;
+    const int64_t i = live ? (f.perm ? (int64_t)f.perm[s] : s) : 0;
+    if (w == kSlotWarps) {
+        const double c1 = constant_term(f.C, f.Rbox, P, f.mean, f.zero_mean);
+        if (blockIdx.x == 0 && lane == 0) f.C[0] = c1;
+        for (int t = lane; t < P; t += 32) s_C[t] = (float)(t ? f.C[t] : c1);
+        for (int t = lane; t < nt; t += 32) s_tab[t] = tab[t];
+        __syncwarp();
+        const float ux = (float)(f.x[3 * i] * f.inv_R0), uy = (float)(f.x[3 * i + 1] * f.inv_R0),
+                    uz = (float)(f.x[3 * i + 2] * f.inv_R0);
+        float v = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
+        // the t = 1 term of the sum is C_1 R^_0^0 = C_1: included by the visitor
+        sh_visit_tab<kGrad>(ux, uy, uz, p, s_tab, [&](int nn, int mm, float h, float hx, float hy, float hz) {
+            const float c = s_C[sh_index(nn, mm)];
+            v = fma(c, h, v);
+            if (kGrad) {
+                gx = fma(c, hx, gx);
+                gy = fma(c, hy, gy);
+                gz = fma(c, hz, gz);
+            }
+        });
+        s_far[lane] = (double)v;
         if (kGrad) {
-            gx = fma(c.y, v, gx);
-            gy = fma(c.z, v, gy);
-            gz = fma(c.w, v, gz);
+            s_far[32 + lane] = (double)gx * f.inv_R0;
+            s_far[64 + lane] = (double)gy * f.inv_R0;
+            s_far[96 + lane] = (double)gz * f.inv_R0;
         }
-    });
-    s_red[(w * 4) * 32 + lane] = f;
-    if (kGrad) {
-        s_red[(w * 4 + 1) * 32 + lane] = gx;
-        s_red[(w * 4 + 2) * 32 + lane] = gy;
-        s_red[(w * 4 + 3) * 32 + lane] = gz;
+    } else if (live) {
+        double acc[4];
+        slot_sums<kGrad>(a, s, w, acc);
+#pragma unroll
+        for (int c = 0; c < (kGrad ? 4 : 1); ++c) s_part[(w * 4 + c) * 32 + lane] = acc[c];
     }
     __syncthreads();
-    // warp 0 finishes the potential, the next ones a field component each (a fixed order of warps)
-    for (int c = w; c < (kGrad ? 4 : 1) && live; c += W) {
-        double v = s_red[c * 32 + lane];
-        for (int k = 1; k < W; ++k) v += s_red[(k * 4 + c) * 32 + lane];
-        const bool failed = (*status & (kStatNonNeutral | kStatOutOfBox | kStatNonFinite | kStatTimeout | kStatBounds)) != 0;
-        const double r = failed ? __longlong_as_double(0x7ff8000000000000ll)
-                                : c == 0 ? phi_near[s] + v : grad_near[3 * s + c - 1] + v * inv_R0;
-        if (c == 0)
-            phi[i] = r;
-        else
-            grad[3 * i + c - 1] = r;
-        if (!failed && !(fabs(r) <= 1.7976931348623157e308)) flag_nonfinite(status_out, plan_status);
+    if (w < (kGrad ? 4 : 1) && live)
+        write_point(a, s_part, lane, s, i, w, s_far[w * 32 + lane], (*a.status & kStatFailed) != 0, f.phi, f.grad,
+                    a.status, f.plan_status);
+}
+
+// FP64 and FF plans: in float64, the columns of the expansion shared out to the other warps of the
+// block (harmonics.cuh), which form each coefficient with the gradient's first.  One thread per point
+// with the gradient carried through the recurrence kept the float64 pipes of a few SMs busy for
+// 61 us at 1000 charges and degree 8 (a float64 warp instruction takes a scheduler 64 cycles); by
+// columns, a launch of its own, 12 us.
+constexpr int kFar64Threads = 32 * (kSlotWarps + (kMaxDegree + 2) / 2);
+
+template <bool kGrad>
+__global__ void __launch_bounds__(kFar64Threads) k_sum_far64(FarArgs f, NearSlots a, const double* __restrict__ tab,
+                                                             const double* __restrict__ grad_tab) {
+    merge_status(a.status, f.plan_status);
+    extern __shared__ double4_32a s_C4[];
+    const int p = f.p, P = (p + 1) * (p + 1), nt = sh_tab_size(p), W = blockDim.x / 32 - kSlotWarps;
+    double* s_part = (double*)(s_C4 + P);              // [8][4][32]
+    double* s_red = s_part + kSlotWarps * 4 * 32;      // [W][4][32]
+    double* s_tab = s_red + W * 4 * 32;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t s = (int64_t)blockIdx.x * 32 + lane;
+    const bool live = s < f.n;
+    const int64_t i = live ? (f.perm ? (int64_t)f.perm[s] : s) : 0;
+    if (w >= kSlotWarps) {
+        const int t0 = threadIdx.x - 32 * kSlotWarps;
+        if (w == kSlotWarps) {
+            const double c1 = constant_term(f.C, f.Rbox, P, f.mean, f.zero_mean);
+            if (lane == 0) {
+                s_C4[0].x = c1;
+                if (blockIdx.x == 0) f.C[0] = c1;
+            }
+        }
+        for (int t = t0; t < P; t += 32 * W) {
+            double cx = 0.0, cy = 0.0, cz = 0.0;
+            if (kGrad) grad_coeffs(f.C, grad_tab, p, t, cx, cy, cz);
+            if (t) s_C4[t].x = f.C[t];
+            s_C4[t].y = cx;
+            s_C4[t].z = cy;
+            s_C4[t].w = cz;
+        }
+        for (int t = t0; t < nt; t += 32 * W) s_tab[t] = tab[t];
+        const double ux = f.x[3 * i] * f.inv_R0, uy = f.x[3 * i + 1] * f.inv_R0, uz = f.x[3 * i + 2] * f.inv_R0;
+        asm volatile("bar.sync 1, %0;" ::"r"(32 * W) : "memory");    // the column warps among themselves
+        double v = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+        harmonic_columns(ux, uy, uz, p, w - kSlotWarps, s_tab, [&](int t, double h) {
+            const double4_32a c = s_C4[t];
+            v = fma(c.x, h, v);
+            if (kGrad) {
+                gx = fma(c.y, h, gx);
+                gy = fma(c.z, h, gy);
+                gz = fma(c.w, h, gz);
+            }
+        });
+        double* r = s_red + (w - kSlotWarps) * 4 * 32 + lane;
+        r[0] = v;
+        if (kGrad) {
+            r[32] = gx;
+            r[64] = gy;
+            r[96] = gz;
+        }
+    } else if (live) {
+        double acc[4];
+        slot_sums<kGrad>(a, s, w, acc);
+#pragma unroll
+        for (int c = 0; c < (kGrad ? 4 : 1); ++c) s_part[(w * 4 + c) * 32 + lane] = acc[c];
+    }
+    __syncthreads();
+    if (w < (kGrad ? 4 : 1) && live) {
+        double v = s_red[w * 32 + lane];
+        for (int k = 1; k < W; ++k) v += s_red[(k * 4 + w) * 32 + lane];
+        write_point(a, s_part, lane, s, i, w, w == 0 ? v : v * f.inv_R0, (*a.status & kStatFailed) != 0, f.phi, f.grad,
+                    a.status, f.plan_status);
     }
 }
 
@@ -452,9 +524,12 @@ cudaError_t launch_prepare(const double* x, const double* q, int64_t n, const do
     return cudaGetLastError();
 }
 
+// At most four blocks an SM: two warps a scheduler keep its float64 pipe busy, and the mean, which
+// starts first, leaves registers for the sort and the packing beside it (with sixteen they waited for
+// its first wave: 117 us until the pair sum at 20 000 charges, of which 62 us of their own).
 int mean_blocks(int64_t n, int num_sms) {
     int64_t nb = (kMeanTerms * n + kMeanThreads - 1) / kMeanThreads;
-    const int64_t cap = 16LL * num_sms;
+    const int64_t cap = 4LL * num_sms;
     if (nb > cap) nb = cap;
     return nb < 1 ? 1 : (int)nb;
 }
@@ -479,37 +554,35 @@ cudaError_t launch_project(const double* pinv, int rows, int M, const double* ph
     return cudaGetLastError();
 }
 
-cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean_partial, int nblk,
-                            double inv_V0, int zero_mean, const double* val_partial, int nblk_val, int* status,
-                            cudaStream_t st, double4_32a* C4, const double* grad_tab, int p) {
-    k_constant<<<1, kRedThreads, 0, st>>>(C, Rbox, P, mean_partial, nblk, inv_V0, zero_mean, val_partial, nblk_val,
-                                          status, C4, grad_tab, p);
+cudaError_t launch_totals(const double* mean_partial, int nblk, double inv_V0, const double* val_partial, int nblk_val,
+                          int* status, double* mean, cudaStream_t st) {
+    k_totals<<<1, kRedThreads, 0, st>>>(mean_partial, nblk, inv_V0, val_partial, nblk_val, status, mean);
     return cudaGetLastError();
 }
 
-cudaError_t launch_far_combine(const double* x, int64_t n, const int* perm, const double* phi_near,
-                               const double* grad_near, const double* C, int p, double inv_R0, const float* tab32,
-                               const int* status, double* phi, double* grad, int* status_out, int* plan_status,
-                               cudaStream_t st) {
-    const int P = (p + 1) * (p + 1);
-    const unsigned nb = (unsigned)((n + kFarThreads - 1) / kFarThreads);
-    k_far_combine<<<nb, kFarThreads, sizeof(float) * (P + sh_tab_size(p)), st>>>(
-        x, n, perm, phi_near, grad_near, C, p, inv_R0, tab32, status, phi, grad, status_out, plan_status);
+cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean, int zero_mean, cudaStream_t st) {
+    k_constant<<<1, 32, 0, st>>>(C, Rbox, P, mean, zero_mean);
     return cudaGetLastError();
 }
 
-cudaError_t launch_far64(const double* x, int64_t n, const int* perm, const double* phi_near, const double* grad_near,
-                         const double4_32a* C4, int p, double inv_R0, const double* tab64, const int* status,
-                         double* phi, double* grad, int* status_out, int* plan_status, cudaStream_t st) {
-    const int W = harmonic_warps(p);
-    const size_t smem = sizeof(double4_32a) * (size_t)(p + 1) * (p + 1) + sizeof(double) * (W * 128 + sh_tab_size(p));
-    const auto kernel = grad ? k_far64<true> : k_far64<false>;
+cudaError_t launch_sum_far32(const FarArgs& f, const NearSlots& a, const float* tab32, cudaStream_t st) {
+    const int P = (f.p + 1) * (f.p + 1);
+    const size_t smem = sizeof(double) * (kSlotWarps + 1) * 128 + sizeof(float) * (P + sh_tab_size(f.p));
+    const auto kernel = f.grad ? k_sum_far32<true> : k_sum_far32<false>;
+    kernel<<<(unsigned)((f.n + 31) / 32), 32 * (kSlotWarps + 1), smem, st>>>(f, a, tab32);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sum_far64(const FarArgs& f, const NearSlots& a, const double* tab64, const double* grad_tab,
+                             cudaStream_t st) {
+    const int P = (f.p + 1) * (f.p + 1), W = harmonic_warps(f.p);
+    const size_t smem = sizeof(double4_32a) * P + sizeof(double) * ((W + kSlotWarps) * 128 + sh_tab_size(f.p));
+    const auto kernel = f.grad ? k_sum_far64<true> : k_sum_far64<false>;
     if (smem > 48 * 1024) {              // high degrees
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kernel<<<(unsigned)((n + 31) / 32), 32 * W, smem, st>>>(x, n, perm, phi_near, grad_near, C4, p, inv_R0, tab64, status,
-                                                           phi, grad, status_out, plan_status);
+    kernel<<<(unsigned)((f.n + 31) / 32), 32 * (W + kSlotWarps), smem, st>>>(f, a, tab64, grad_tab);
     return cudaGetLastError();
 }
 

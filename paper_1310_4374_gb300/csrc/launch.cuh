@@ -94,18 +94,58 @@ cudaError_t launch_box_mean_ball(const double* x, const double* q, const uint32_
                                  cudaStream_t st);
 cudaError_t launch_project(const double* pinv, int rows, int M, const double* phi_check, const int* check_pos,
                            double* C, cudaStream_t st, bool layers = false);
-cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean_partial, int nblk,
-                            double inv_V0, int zero_mean, const double* val_partial, int nblk_val, int* status,
-                            cudaStream_t st, double4_32a* C4 = nullptr, const double* grad_tab = nullptr, int p = 0);
-// the far field and the sum: in float32 (FP32C plans), or in float64 from the coefficients with the
-// gradient's that launch_constant has formed
-cudaError_t launch_far_combine(const double* x, int64_t n, const int* perm, const double* phi_near,
-                               const double* grad_near, const double* C, int p, double inv_R0, const float* tab32,
-                               const int* status, double* phi, double* grad, int* status_out, int* plan_status,
-                               cudaStream_t st);
-cudaError_t launch_far64(const double* x, int64_t n, const int* perm, const double* phi_near, const double* grad_near,
-                         const double4_32a* C4, int p, double inv_R0, const double* tab64, const int* status,
-                         double* phi, double* grad, int* status_out, int* plan_status, cudaStream_t st);
+// the box mean of phi_near from its partial sums (nblk of them; 0 without the mean condition) and the
+// end of the validation
+cudaError_t launch_totals(const double* mean_partial, int nblk, double inv_V0, const double* val_partial, int nblk_val,
+                          int* status, double* mean, cudaStream_t st);
+// C_1 as a launch of its own (RBF plans)
+cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* mean, int zero_mean, cudaStream_t st);
+// the pair sums' partial slots as the far-field kernels read them
+struct NearSlots {
+    const double* partial;
+    int sym;                    // 1: the symmetric kernels' last band (symsys), 0: one-sided (near, U, W)
+    int tile;                   // targets per tile
+    NearSys near;
+    SymSys symsys;
+    int64_t U, W;
+    int max_contrib;
+    const double *phi_acc, *grad_acc;   // sums of the earlier bands (null: none)
+    int64_t limit;              // doubles of the partial buffer (debug bounds checks)
+    int* status;
+};
+struct FarArgs {
+    const double* x;            // the points, caller order
+    int64_t n;
+    const int* perm;            // packed order (null: the caller's)
+    double* C;                  // C_2..C_P in, C_1 out
+    const double* Rbox;
+    const double* mean;
+    int zero_mean, p;
+    double inv_R0;
+    double *phi, *grad;
+    int* plan_status;
+};
+// the sum of near and far field at the points, written in the caller's order: the far field in
+// float32 (FP32C plans) or float64
+cudaError_t launch_sum_far32(const FarArgs& f, const NearSlots& a, const float* tab32, cudaStream_t st);
+cudaError_t launch_sum_far64(const FarArgs& f, const NearSlots& a, const double* tab64, const double* grad_tab,
+                             cudaStream_t st);
+int64_t sym_limit(const NearSymLaunch& S);   // doubles of the partial buffer as the debug checks see it
+constexpr int kSlotWarps = 8;
+
+// Debug builds (-DPSUM_DEBUG_CHECKS=1) check every write and read of the pair kernels'
+// partial sums against the buffer's size: an access outside it is skipped and flagged in the
+// launch's status words (kStatBounds, PSUM_ERR_INTERNAL at psum_sync) instead of faulting.
+__device__ __forceinline__ bool debug_in_range(int64_t off, int64_t n, int64_t limit, int* status, int n_status) {
+#if PSUM_DEBUG_CHECKS
+    if (off < 0 || off + n > limit) {
+        for (int k = 0; k < n_status; ++k) atomicOr(status + k, kStatBounds);
+        return false;
+    }
+#endif
+    return true;
+}
+
 // backward.cu
 // the moments w (P) of the charges and the far field of the coefficients C at them; C4: P scratch
 cudaError_t launch_moments(const double* x, const double* q, int64_t n, const double* C, double4_32a* C4, int p,

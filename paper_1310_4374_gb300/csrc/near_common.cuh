@@ -412,19 +412,6 @@ __device__ __forceinline__ double rsqrt_f64_k0(double r2) {
     return r2f > 0.f ? ri : 0.0;
 }
 
-// Debug builds (-DPSUM_DEBUG_CHECKS=1) check every write and read of the pair kernels'
-// partial sums against the buffer's size: an access outside it is skipped and flagged in the
-// launch's status words (kStatBounds, PSUM_ERR_INTERNAL at psum_sync) instead of faulting.
-__device__ __forceinline__ bool debug_in_range(int64_t off, int64_t n, int64_t limit, int* status, int n_status) {
-#if PSUM_DEBUG_CHECKS
-    if (off < 0 || off + n > limit) {
-        for (int k = 0; k < n_status; ++k) atomicOr(status + k, kStatBounds);
-        return false;
-    }
-#endif
-    return true;
-}
-
 // warps of the reduction kernels (fixed-order combination of the partial slots)
 constexpr int kReduceWarps = 8;
 

@@ -611,7 +611,6 @@ int build_plan(const psum_opts& o, Plan& pl) {
             std::vector<double> gt(grad_tab_size(p));
             grad_tab_fill(p, gt.data());
             if ((s2 = upload(&pl.d_gradtab, gt.data(), gt.size()))) return s2;
-            PSUM_CUDA_TRY(cudaMalloc((void**)&pl.d_C4, sizeof(double4_32a) * pl.P));
         }
     }
     PSUM_CUDA_TRY(cudaMalloc((void**)&pl.d_C, sizeof(double) * pl.P));
@@ -648,7 +647,6 @@ void free_plan_device(Plan& pl) {
     cudaFree(pl.d_shtab64);
     cudaFree(pl.d_shtab32);
     cudaFree(pl.d_gradtab);
-    cudaFree(pl.d_C4);
     cudaFree(pl.d_C);
     cudaFree(pl.d_status);
     if (pl.h_status) cudaFreeHost(pl.h_status);

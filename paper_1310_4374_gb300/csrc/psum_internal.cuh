@@ -348,7 +348,6 @@ struct Plan {
     double* d_shifts = nullptr;
     double* d_rbf = nullptr;        // RBF basis: the n_rbf centres, 3 each
     double* d_C = nullptr;          // P coefficients of the last evaluation
-    double4_32a* d_C4 = nullptr;    // ... with those of the gradient (harmonics.cuh), float64 far fields
     int* d_status = nullptr;
     int* h_status = nullptr;        // pinned
 

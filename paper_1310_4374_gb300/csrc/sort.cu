@@ -366,6 +366,13 @@ cudaError_t launch_radix_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t
 // (20 000 points with four per lane: 51 us).
 constexpr int kRankWarps = 16;
 
+// min(max(a - b, 0), 1) in one instruction
+__device__ __forceinline__ float sub_sat(float a, float b) {
+    float r;
+    asm("sub.rn.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 template <int kPer>
 __global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const float* __restrict__ keys, int n,
                                                                 uint32_t* __restrict__ perm) {
@@ -389,10 +396,10 @@ __global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const float* __r
         const float4 k = k4[j];
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
-            c0[r] += __saturatef(key1[r] - k.x);
-            c1[r] += __saturatef(key1[r] - k.y);
-            c0[r] += __saturatef(key1[r] - k.z);
-            c1[r] += __saturatef(key1[r] - k.w);
+            c0[r] += sub_sat(key1[r], k.x);
+            c1[r] += sub_sat(key1[r], k.y);
+            c0[r] += sub_sat(key1[r], k.z);
+            c1[r] += sub_sat(key1[r], k.w);
         }
     }
 #pragma unroll 4
@@ -400,10 +407,10 @@ __global__ void __launch_bounds__(32 * kRankWarps) k_rank_order(const float* __r
         const float4 k = k4[j];
 #pragma unroll
         for (int r = 0; r < kPer; ++r) {
-            c0[r] += __saturatef(key[r] - k.x);
-            c1[r] += __saturatef(key[r] - k.y);
-            c0[r] += __saturatef(key[r] - k.z);
-            c1[r] += __saturatef(key[r] - k.w);
+            c0[r] += sub_sat(key[r], k.x);
+            c1[r] += sub_sat(key[r], k.y);
+            c0[r] += sub_sat(key[r], k.z);
+            c1[r] += sub_sat(key[r], k.w);
         }
     }
 #pragma unroll
