@@ -588,21 +588,20 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
         }
         // the weight (1, -1 or 0) goes onto the charge's bits: no float64 operation
         const int w_and = w != 0.0 ? -1 : 0, w_xor = w < 0.0 ? (int)0x80000000 : 0;
-#pragma unroll 4
+#pragma unroll 2
         for (int s = 0; s < kNearChunk; ++s) {
             const double4_32a Q = src[s];
             const double ex = Q.x - px, ey = Q.y - py, ez = Q.z - pz;   // x_i + p - y
             const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
-            const double ri = rsqrt_f64_k0(r2);           // K(0) = 0
             if (kGrad) {
-                acc[0] = fma(Q.w, ri, acc[0]);
-                const double g = Q.w * (ri * ri * ri);
+                const double g = Q.w * rsqrt3_f64_k0(r2);     // K(0) = 0
+                acc[0] = fma(g, r2, acc[0]);
                 acc[1 % NQ] = fma(ex, g, acc[1 % NQ]);
                 acc[2 % NQ] = fma(ey, g, acc[2 % NQ]);
                 acc[3 % NQ] = fma(ez, g, acc[3 % NQ]);
             } else {
                 const double qw = __hiloint2double((__double2hiint(Q.w) & w_and) ^ w_xor, __double2loint(Q.w) & w_and);
-                acc[0] = fma(qw, ri, acc[0]);
+                acc[0] = fma(qw, rsqrt_f64_k0(r2), acc[0]);
             }
         }
         ++u;

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "launch.cuh"
+#include "rsqrt64.cuh"
 
 namespace psum {
 
@@ -388,41 +389,18 @@ __device__ __forceinline__ void pair_loop_ff(const float4* __restrict__ s_hi, co
     }
 }
 
-// 1/sqrt(r2), or 0 for r2 = 0 (K(0) = 0, Eq. 1), in float64: the MUFU estimate y (relative error
-// below 2^-22) and one third-order correction: with e = 1 - r2 y^2,
-// 1/sqrt(r2) = y (1 - e)^(-1/2) = y + (y/2)(e + (3/4) e^2) + O(y e^3), whose truncation
-// (5/16)|e|^3 < 1e-19 is below float64 rounding.  The float64 pipe bounds these kernels (one warp
-// instruction per scheduler in 64 cycles, conversions included), so only e, its square's term and the
-// final multiply-add are float64 operations; the rest goes over the bit patterns on idle pipes:
-//   * the float32 copy of r2 keeps the top 23 mantissa bits (truncated, relative error below 2^-23,
-//     so |e| < 2^-21), the zero test is taken on it, and the estimate is widened exactly; r2 below
-//     2^-126 counts as zero, which would need two distinct charges within 1e-19 of each other;
-//   * y^2 is the exact 48-bit square of y's 24-bit mantissa, an integer product put back under its
-//     exponent;
-//   * the factor 3/4 e needs 10 bits: it is float32, widened.
-// Three float64 operations where the estimate's square, the series and its products took five.
+// 1/sqrt(r2) and r2^(-3/2), or 0 for r2 = 0 (K(0) = 0, Eq. 1), in float64: the MUFU estimate of the
+// float32 copy of r2, refined (rsqrt64.cuh); the zero test is taken on that copy (a float32 compare and
+// selects instead of a float64 compare).
 __device__ __forceinline__ double rsqrt_f64_k0(double r2) {
-    // float32 bits: the float64 exponent rebiased (1023 -> 127) and the mantissa cut to 23 bits
-    const long long t = (__double_as_longlong(r2) >> 29) - (896LL << 23);
-    const float r2f = __int_as_float(t >= 1LL << 23 ? (int)t : 0);
-    const uint32_t yb = __float_as_uint(rsqrt_mufu(r2f));
-    // float64 bits of the (positive, normal) estimate: exponent rebiased, mantissa widened
-    const long long yw = ((long long)yb << 29) + (896LL << 52);
-    // y^2 = 2^(2 E) (m / 2^23)^2 with m in [2^23, 2^24): a product of 47 or 48 bits, whose leading
-    // one, shifted to bit 52, adds itself to the exponent below it
-    const uint32_t m = (yb & 0x7fffffu) | 0x800000u;
-    const uint64_t mm = (uint64_t)m * m;
-    const int top = (int)(mm >> 47);                                   // 1: (m / 2^23)^2 >= 2
-    const long long ex = 2 * (long long)(yb >> 23) - 254 + 1022 + top;
-    const double yy = __longlong_as_double((ex << 52) + (long long)(mm << (6 - top)));
-    const double e = fma(-r2, yy, 1.0);
-    // 3/4 e from the top 20 mantissa bits of e; below 2^-100 its term adds nothing
-    const int eh = __double2hiint(e), ea = eh & 0x7fffffff;
-    const float ef = __int_as_float(ea > (923 << 20) ? (ea - (896 << 20)) << 3 : 0);
-    const uint32_t gb = __float_as_uint(0.75f * ef);
-    const double g = __hiloint2double((int)((gb >> 3) + (gb ? 896u << 20 : 0u)) | (eh & (int)0x80000000), (int)(gb << 29));
-    const double ri = fma(__longlong_as_double(yw - (1LL << 52)), fma(g, e, e), __longlong_as_double(yw));
+    const float r2f = estimate_arg(r2);
+    const double ri = rsqrt_refined(r2, __float_as_uint(rsqrt_mufu(r2f)));
     return r2f > 0.f ? ri : 0.0;
+}
+__device__ __forceinline__ double rsqrt3_f64_k0(double r2) {
+    const float r2f = estimate_arg(r2);
+    const double ri3 = rsqrt3_refined(r2, __float_as_uint(rsqrt_mufu(r2f)));
+    return r2f > 0.f ? ri3 : 0.0;
 }
 
 // warps of the reduction kernels (fixed-order combination of the partial slots)

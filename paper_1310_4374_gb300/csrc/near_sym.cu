@@ -915,9 +915,8 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
                 const double4_32a Q = s_src[s];
                 const double ex = Q.x - px, ey = Q.y - py, ez = Q.z - pz;
                 const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
-                const double ri = rsqrt_f64_k0(r2);      // K(0) = 0
-                acc[0] = fma(Q.w, ri, acc[0]);
-                const double w = Q.w * (ri * ri * ri);
+                const double w = Q.w * rsqrt3_f64_k0(r2);    // K(0) = 0
+                acc[0] = fma(w, r2, acc[0]);
                 acc[1] = fma(ex, w, acc[1]);
                 acc[2] = fma(ey, w, acc[2]);
                 acc[3] = fma(ez, w, acc[3]);
@@ -932,15 +931,14 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
                 const double4_32a Q = s_src[32 * g + ((lane + k) & 31)];
                 const double ex = Q.x - px, ey = Q.y - py, ez = Q.z - pz;   // x_s + p - y
                 const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
-                const double ri = rsqrt_f64_k0(r2);
-                const double ri3 = ri * ri * ri;
-                acc[0] = fma(Q.w, ri, acc[0]);           // action
-                const double wa = Q.w * ri3;
+                const double ri3 = rsqrt3_f64_k0(r2);
+                const double wa = Q.w * ri3;             // action
+                acc[0] = fma(wa, r2, acc[0]);
                 acc[1] = fma(ex, wa, acc[1]);
                 acc[2] = fma(ey, wa, acc[2]);
                 acc[3] = fma(ez, wa, acc[3]);
-                rp = fma(t.w, ri, rp);                   // reaction (field sign folded later)
-                const double wb = t.w * ri3;
+                const double wb = t.w * ri3;             // reaction (field sign folded later)
+                rp = fma(wb, r2, rp);
                 rx = fma(ex, wb, rx);
                 ry = fma(ey, wb, ry);
                 rz = fma(ez, wb, rz);
