@@ -316,14 +316,19 @@ __global__ void __launch_bounds__(32 * (kSlotWarps + 1)) k_sum_far32(FarArgs f, 
     const int64_t s = (int64_t)blockIdx.x * 32 + lane;
     const bool live = s < f.n;
     const int64_t i = live ? (f.perm ? (int64_t)f.perm[s] : s) : 0;
+    // every warp loads its part of the tables at once; the slot warps then go on without waiting
+    for (int t = threadIdx.x; t < P; t += 32 * (kSlotWarps + 1))
+        if (t) s_C[t] = (float)f.C[t];
+    for (int t = threadIdx.x; t < nt; t += 32 * (kSlotWarps + 1)) s_tab[t] = tab[t];
     if (w == kSlotWarps) {
+        const double x0 = f.x[3 * i], x1 = f.x[3 * i + 1], x2 = f.x[3 * i + 2];
         const double c1 = constant_term(f.C, f.Rbox, P, f.mean, f.zero_mean);
-        if (blockIdx.x == 0 && lane == 0) f.C[0] = c1;
-        for (int t = lane; t < P; t += 32) s_C[t] = (float)(t ? f.C[t] : c1);
-        for (int t = lane; t < nt; t += 32) s_tab[t] = tab[t];
-        __syncwarp();
-        const float ux = (float)(f.x[3 * i] * f.inv_R0), uy = (float)(f.x[3 * i + 1] * f.inv_R0),
-                    uz = (float)(f.x[3 * i + 2] * f.inv_R0);
+        if (lane == 0) {
+            if (blockIdx.x == 0) f.C[0] = c1;
+            s_C[0] = (float)c1;
+        }
+        asm volatile("bar.sync 1, %0;" ::"r"(32 * (kSlotWarps + 1)) : "memory");
+        const float ux = (float)(x0 * f.inv_R0), uy = (float)(x1 * f.inv_R0), uz = (float)(x2 * f.inv_R0);
         float v = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
         // the t = 1 term of the sum is C_1 R^_0^0 = C_1: included by the visitor
         sh_visit_tab<kGrad>(ux, uy, uz, p, s_tab, [&](int nn, int mm, float h, float hx, float hy, float hz) {
@@ -341,11 +346,14 @@ __global__ void __launch_bounds__(32 * (kSlotWarps + 1)) k_sum_far32(FarArgs f, 
             s_far[64 + lane] = (double)gy * f.inv_R0;
             s_far[96 + lane] = (double)gz * f.inv_R0;
         }
-    } else if (live) {
-        double acc[4];
-        slot_sums<kGrad>(a, s, w, acc);
+    } else {
+        asm volatile("bar.arrive 1, %0;" ::"r"(32 * (kSlotWarps + 1)) : "memory");
+        if (live) {
+            double acc[4];
+            slot_sums<kGrad>(a, s, w, acc);
 #pragma unroll
-        for (int c = 0; c < (kGrad ? 4 : 1); ++c) s_part[(w * 4 + c) * 32 + lane] = acc[c];
+            for (int c = 0; c < (kGrad ? 4 : 1); ++c) s_part[(w * 4 + c) * 32 + lane] = acc[c];
+        }
     }
     __syncthreads();
     if (w < (kGrad ? 4 : 1) && live)
