@@ -22,11 +22,13 @@ class _EnergyFn(torch.autograd.Function):
         N = q.numel()
         phi = torch.empty(N, dtype=torch.float64, device=x.device)
         grad = torch.empty((N, 3), dtype=torch.float64, device=x.device)
-        B.psum_eval(module.plan, x, q, phi, grad, check=module.check)
         E = torch.empty(1, dtype=torch.float64, device=x.device)
-        B.psum_energy(module.plan, q, phi, E)
         C = torch.empty(module.P, dtype=torch.float64, device=x.device)
+        B.psum_eval(module.plan, x, q, phi, grad)
+        B.psum_energy(module.plan, q, phi, E)
         B.psum_coeffs_device(module.plan, C)
+        if module.check:                       # after the energy and the copy are queued: one wait for all
+            B._check(B.psum_sync(module.plan), "psum_eval (device)")
         ctx.module = module
         ctx.save_for_backward(x, q, phi, grad, C)
         return E[0]

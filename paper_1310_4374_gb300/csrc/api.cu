@@ -346,6 +346,16 @@ int ensure_scratch(Plan& pl, size_t need, int* fail_allocs = nullptr) {
     return PSUM_OK;
 }
 
+// The scratch for N charges, grown if it must be, laid out in L (once, where the buffer is large enough).
+int take_scratch(psum_plan_s* h, int64_t N, Layout& L, bool backward = false, int64_t T = -1) {
+    Plan& pl = h->pl;
+    const size_t need = layout(pl, N, (char*)pl.scratch.ptr, L, backward, 0, T);
+    if (need <= pl.scratch.bytes) return PSUM_OK;
+    const int rs = ensure_scratch(pl, need, &h->fail_allocs);
+    if (rs == PSUM_OK) layout(pl, N, (char*)pl.scratch.ptr, L, backward, 0, T);
+    return rs;
+}
+
 // Algorithm "get" on the device for the charges (x, q), with the scratch laid out in L;
 // every kernel is queued on `st`.
 int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, double* phi, double* grad,
@@ -544,22 +554,16 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
 
 int eval_device(psum_plan_s* h, int64_t N, const double* x, const double* q, double* phi, double* grad,
                 cudaStream_t st) {
-    Plan& pl = h->pl;
     Layout L;
-    int rs = ensure_scratch(pl, layout(pl, N, nullptr, L), &h->fail_allocs);
-    if (rs != PSUM_OK) return rs;
-    layout(pl, N, (char*)pl.scratch.ptr, L);
-    return queue_forward(h, N, x, q, phi, grad, L, st);
+    const int rs = take_scratch(h, N, L);
+    return rs != PSUM_OK ? rs : queue_forward(h, N, x, q, phi, grad, L, st);
 }
 
 int eval_points_device(psum_plan_s* h, int64_t N, const double* x, const double* q, int64_t T, const double* y,
                        double* phi, double* grad, cudaStream_t st) {
-    Plan& pl = h->pl;
     Layout L;
-    int rs = ensure_scratch(pl, layout(pl, N, nullptr, L, false, 0, T), &h->fail_allocs);
-    if (rs != PSUM_OK) return rs;
-    layout(pl, N, (char*)pl.scratch.ptr, L, false, 0, T);
-    return queue_forward(h, N, x, q, phi, grad, L, st, T, y);
+    const int rs = take_scratch(h, N, L, false, T);
+    return rs != PSUM_OK ? rs : queue_forward(h, N, x, q, phi, grad, L, st, T, y);
 }
 
 // The energy derivatives (the exact adjoint of the discrete method: moments w = sum q R^(x/R0),
@@ -571,9 +575,8 @@ int backward_device(psum_plan_s* h, int64_t N, const double* x, const double* q,
     Plan& pl = h->pl;
     const psum_opts& o = pl.opt;
     Layout L;
-    int rs = ensure_scratch(pl, layout(pl, N, nullptr, L, true), &h->fail_allocs);
+    const int rs = take_scratch(h, N, L, true);
     if (rs != PSUM_OK) return rs;
-    layout(pl, N, (char*)pl.scratch.ptr, L, true);
     const bool fp32 = o.precision != PSUM_FP64;       // float32 packing (FP32C and FF)
     const bool ff = o.precision == PSUM_FF;
     const int M = o.M, P = pl.P;
@@ -953,9 +956,8 @@ int psum_energy(psum_plan_t h, int64_t N, const double* q, const double* phi, do
     if (!h || N < 1 || N > (int64_t)1 << 30 || !q || !phi || !E) return PSUM_ERR_ARG;
     DeviceGuard g(h->pl.device);
     Layout L;
-    int rs = ensure_scratch(h->pl, layout(h->pl, N, nullptr, L), &h->fail_allocs);
+    const int rs = take_scratch(h, N, L);
     if (rs != PSUM_OK) return rs;
-    layout(h->pl, N, (char*)h->pl.scratch.ptr, L);
     TRY(launch_energy(q, phi, N, L.val_part, L.nblk_val, E, (cudaStream_t)stream));
     h->launches += 2;
     return PSUM_OK;
