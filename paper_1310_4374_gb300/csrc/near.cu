@@ -383,35 +383,15 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
             }
         } else if (cls & kUnitNear) {
             // near pairs: t' = t + delta in float-float (hi by rounding, lo = exact remainder +
-            // both lo parts); a pair whose two groups are both far takes the far loop alone
-#pragma unroll 1
-            for (int j = 0; j < n_pairs; ++j) {
+            // both lo parts); target lo parts are read from global memory
+            auto near_offsets = [&](int j, float2 (&nh)[3], float2 (&nl)[3]) {
                 const float* d0 = dptr(2 * j);
                 const float* d1 = dptr(2 * j + 1);
-                if (!(cls & (j ? kUnitNear1 : kUnitNear0))) {
-                    const float2 tx = s_th[0][j][tid], ty = s_th[1][j][tid], tz = s_th[2][j][tid];
-                    const float2 nx[1] = {make_float2(-(tx.x + d0[0]), -(tx.y + d1[0]))};
-                    const float2 ny[1] = {make_float2(-(ty.x + d0[1]), -(ty.y + d1[1]))};
-                    const float2 nz[1] = {make_float2(-(tz.x + d0[2]), -(tz.y + d1[2]))};
-                    float2 aphi[1] = {make_float2(0.f, 0.f)}, agx[1] = {aphi[0]}, agy[1] = {aphi[0]},
-                           agz[1] = {aphi[0]};
-                    pair_loop_far<kGrad, 1>(uhi, nx, ny, nz, aphi, agx, agy, agz, un);
-                    if constexpr (!kGrad) aphi[0] = __fmul2_rn(aphi[0], wpair(j));
-                    two_sum_acc2(s_acc[0][j][0][tid], s_acc[0][j][1][tid], aphi[0]);
-                    if (kGrad) {
-                        two_sum_acc2(s_acc[1 % NQ][j][0][tid], s_acc[1 % NQ][j][1][tid], agx[0]);
-                        two_sum_acc2(s_acc[2 % NQ][j][0][tid], s_acc[2 % NQ][j][1][tid], agy[0]);
-                        two_sum_acc2(s_acc[3 % NQ][j][0][tid], s_acc[3 % NQ][j][1][tid], agz[0]);
-                    }
-                    continue;
-                }
-                // target lo parts are read from global memory: near pairs are rare
                 const int64_t i0 = (cur_tile * kTgt32 + 2 * j) * kGroup + tid;
                 const int64_t i1 = i0 + kGroup;
                 const float4 C0 = a.tgt_lo[2 * i0], D0 = a.tgt_lo[2 * i0 + 1];
                 const float4 C1 = a.tgt_lo[2 * i1], D1 = a.tgt_lo[2 * i1 + 1];
                 const float2 tls[3] = {make_float2(C0.x, C1.x), make_float2(C0.z, C1.z), make_float2(D0.x, D1.x)};
-                float2 nh[3], nl[3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const float2 th = s_th[c][j][tid], tl = tls[c];
@@ -421,10 +401,8 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
                     nh[c] = make_float2(-h0, -h1);
                     nl[c] = make_float2(-(e0 + (tl.x + d0[3 + c])), -(e1 + (tl.y + d1[3 + c])));
                 }
-                float2 aphi = make_float2(0.f, 0.f), aphi_lo = aphi, agx = aphi, agy = aphi, agz = aphi;
-                const float tau2 = Sp->tau2;
-                pair_loop_near<kGrad>(uhi, ulo, nh[0], nh[1], nh[2], nl[0], nl[1], nl[2], aphi, aphi_lo, agx, agy,
-                                      agz, tau2, un);
+            };
+            auto add_near = [&](int j, float2 aphi, float2 aphi_lo, float2 agx, float2 agy, float2 agz) {
                 if constexpr (!kGrad) {
                     aphi = __fmul2_rn(aphi, wpair(j));
                     aphi_lo = __fmul2_rn(aphi_lo, wpair(j));
@@ -435,6 +413,45 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
                     two_sum_acc2(s_acc[1 % NQ][j][0][tid], s_acc[1 % NQ][j][1][tid], agx);
                     two_sum_acc2(s_acc[2 % NQ][j][0][tid], s_acc[2 % NQ][j][1][tid], agy);
                     two_sum_acc2(s_acc[3 % NQ][j][0][tid], s_acc[3 % NQ][j][1][tid], agz);
+                }
+            };
+            const float2 z = make_float2(0.f, 0.f);
+            const float tau2 = Sp->tau2;
+            if ((cls & kUnitNear) == kUnitNear && n_pairs == 2) {
+                float2 nh[2][3], nl[2][3];
+                near_offsets(0, nh[0], nl[0]);
+                near_offsets(1, nh[1], nl[1]);
+                float2 aphi[2] = {z, z}, aphi_lo[2] = {z, z}, agx[2] = {z, z}, agy[2] = {z, z}, agz[2] = {z, z};
+                pair_loop_near<kGrad, 2>(uhi, ulo, nh, nl, aphi, aphi_lo, agx, agy, agz, tau2, un);
+                add_near(0, aphi[0], aphi_lo[0], agx[0], agy[0], agz[0]);
+                add_near(1, aphi[1], aphi_lo[1], agx[1], agy[1], agz[1]);
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < n_pairs; ++j) {
+                    if (cls & (j ? kUnitNear1 : kUnitNear0)) {
+                        float2 nh[1][3], nl[1][3];
+                        near_offsets(j, nh[0], nl[0]);
+                        float2 aphi[1] = {z}, aphi_lo[1] = {z}, agx[1] = {z}, agy[1] = {z}, agz[1] = {z};
+                        pair_loop_near<kGrad, 1>(uhi, ulo, nh, nl, aphi, aphi_lo, agx, agy, agz, tau2, un);
+                        add_near(j, aphi[0], aphi_lo[0], agx[0], agy[0], agz[0]);
+                        continue;
+                    }
+                    // a pair whose two groups are both far takes the far loop alone
+                    const float* d0 = dptr(2 * j);
+                    const float* d1 = dptr(2 * j + 1);
+                    const float2 tx = s_th[0][j][tid], ty = s_th[1][j][tid], tz = s_th[2][j][tid];
+                    const float2 nx[1] = {make_float2(-(tx.x + d0[0]), -(tx.y + d1[0]))};
+                    const float2 ny[1] = {make_float2(-(ty.x + d0[1]), -(ty.y + d1[1]))};
+                    const float2 nz[1] = {make_float2(-(tz.x + d0[2]), -(tz.y + d1[2]))};
+                    float2 aphi[1] = {z}, agx[1] = {z}, agy[1] = {z}, agz[1] = {z};
+                    pair_loop_far<kGrad, 1>(uhi, nx, ny, nz, aphi, agx, agy, agz, un);
+                    if constexpr (!kGrad) aphi[0] = __fmul2_rn(aphi[0], wpair(j));
+                    two_sum_acc2(s_acc[0][j][0][tid], s_acc[0][j][1][tid], aphi[0]);
+                    if (kGrad) {
+                        two_sum_acc2(s_acc[1 % NQ][j][0][tid], s_acc[1 % NQ][j][1][tid], agx[0]);
+                        two_sum_acc2(s_acc[2 % NQ][j][0][tid], s_acc[2 % NQ][j][1][tid], agy[0]);
+                        two_sum_acc2(s_acc[3 % NQ][j][0][tid], s_acc[3 % NQ][j][1][tid], agz[0]);
+                    }
                 }
             }
         } else if (!pair1_live) {

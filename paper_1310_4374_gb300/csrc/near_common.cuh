@@ -218,7 +218,7 @@ __device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 v) {
     hi = s;
 }
 
-// Near units: one packed target pair at a time, offsets from hi + lo coordinates,
+// Near units: offsets from hi + lo coordinates,
 // K(0) = 0 applied.  They hold the closest pairs, whose large terms would dominate the
 // rounding of a plain float32 running sum of the potential: blocks of kNearFold terms are
 // summed in float32 and each block is added with its rounding error carried (two-sum into
@@ -226,14 +226,17 @@ __device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 v) {
 constexpr int kNearFold = 4;
 static_assert(kNearChunk % kNearFold == 0, "whole blocks per chunk");
 
-template <bool kGrad>
+// NP packed target pairs at a time: a unit that is near for both of a thread's pairs runs them
+// together (half the source loads, and two chains of dependent operations to fill each other's
+// latencies: small systems are mostly such units).
+template <bool kGrad, int NP>
 __device__ __forceinline__ void pair_loop_near(const float4* __restrict__ s_hi, const float4* __restrict__ s_lo,
-                                               float2 nhx, float2 nhy, float2 nhz, float2 nlx, float2 nly,
-                                               float2 nlz, float2& aphi, float2& aphi_lo, float2& agx, float2& agy,
-                                               float2& agz, float tau2, int n = kNearChunk) {
+                                               const float2 (&nh)[NP][3], const float2 (&nl)[NP][3],
+                                               float2 (&aphi)[NP], float2 (&aphi_lo)[NP], float2 (&agx)[NP],
+                                               float2 (&agy)[NP], float2 (&agz)[NP], float tau2, int n = kNearChunk) {
 #pragma unroll 1
     for (int s0 = 0; s0 < n; s0 += kNearFold) {
-        float2 blk = make_float2(0.f, 0.f);
+        float2 blk[NP];
 #pragma unroll
         for (int k = 0; k < kNearFold; ++k) {
             const int s = s0 + k;
@@ -241,25 +244,29 @@ __device__ __forceinline__ void pair_loop_near(const float4* __restrict__ s_hi, 
             const float4 B = s_hi[2 * s + 1];
             const float4 C = s_lo[2 * s];
             const float4 D = s_lo[2 * s + 1];
-            const float2 ex = __fadd2_rn(__fadd2_rn(make_float2(A.x, A.y), nhx), __fadd2_rn(make_float2(C.x, C.y), nlx));
-            const float2 ey = __fadd2_rn(__fadd2_rn(make_float2(A.z, A.w), nhy), __fadd2_rn(make_float2(C.z, C.w), nly));
-            const float2 ez = __fadd2_rn(__fadd2_rn(make_float2(B.x, B.y), nhz), __fadd2_rn(make_float2(D.x, D.y), nlz));
-            float2 r2 = __fmul2_rn(ex, ex);
-            r2 = __ffma2_rn(ey, ey, r2);
-            r2 = __ffma2_rn(ez, ez, r2);
-            float2 ri = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-            ri.x = r2.x > tau2 ? ri.x : 0.f;                  // K(0) = 0 (Eq. 1), coincident_r2 (psum_internal.cuh)
-            ri.y = r2.y > tau2 ? ri.y : 0.f;
-            const float2 qr = __fmul2_rn(make_float2(B.z, B.w), ri);
-            blk = k == 0 ? qr : __fadd2_rn(blk, qr);
-            if (kGrad) {
-                const float2 w = __fmul2_rn(qr, __fmul2_rn(ri, ri));
-                agx = __ffma2_rn(ex, w, agx);
-                agy = __ffma2_rn(ey, w, agy);
-                agz = __ffma2_rn(ez, w, agz);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                const float2 ex = __fadd2_rn(__fadd2_rn(make_float2(A.x, A.y), nh[j][0]), __fadd2_rn(make_float2(C.x, C.y), nl[j][0]));
+                const float2 ey = __fadd2_rn(__fadd2_rn(make_float2(A.z, A.w), nh[j][1]), __fadd2_rn(make_float2(C.z, C.w), nl[j][1]));
+                const float2 ez = __fadd2_rn(__fadd2_rn(make_float2(B.x, B.y), nh[j][2]), __fadd2_rn(make_float2(D.x, D.y), nl[j][2]));
+                float2 r2 = __fmul2_rn(ex, ex);
+                r2 = __ffma2_rn(ey, ey, r2);
+                r2 = __ffma2_rn(ez, ez, r2);
+                float2 ri = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
+                ri.x = r2.x > tau2 ? ri.x : 0.f;              // K(0) = 0 (Eq. 1), coincident_r2 (psum_internal.cuh)
+                ri.y = r2.y > tau2 ? ri.y : 0.f;
+                const float2 qr = __fmul2_rn(make_float2(B.z, B.w), ri);
+                blk[j] = k == 0 ? qr : __fadd2_rn(blk[j], qr);
+                if (kGrad) {
+                    const float2 w = __fmul2_rn(qr, __fmul2_rn(ri, ri));
+                    agx[j] = __ffma2_rn(ex, w, agx[j]);
+                    agy[j] = __ffma2_rn(ey, w, agy[j]);
+                    agz[j] = __ffma2_rn(ez, w, agz[j]);
+                }
             }
         }
-        two_sum_acc2(aphi, aphi_lo, blk);
+#pragma unroll
+        for (int j = 0; j < NP; ++j) two_sum_acc2(aphi[j], aphi_lo[j], blk[j]);
     }
 }
 

@@ -534,24 +534,23 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) 
                     const float4 C1 = a.pk_lo[2 * i1], D1 = a.pk_lo[2 * i1 + 1];
                     const float2 tls[3] = {make_float2(C0.x, C1.x), make_float2(C0.z, C1.z), make_float2(D0.x, D1.x)};
                     const float2 ths[3] = {tx, ty, tz};
-                    float2 nh[3], nl[3];
+                    float2 nh[1][3], nl[1][3];
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         float e0, e1;
                         const float h0 = two_sum(ths[c].x, d0[c], e0);
                         const float h1 = two_sum(ths[c].y, d1[c], e1);
-                        nh[c] = make_float2(-h0, -h1);
-                        nl[c] = make_float2(-(e0 + (tls[c].x + d0[3 + c])), -(e1 + (tls[c].y + d1[3 + c])));
+                        nh[0][c] = make_float2(-h0, -h1);
+                        nl[0][c] = make_float2(-(e0 + (tls[c].x + d0[3 + c])), -(e1 + (tls[c].y + d1[3 + c])));
                     }
-                    float2 aphi = make_float2(0.f, 0.f), aphi_lo = aphi, agx = aphi, agy = aphi, agz = aphi;
-                    const float tau2 = S.tau2;
-                    pair_loop_near<true>(s_hi, s_lo, nh[0], nh[1], nh[2], nl[0], nl[1], nl[2], aphi, aphi_lo, agx,
-                                         agy, agz, tau2);
-                    two_sum_acc2(s_acc[0][j][0][tid], s_acc[0][j][1][tid], aphi);
-                    s_acc[0][j][1][tid] = __fadd2_rn(s_acc[0][j][1][tid], aphi_lo);
-                    two_sum_acc2(s_acc[1][j][0][tid], s_acc[1][j][1][tid], agx);
-                    two_sum_acc2(s_acc[2][j][0][tid], s_acc[2][j][1][tid], agy);
-                    two_sum_acc2(s_acc[3][j][0][tid], s_acc[3][j][1][tid], agz);
+                    const float2 z = make_float2(0.f, 0.f);
+                    float2 aphi[1] = {z}, aphi_lo[1] = {z}, agx[1] = {z}, agy[1] = {z}, agz[1] = {z};
+                    pair_loop_near<true, 1>(s_hi, s_lo, nh, nl, aphi, aphi_lo, agx, agy, agz, S.tau2);
+                    two_sum_acc2(s_acc[0][j][0][tid], s_acc[0][j][1][tid], aphi[0]);
+                    s_acc[0][j][1][tid] = __fadd2_rn(s_acc[0][j][1][tid], aphi_lo[0]);
+                    two_sum_acc2(s_acc[1][j][0][tid], s_acc[1][j][1][tid], agx[0]);
+                    two_sum_acc2(s_acc[2][j][0][tid], s_acc[2][j][1][tid], agy[0]);
+                    two_sum_acc2(s_acc[3][j][0][tid], s_acc[3][j][1][tid], agz[0]);
                 }
                 continue;
             }
