@@ -219,10 +219,12 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
         int64_t gmax = (int64_t)pl.num_sms * near64_occupancy_ctas();
         if (g_cap > 0 && gmax > g_cap) gmax = g_cap;
         L.Ln = near_partition(L.n_tiles, L.n_chunks, n_img, gmax, ipc);
+        L.Ln.tab.one.fix = fixed_scale(pl.opt.d, pl.opt.K);
         const bool layers = pl.lc_tiles > 0;
         const int64_t c_tiles = layers ? pl.lc_tiles : pl.n_check_tiles;
         L.Lc = near_partition(c_tiles, L.n_chunks, layers ? pl.lc_img : n_img, gmax,
                               g_cap > 0 ? 1 : kCheckItemsPerCta);
+        L.Lc.tab.one.fix = fixed_scale(pl.opt.d, pl.opt.K);
         // the symmetric float64 kernel: charges, block image set, a normal (growing) scratch
         L.sym = false;
         const int pk = pl.opt.pair_kernel;
@@ -235,6 +237,7 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
             one[0].last_n = (int)(N - (L.n_chunks - 1) * kTile64);
             one[0].shift0 = 0;
             one[0].n_img = n_img;
+            one[0].fix = fixed_scale(pl.opt.d, pl.opt.K);
             L.S = sym_partition(one, (int64_t)pl.num_sms * near64s_occupancy_ctas(), kTile64);
             sym_bands(L, kTile64, pl.sym_band_bytes);
             L.sym = true;
@@ -285,6 +288,7 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
                                    : near64_occupancy_ctas());
         L.Lb = near_partition(L.n_tiles, n_chk_chunks, n_img, gmax);
         L.Lb.tab.one.tau2 = coincident_r2(pl.opt.d);
+        L.Lb.tab.one.fix = fixed_scale(pl.opt.d, pl.opt.K);
         L.Lb.counter = flags + 3;
         L.Lb.status = flags;
         L.Lb.n_status = 1;

@@ -503,7 +503,8 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
 }
 
 // ---------------------------------------------------------------------------
-// FP64 kernel
+// FP64 kernel: the pair's geometry in integers (fixed64.cuh), leaving one float64 operation per pair for
+// the potential and five with the field to the float64 pipe, which ran 10 and 13.
 // ---------------------------------------------------------------------------
 struct Near64Args {
     const double4_32a* src;      // (x, y, z, q), absolute
@@ -527,12 +528,12 @@ struct Near64Args {
 template <bool kGrad>
 __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
     __shared__ double4_32a s_src[kNearChunk];
-    __shared__ double4_32a s_srcm[kNearChunk];        // the chunk with the image's masked charges
+    __shared__ FixedPoint s_fix[kNearChunk];
     constexpr int NQ = kGrad ? 4 : 1;
     __shared__ int s_item;
     const int tid = threadIdx.x;
     int64_t item = 0;
-    double tx = 0, ty = 0, tz = 0;
+    FixedPoint tf = {0, 0, 0, 0.0};
     int tcls = 0;                        // the target's class (two-layer check sums)
     bool live = true;                    // false: a warp of padding (check points)
     double acc[NQ];
@@ -568,7 +569,7 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
         if (tile != cur_tile) {
             if (cur_tile >= 0) flush(cur_tile, cur_first);
             const double4_32a t = a.tgt[tile * kTile64 + tid];
-            tx = t.x; ty = t.y; tz = t.z;
+            tf = fixed_point(t, S.fix);
             // a class outside 0..n_cls-1 reads class 0: the index stays inside the tables
             tcls = (!kGrad && a.n_cls > 1 && t.w >= 0.0 && t.w < (double)a.n_cls) ? (int)t.w : 0;
             // check points are distinct, so a warp of targets at the padding's place holds padding alone:
@@ -582,7 +583,11 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
         }
         if (chunk != cur_chunk) {
             __syncthreads();
-            for (int i = tid; i < kNearChunk; i += kThreads64) s_src[i] = a.src[chunk * kNearChunk + i];
+            for (int i = tid; i < kNearChunk; i += kThreads64) {
+                const double4_32a src = a.src[chunk * kNearChunk + i];
+                s_src[i] = src;
+                s_fix[i] = fixed_point(src, S.fix);
+            }
             __syncthreads();
             cur_chunk = chunk;
         }
@@ -598,32 +603,35 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
                 continue;
             }
         }
-        const double px = tx - sh[0], py = ty - sh[1], pz = tz - sh[2];
-        const double4_32a* src = s_src;
+        const long long fx = fixed_minus(tf.x, to_fixed(sh[0], S.fix)), fy = fixed_minus(tf.y, to_fixed(sh[1], S.fix)),
+                        fz = fixed_minus(tf.z, to_fixed(sh[2], S.fix));
         if (a.Rb > 0.0) {
             __syncthreads();
             const double4_32a Q = s_src[tid];
-            s_srcm[tid] = make_double4_32a(Q.x, Q.y, Q.z, in_ball(Q.x, Q.y, Q.z, sh, a.Rb) ? Q.w : 0.0);
+            s_fix[tid].q = in_ball(Q.x, Q.y, Q.z, sh, a.Rb) ? Q.w : 0.0;
             __syncthreads();
-            src = s_srcm;
         }
         // the weight (1, -1 or 0) goes onto the charge's bits: no float64 operation
         const int w_and = w != 0.0 ? -1 : 0, w_xor = w < 0.0 ? (int)0x80000000 : 0;
         const int n_src = live ? kNearChunk : 0;
 #pragma unroll 2
         for (int s = 0; s < n_src; ++s) {
-            const double4_32a Q = src[s];
-            const double ex = Q.x - px, ey = Q.y - py, ez = Q.z - pz;   // x_i + p - y
-            const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
+            const FixedPoint Q = s_fix[s];
+            FixedPair v;                                          // x_i + p - y
+            const bool near = !fixed_pair<kGrad>(Q, fx, fy, fz, S.fix, v);
+            if (__any_sync(0xffffffffu, near)) {
+                __syncwarp();
+                if (near) float64_pair<kGrad>(s_src[s], a.tgt[tile * kTile64 + tid], sh, v);
+            }
             if (kGrad) {
-                const double g = Q.w * rsqrt3_f64_k0(r2);     // K(0) = 0
-                acc[0] = fma(g, r2, acc[0]);
-                acc[1 % NQ] = fma(ex, g, acc[1 % NQ]);
-                acc[2 % NQ] = fma(ey, g, acc[2 % NQ]);
-                acc[3 % NQ] = fma(ez, g, acc[3 % NQ]);
+                const double g = Q.q * v.ri3;
+                acc[0] = fma(Q.q, v.ri, acc[0]);
+                acc[1 % NQ] = fma(v.ex, g, acc[1 % NQ]);
+                acc[2 % NQ] = fma(v.ey, g, acc[2 % NQ]);
+                acc[3 % NQ] = fma(v.ez, g, acc[3 % NQ]);
             } else {
-                const double qw = __hiloint2double((__double2hiint(Q.w) & w_and) ^ w_xor, __double2loint(Q.w) & w_and);
-                acc[0] = fma(qw, rsqrt_f64_k0(r2), acc[0]);
+                const double qw = __hiloint2double((__double2hiint(Q.q) & w_and) ^ w_xor, __double2loint(Q.q) & w_and);
+                acc[0] = fma(qw, v.ri, acc[0]);
             }
         }
         ++u;

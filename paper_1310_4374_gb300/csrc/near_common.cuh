@@ -4,7 +4,6 @@
 #pragma once
 
 #include "launch.cuh"
-#include "rsqrt64.cuh"
 
 namespace psum {
 
@@ -408,6 +407,60 @@ __device__ __forceinline__ double rsqrt3_f64_k0(double r2) {
     const float r2f = estimate_arg(r2);
     const double ri3 = rsqrt3_refined(r2, __float_as_uint(rsqrt_mufu(r2f)));
     return r2f > 0.f ? ri3 : 0.0;
+}
+
+// A packed point in integer coordinates (fixed64.cuh).  The packs' padding (1e3, 1e3, 1e3), no charge, is
+// put at the origin: outside the range it would send every pair of its warp through the float64 form.
+struct __align__(32) FixedPoint {
+    long long x, y, z;
+    double q;
+};
+__device__ __forceinline__ FixedPoint fixed_point(const double4_32a& v, int k) {
+    const bool pad = v.x == 1.0e3 && v.y == 1.0e3 && v.z == 1.0e3;
+    FixedPoint f;
+    f.x = pad ? 0 : to_fixed(v.x, k);
+    f.y = pad ? 0 : to_fixed(v.y, k);
+    f.z = pad ? 0 : to_fixed(v.z, k);
+    f.q = v.w;
+    return f;
+}
+__device__ __forceinline__ long long fixed_minus(long long a, long long b) {
+    return (long long)((uint64_t)a - (uint64_t)b);
+}
+
+// The geometry of one pair for the float64 sums: 1/r, and with kField 1/r^3 and the difference s - t.  false:
+// the pair is left to the float64 form (near, coincident or outside the range).
+struct FixedPair {
+    double ri, ri3, ex, ey, ez;
+};
+template <bool kField>
+__device__ __forceinline__ bool fixed_pair(const FixedPoint& s, long long tx, long long ty, long long tz, int k,
+                                           FixedPair& o) {
+    const FixedDelta dx = fixed_delta(s.x, tx), dy = fixed_delta(s.y, ty), dz = fixed_delta(s.z, tz);
+    const uint32_t high = (uint32_t)((dx.a | dy.a | dz.a) >> 32);
+    if (high - kFixedNear >= kFixedFar - kFixedNear) return false;
+    const FixedR2 r = fixed_r2(dx, dy, dz, high);
+    const FixedInverse v = fixed_inverse(r, k, __float_as_uint(rsqrt_mufu(fixed_estimate_arg(r.R))));
+    o.ri = fixed_ri(v);
+    if (kField) {
+        o.ri3 = fixed_ri3(v);
+        o.ex = fixed_value(dx, k);
+        o.ey = fixed_value(dy, k);
+        o.ez = fixed_value(dz, k);
+    }
+    return true;
+}
+
+// ... in float64.  Callers branch to it by a warp vote and a warp barrier, lest it be compiled into
+// predicated instructions, which would take the float64 pipe on or off.
+template <bool kField>
+__device__ __forceinline__ void float64_pair(const double4_32a& s, const double4_32a& t, const double* sh, FixedPair& o) {
+    o.ex = s.x - (t.x - sh[0]);
+    o.ey = s.y - (t.y - sh[1]);
+    o.ez = s.z - (t.z - sh[2]);
+    const double r2 = fma(o.ez, o.ez, fma(o.ey, o.ey, o.ex * o.ex));
+    if (kField) o.ri3 = rsqrt3_f64_k0(r2);
+    o.ri = kField ? o.ri3 * r2 : rsqrt_f64_k0(r2);               // K(0) = 0
 }
 
 // warps of the reduction kernels (fixed-order combination of the partial slots)

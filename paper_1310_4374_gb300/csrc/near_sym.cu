@@ -856,6 +856,12 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) 
 // per step (float64 shuffles); every warp keeps its own float64 reaction sums per source,
 // added in a fixed order when the item is done.  A tile against itself takes one image of
 // each mirror pair with reactions onto its own charges, and the zero image one-sided.
+//
+// Bound by the float64 pipe (93% busy): 10 float64 operations per mirror pair, two products and eight
+// multiply-adds, the pair's geometry being integer work beside them (fixed64.cuh), 38% of the issue slots.
+// With the differences, the squared distance and the last steps of 1/r^3 in float64 (18 operations) 12 001
+// charges took 64.0 ms where they take 34.7, a 16^3 lattice 7.98 where it takes 4.35, 1000 charges 0.69
+// where they take 0.41.
 // ---------------------------------------------------------------------------
 struct Near64SymArgs {
     const double4_32a* pk;   // charges (x, y, z, q), absolute, padded with far-away zero charges
@@ -873,6 +879,7 @@ template <int kMinB>
 __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) {
     constexpr int kWarps = kThreads64 / 32;
     __shared__ double4_32a s_src[kNearChunk];
+    __shared__ FixedPoint s_fix[kNearChunk];
     __shared__ double s_re[kWarps][4][kNearChunk];   // reaction sums [warp][quantity][source]
     __shared__ int s_item;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -893,7 +900,10 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
     const int im0 = gi * S.img_per_g;
     const int nimg = min(S.img_per_g, S.n_img - im0);
     const double4_32a t = a.pk[(S.tile0 + ta) * kTile64 + tid];
-    s_src[tid] = a.pk[(S.tile0 + tb) * kTile64 + tid];
+    const double4_32a src = a.pk[(S.tile0 + tb) * kTile64 + tid];
+    s_src[tid] = src;
+    s_fix[tid] = fixed_point(src, S.fix);
+    const FixedPoint tf = fixed_point(t, S.fix);
 #pragma unroll
     for (int qi = 0; qi < 4; ++qi)
 #pragma unroll
@@ -907,8 +917,8 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
         const double* sh = a.shifts + 3 * (S.shift0 + im0 + im);
         const int sg = diag ? shift_sign(sh) : 1;
         if (sg < 0) continue;                    // a tile against itself: image -p by reaction
-        const double px = t.x - sh[0], py = t.y - sh[1], pz = t.z - sh[2];
         if (sg == 0) {                           // ... and its zero image one-sided
+            const double px = t.x - sh[0], py = t.y - sh[1], pz = t.z - sh[2];
 #pragma unroll 4
             for (int s = 0; s < kNearChunk; ++s) {
                 const double4_32a Q = s_src[s];
@@ -922,25 +932,31 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
             }
             continue;
         }
+        const long long fx = fixed_minus(tf.x, to_fixed(sh[0], S.fix)), fy = fixed_minus(tf.y, to_fixed(sh[1], S.fix)),
+                        fz = fixed_minus(tf.z, to_fixed(sh[2], S.fix));
 #pragma unroll 1
         for (int g = 0; g < nb32; ++g) {
             double rp = 0.0, rx = 0.0, ry = 0.0, rz = 0.0;
 #pragma unroll 2
             for (int k = 0; k < 32; ++k) {
-                const double4_32a Q = s_src[32 * g + ((lane + k) & 31)];
-                const double ex = Q.x - px, ey = Q.y - py, ez = Q.z - pz;   // x_s + p - y
-                const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
-                const double ri3 = rsqrt3_f64_k0(r2);
-                const double wa = Q.w * ri3;             // action
-                acc[0] = fma(wa, r2, acc[0]);
-                acc[1] = fma(ex, wa, acc[1]);
-                acc[2] = fma(ey, wa, acc[2]);
-                acc[3] = fma(ez, wa, acc[3]);
-                const double wb = t.w * ri3;             // reaction (field sign folded later)
-                rp = fma(wb, r2, rp);
-                rx = fma(ex, wb, rx);
-                ry = fma(ey, wb, ry);
-                rz = fma(ez, wb, rz);
+                const int s = 32 * g + ((lane + k) & 31);
+                const FixedPoint Q = s_fix[s];
+                FixedPair v;                             // x_s + p - y
+                const bool near = !fixed_pair<true>(Q, fx, fy, fz, S.fix, v);
+                if (__any_sync(0xffffffffu, near)) {
+                    __syncwarp();
+                    if (near) float64_pair<true>(s_src[s], a.pk[(S.tile0 + ta) * kTile64 + tid], sh, v);
+                }
+                const double wa = Q.q * v.ri3;           // action
+                acc[0] = fma(Q.q, v.ri, acc[0]);
+                acc[1] = fma(v.ex, wa, acc[1]);
+                acc[2] = fma(v.ey, wa, acc[2]);
+                acc[3] = fma(v.ez, wa, acc[3]);
+                const double wb = t.w * v.ri3;           // reaction (field sign folded later)
+                rp = fma(t.w, v.ri, rp);
+                rx = fma(v.ex, wb, rx);
+                ry = fma(v.ey, wb, ry);
+                rz = fma(v.ez, wb, rz);
                 rp = __shfl_sync(0xffffffffu, rp, up);
                 rx = __shfl_sync(0xffffffffu, rx, up);
                 ry = __shfl_sync(0xffffffffu, ry, up);

@@ -9,6 +9,7 @@
 #include <cmath>
 #include <vector>
 
+#include "fixed64.cuh"
 #include "psum.h"
 
 namespace psum {
@@ -396,6 +397,18 @@ inline float coincident_r2(const double d[3]) {
     return (float)(t * t);
 }
 
+// The exponent k of the float64 pair kernels' integer coordinates (fixed64.cuh): 2^(62-k) above every
+// coordinate difference y - x - p, y in the box or on the sphere around it (half diagonal R0), x in the
+// box, p an image of the block or of the layer next to it.  Outside 2^+-60 every pair is float64 throughout.
+inline int fixed_scale(const double d[3], const int K[3]) {
+    double m = 0.0;
+    for (int i = 0; i < 3; ++i) m = std::fmax(m, (K[i] + 2.0) * d[i]);
+    m += 0.5 * std::sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    int e;
+    std::frexp(m * (1.0 + 1e-6), &e);
+    return e >= -60 && e <= 60 ? 62 - e : kNoFixed;
+}
+
 struct NearSys {
     int64_t unit0;       // first unit
     int64_t tile0;       // first tile of the system in the target pack (= its first partial-buffer row)
@@ -406,6 +419,7 @@ struct NearSys {
     int n_img;
     int64_t chunk_stride;  // a tile visits its chunks in the order (k * chunk_stride) mod n_chunks
     float tau2;          // coincident_r2 of the system's box (float32 kernels)
+    int fix;             // fixed_scale of the system's box (float64 kernels)
 };
 
 // A stride near n / golden ratio, coprime to n: consecutive steps land far apart in the
@@ -524,6 +538,7 @@ struct SymSys {
     int n_g, img_per_g;       // image groups per tile pair and images per group
     int last_n;               // charges in the system's last chunk (1..kNearChunk; 0 = a full chunk)
     float tau2;               // coincident_r2 of the system's box (float32 kernels)
+    int fix;                  // fixed_scale of the system's box (float64 kernels)
 };
 struct SymSysTable {
     SymSys one;
