@@ -503,8 +503,8 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
 }
 
 // ---------------------------------------------------------------------------
-// FP64 kernel: the pair's geometry in integers (fixed64.cuh), leaving one float64 operation per pair for
-// the potential and five with the field to the float64 pipe, which ran 10 and 13.
+// FP64 kernel: the pair's geometry and weight in integers (fixed64.cuh), leaving one float64 operation per
+// pair for the potential and four with the field to the float64 pipe, which ran 10 and 13.
 // ---------------------------------------------------------------------------
 struct Near64Args {
     const double4_32a* src;      // (x, y, z, q), absolute
@@ -528,12 +528,12 @@ struct Near64Args {
 template <bool kGrad>
 __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
     __shared__ double4_32a s_src[kNearChunk];
-    __shared__ FixedPoint s_fix[kNearChunk];
+    __shared__ FixedSource s_fix[kNearChunk];
     constexpr int NQ = kGrad ? 4 : 1;
     __shared__ int s_item;
     const int tid = threadIdx.x;
     int64_t item = 0;
-    FixedPoint tf = {0, 0, 0, 0.0};
+    FixedSpot tf = {0, 0, 0};
     int tcls = 0;                        // the target's class (two-layer check sums)
     bool live = true;                    // false: a warp of padding (check points)
     double acc[NQ];
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
         if (tile != cur_tile) {
             if (cur_tile >= 0) flush(cur_tile, cur_first);
             const double4_32a t = a.tgt[tile * kTile64 + tid];
-            tf = fixed_point(t, S.fix);
+            tf = fixed_spot(t, S.fix);
             // a class outside 0..n_cls-1 reads class 0: the index stays inside the tables
             tcls = (!kGrad && a.n_cls > 1 && t.w >= 0.0 && t.w < (double)a.n_cls) ? (int)t.w : 0;
             // check points are distinct, so a warp of targets at the padding's place holds padding alone:
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
             for (int i = tid; i < kNearChunk; i += kThreads64) {
                 const double4_32a src = a.src[chunk * kNearChunk + i];
                 s_src[i] = src;
-                s_fix[i] = fixed_point(src, S.fix);
+                s_fix[i] = fixed_source(src, S.fix);
             }
             __syncthreads();
             cur_chunk = chunk;
@@ -603,12 +603,12 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
                 continue;
             }
         }
-        const long long fx = fixed_minus(tf.x, to_fixed(sh[0], S.fix)), fy = fixed_minus(tf.y, to_fixed(sh[1], S.fix)),
-                        fz = fixed_minus(tf.z, to_fixed(sh[2], S.fix));
+        const FixedSpot f = fixed_minus(tf, sh, S.fix);
         if (a.Rb > 0.0) {
             __syncthreads();
             const double4_32a Q = s_src[tid];
             s_fix[tid].q = in_ball(Q.x, Q.y, Q.z, sh, a.Rb) ? Q.w : 0.0;
+            fixed_charge(s_fix[tid].q, s_fix[tid].c);
             __syncthreads();
         }
         // the weight (1, -1 or 0) goes onto the charge's bits: no float64 operation
@@ -616,19 +616,18 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
         const int n_src = live ? kNearChunk : 0;
 #pragma unroll 2
         for (int s = 0; s < n_src; ++s) {
-            const FixedPoint Q = s_fix[s];
+            const FixedSource Q = s_fix[s];
             FixedPair v;                                          // x_i + p - y
-            const bool near = !fixed_pair<kGrad>(Q, fx, fy, fz, S.fix, v);
+            const bool near = !fixed_pair<kGrad, false>(Q, f, Q.c, 0.0, S.fix, v);
             if (__any_sync(0xffffffffu, near)) {
                 __syncwarp();
-                if (near) float64_pair<kGrad>(s_src[s], a.tgt[tile * kTile64 + tid], sh, v);
+                if (near) float64_pair<kGrad, false>(s_src[s], a.tgt[tile * kTile64 + tid], sh, Q.q, v);
             }
             if (kGrad) {
-                const double g = Q.q * v.ri3;
                 acc[0] = fma(Q.q, v.ri, acc[0]);
-                acc[1 % NQ] = fma(v.ex, g, acc[1 % NQ]);
-                acc[2 % NQ] = fma(v.ey, g, acc[2 % NQ]);
-                acc[3 % NQ] = fma(v.ez, g, acc[3 % NQ]);
+                acc[1 % NQ] = fma(v.ex, v.wa, acc[1 % NQ]);
+                acc[2 % NQ] = fma(v.ey, v.wa, acc[2 % NQ]);
+                acc[3 % NQ] = fma(v.ez, v.wa, acc[3 % NQ]);
             } else {
                 const double qw = __hiloint2double((__double2hiint(Q.q) & w_and) ^ w_xor, __double2loint(Q.q) & w_and);
                 acc[0] = fma(qw, v.ri, acc[0]);

@@ -410,57 +410,82 @@ __device__ __forceinline__ double rsqrt3_f64_k0(double r2) {
 }
 
 // A packed point in integer coordinates (fixed64.cuh).  The packs' padding (1e3, 1e3, 1e3), no charge, is
-// put at the origin: outside the range it would send every pair of its warp through the float64 form.
-struct __align__(32) FixedPoint {
+// put at the origin: outside the range it would send every pair of its warp through the float64 form, as
+// kFixedOut does on purpose for a charge without integer form (x of a source, y of a target: both at once are
+// out of range too).
+struct FixedSpot {
     long long x, y, z;
-    double q;
 };
-__device__ __forceinline__ FixedPoint fixed_point(const double4_32a& v, int k) {
+__device__ __forceinline__ FixedSpot fixed_spot(const double4_32a& v, int k) {
     const bool pad = v.x == 1.0e3 && v.y == 1.0e3 && v.z == 1.0e3;
-    FixedPoint f;
+    FixedSpot f;
     f.x = pad ? 0 : to_fixed(v.x, k);
     f.y = pad ? 0 : to_fixed(v.y, k);
     f.z = pad ? 0 : to_fixed(v.z, k);
-    f.q = v.w;
     return f;
 }
-__device__ __forceinline__ long long fixed_minus(long long a, long long b) {
-    return (long long)((uint64_t)a - (uint64_t)b);
+__device__ __forceinline__ FixedSpot fixed_minus(const FixedSpot& a, const double* sh, int k) {
+    FixedSpot f;
+    f.x = (long long)((uint64_t)a.x - (uint64_t)to_fixed(sh[0], k));
+    f.y = (long long)((uint64_t)a.y - (uint64_t)to_fixed(sh[1], k));
+    f.z = (long long)((uint64_t)a.z - (uint64_t)to_fixed(sh[2], k));
+    return f;
+}
+struct __align__(16) FixedSource {
+    FixedSpot at;
+    double q;
+    FixedCharge c;
+};
+__device__ __forceinline__ FixedSource fixed_source(const double4_32a& v, int k) {
+    FixedSource f;
+    f.at = fixed_spot(v, k);
+    f.q = v.w;
+    if (!fixed_charge(v.w, f.c)) f.at.x = kFixedOut;
+    return f;
 }
 
-// The geometry of one pair for the float64 sums: 1/r, and with kField 1/r^3 and the difference s - t.  false:
-// the pair is left to the float64 form (near, coincident or outside the range).
+// One pair for the float64 sums: 1/r, and with kField the difference s - t, the action q_s / r^3 and with
+// kMirror the reaction q_t / r^3.  false: the pair is left to the float64 form (near, coincident, or outside
+// the range).
 struct FixedPair {
-    double ri, ri3, ex, ey, ez;
+    double ri, ex, ey, ez, wa, wb;
 };
-template <bool kField>
-__device__ __forceinline__ bool fixed_pair(const FixedPoint& s, long long tx, long long ty, long long tz, int k,
+template <bool kField, bool kMirror>
+__device__ __forceinline__ bool fixed_pair(const FixedSource& s, const FixedSpot& t, FixedCharge tc, double tq, int k,
                                            FixedPair& o) {
-    const FixedDelta dx = fixed_delta(s.x, tx), dy = fixed_delta(s.y, ty), dz = fixed_delta(s.z, tz);
+    const FixedDelta dx = fixed_delta(s.at.x, t.x), dy = fixed_delta(s.at.y, t.y), dz = fixed_delta(s.at.z, t.z);
     const uint32_t high = (uint32_t)((dx.a | dy.a | dz.a) >> 32);
     if (high - kFixedNear >= kFixedFar - kFixedNear) return false;
     const FixedR2 r = fixed_r2(dx, dy, dz, high);
     const FixedInverse v = fixed_inverse(r, k, __float_as_uint(rsqrt_mufu(fixed_estimate_arg(r.R))));
     o.ri = fixed_ri(v);
     if (kField) {
-        o.ri3 = fixed_ri3(v);
+        const uint64_t M3 = fixed_cube(v);
+        o.wa = fixed_weight(M3, 3 * v.x, s.c, s.q);
+        if (kMirror) o.wb = fixed_weight(M3, 3 * v.x, tc, tq);
         o.ex = fixed_value(dx, k);
         o.ey = fixed_value(dy, k);
         o.ez = fixed_value(dz, k);
     }
     return true;
 }
-
 // ... in float64.  Callers branch to it by a warp vote and a warp barrier, lest it be compiled into
 // predicated instructions, which would take the float64 pipe on or off.
-template <bool kField>
-__device__ __forceinline__ void float64_pair(const double4_32a& s, const double4_32a& t, const double* sh, FixedPair& o) {
+template <bool kField, bool kMirror>
+__device__ __forceinline__ void float64_pair(const double4_32a& s, const double4_32a& t, const double* sh, double q,
+                                             FixedPair& o) {
     o.ex = s.x - (t.x - sh[0]);
     o.ey = s.y - (t.y - sh[1]);
     o.ez = s.z - (t.z - sh[2]);
     const double r2 = fma(o.ez, o.ez, fma(o.ey, o.ey, o.ex * o.ex));
-    if (kField) o.ri3 = rsqrt3_f64_k0(r2);
-    o.ri = kField ? o.ri3 * r2 : rsqrt_f64_k0(r2);               // K(0) = 0
+    if (kField) {
+        const double ri3 = rsqrt3_f64_k0(r2);                    // K(0) = 0
+        o.ri = ri3 * r2;
+        o.wa = q * ri3;
+        if (kMirror) o.wb = t.w * ri3;
+    } else {
+        o.ri = rsqrt_f64_k0(r2);
+    }
 }
 
 // warps of the reduction kernels (fixed-order combination of the partial slots)

@@ -857,11 +857,11 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) 
 // added in a fixed order when the item is done.  A tile against itself takes one image of
 // each mirror pair with reactions onto its own charges, and the zero image one-sided.
 //
-// Bound by the float64 pipe (93% busy): 10 float64 operations per mirror pair, two products and eight
-// multiply-adds, the pair's geometry being integer work beside them (fixed64.cuh), 38% of the issue slots.
-// With the differences, the squared distance and the last steps of 1/r^3 in float64 (18 operations) 12 001
-// charges took 64.0 ms where they take 34.7, a 16^3 lattice 7.98 where it takes 4.35, 1000 charges 0.69
-// where they take 0.41.
+// Bound by the float64 pipe: 8 float64 operations per mirror pair, the multiply-adds of its eight sums; the
+// pair's geometry and its weights q/r^3 are integer work beside them (fixed64.cuh).  12 001 charges take
+// 28.1 ms; 34.7 with the two weights as float64 products, 64.0 with the differences, the squared distance and
+// the last steps of 1/r^3 in float64 too (18 operations).  A 16^3 lattice 3.61, 4.35, 7.98 ms; 1000 charges
+// 0.345, 0.411, 0.685 ms.
 // ---------------------------------------------------------------------------
 struct Near64SymArgs {
     const double4_32a* pk;   // charges (x, y, z, q), absolute, padded with far-away zero charges
@@ -879,7 +879,7 @@ template <int kMinB>
 __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) {
     constexpr int kWarps = kThreads64 / 32;
     __shared__ double4_32a s_src[kNearChunk];
-    __shared__ FixedPoint s_fix[kNearChunk];
+    __shared__ FixedSource s_fix[kNearChunk];
     __shared__ double s_re[kWarps][4][kNearChunk];   // reaction sums [warp][quantity][source]
     __shared__ int s_item;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -902,8 +902,10 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
     const double4_32a t = a.pk[(S.tile0 + ta) * kTile64 + tid];
     const double4_32a src = a.pk[(S.tile0 + tb) * kTile64 + tid];
     s_src[tid] = src;
-    s_fix[tid] = fixed_point(src, S.fix);
-    const FixedPoint tf = fixed_point(t, S.fix);
+    s_fix[tid] = fixed_source(src, S.fix);
+    FixedSpot tf = fixed_spot(t, S.fix);
+    FixedCharge tc;
+    if (!fixed_charge(t.w, tc)) tf.y = kFixedOut;
 #pragma unroll
     for (int qi = 0; qi < 4; ++qi)
 #pragma unroll
@@ -932,31 +934,28 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
             }
             continue;
         }
-        const long long fx = fixed_minus(tf.x, to_fixed(sh[0], S.fix)), fy = fixed_minus(tf.y, to_fixed(sh[1], S.fix)),
-                        fz = fixed_minus(tf.z, to_fixed(sh[2], S.fix));
+        const FixedSpot f = fixed_minus(tf, sh, S.fix);
 #pragma unroll 1
         for (int g = 0; g < nb32; ++g) {
             double rp = 0.0, rx = 0.0, ry = 0.0, rz = 0.0;
 #pragma unroll 2
             for (int k = 0; k < 32; ++k) {
                 const int s = 32 * g + ((lane + k) & 31);
-                const FixedPoint Q = s_fix[s];
+                const FixedSource Q = s_fix[s];
                 FixedPair v;                             // x_s + p - y
-                const bool near = !fixed_pair<true>(Q, fx, fy, fz, S.fix, v);
+                const bool near = !fixed_pair<true, true>(Q, f, tc, t.w, S.fix, v);
                 if (__any_sync(0xffffffffu, near)) {
                     __syncwarp();
-                    if (near) float64_pair<true>(s_src[s], a.pk[(S.tile0 + ta) * kTile64 + tid], sh, v);
+                    if (near) float64_pair<true, true>(s_src[s], a.pk[(S.tile0 + ta) * kTile64 + tid], sh, Q.q, v);
                 }
-                const double wa = Q.q * v.ri3;           // action
-                acc[0] = fma(Q.q, v.ri, acc[0]);
-                acc[1] = fma(v.ex, wa, acc[1]);
-                acc[2] = fma(v.ey, wa, acc[2]);
-                acc[3] = fma(v.ez, wa, acc[3]);
-                const double wb = t.w * v.ri3;           // reaction (field sign folded later)
-                rp = fma(t.w, v.ri, rp);
-                rx = fma(v.ex, wb, rx);
-                ry = fma(v.ey, wb, ry);
-                rz = fma(v.ez, wb, rz);
+                acc[0] = fma(Q.q, v.ri, acc[0]);         // action
+                acc[1] = fma(v.ex, v.wa, acc[1]);
+                acc[2] = fma(v.ey, v.wa, acc[2]);
+                acc[3] = fma(v.ez, v.wa, acc[3]);
+                rp = fma(t.w, v.ri, rp);                 // reaction (field sign folded later)
+                rx = fma(v.ex, v.wb, rx);
+                ry = fma(v.ey, v.wb, ry);
+                rz = fma(v.ez, v.wb, rz);
                 rp = __shfl_sync(0xffffffffu, rp, up);
                 rx = __shfl_sync(0xffffffffu, rx, up);
                 ry = __shfl_sync(0xffffffffu, ry, up);

@@ -2,7 +2,7 @@
 differences with their largest in every binade that takes the integer form, small and zero ones beside it, both
 signs, estimates up to three units in the last place off.  Bounds, in units of 2^-53 (half a unit in the last
 place of 1..2): the rounding to 53 bits is one; the squared distance loses four units of 2^58 at the most
-(2^-56), so 1/r another 2^-4 and 1/r^3 another 3 2^-4 and 2^-4 for its integer products; the differences are
+(2^-56), so 1/r another 2^-4 and q/r^3 another 3 2^-4 and 2^-4 for its integer products; the differences are
 rounded once.  The conversion of coordinates is exact to half a unit and saturates.
 
 Host only: compiled by the C++ compiler against the CUDA headers; skipped where either is missing."""
@@ -56,7 +56,10 @@ int main(int argc, char** argv) {
             memcpy(&yb, &y0, 4);
             const FixedInverse v = fixed_inverse(r, k, yb + q);
             w1 = std::max(w1, fabsl(fixed_ri(v) * rr - 1));
-            w3 = std::max(w3, fabsl(fixed_ri3(v) * rr * rr * rr - 1));
+            const double c = std::ldexp(1.0 + std::ldexp((double)(rng() >> 12), -52), (int)(rng() % 401) - 200) * (rng() & 1 ? 1 : -1);
+            FixedCharge fc, f0;
+            if (!fixed_charge(c, fc) || !fixed_charge(0.0, f0) || fixed_weight(fixed_cube(v), 3 * v.x, f0, 0.0) != 0) return 5;
+            w3 = std::max(w3, fabsl(fixed_weight(fixed_cube(v), 3 * v.x, fc, c) * rr * rr * rr / c - 1));
         }
         for (int i = 0; i < 3; ++i) {
             const long double t = (d[i].sign ? -1.0L : 1.0L) * d[i].a * u, g = fixed_value(d[i], k);
@@ -66,11 +69,17 @@ int main(int argc, char** argv) {
         const double c = std::ldexp((double)(long long)(rng() >> 1) * (rng() & 1 ? 1 : -1), top - 63 - k - (int)(rng() % 70));
         wc = std::max(wc, fabsl((long double)to_fixed(c, k) * u - c) / u);
     }
+    FixedCharge no;
     const double big = std::ldexp(1.0, 62 - k);
-    if (to_fixed(big, k) != 1ll << 62 || to_fixed(-4 * big, k) != -(1ll << 62) || to_fixed(INFINITY, k) != 1ll << 62 ||
-        to_fixed(-INFINITY, k) != -(1ll << 62) || to_fixed(std::nextafter(big, 0.0), k) >= 1ll << 62 ||
+    if (to_fixed(big, k) != kFixedOut || to_fixed(-4 * big, k) != kFixedOut || to_fixed(INFINITY, k) != kFixedOut ||
+        to_fixed(-INFINITY, k) != kFixedOut || to_fixed(NAN, k) != kFixedOut || to_fixed(std::nextafter(big, 0.0), k) >= 1ll << 62 ||
+        fixed_charge(4e-320, no) || fixed_charge(std::ldexp(1.0, 201), no) || fixed_charge(std::ldexp(-1.9, -201), no) ||
         to_fixed(0.0, k) || to_fixed(-5e-324, k) || to_fixed(1.0, kNoFixed) || to_fixed(-1e300, kNoFixed))
         return 4;
+    for (long long t = -(1ll << 62) + 1; t < 1ll << 62; t += (1ll << 58) + 12345) {
+        const FixedDelta d = fixed_delta(kFixedOut, t), b = fixed_delta(t, kFixedOut);
+        if ((d.a >> 32) < kFixedFar || (b.a >> 32) < kFixedFar) return 6;
+    }
     const long double h = ldexpl(1.0L, -53);
     printf("%Lg %Lg %Lg %Lg\n", w1 / h, w3 / h, wd / h, wc);
     return 0;

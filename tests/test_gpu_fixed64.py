@@ -34,7 +34,7 @@ def _run(x, q, d, y=None, **more):
         pc.close()
 
 
-FORMS = {"one_sided": dict(pairs="one-sided"), "symmetric": dict(pairs="symmetric"), "ball": dict(lam=1.6),
+FORMS = {"one-sided": dict(pairs="one-sided"), "symmetric": dict(pairs="symmetric"), "ball": dict(lam=1.6),
          "points": {}, "block_checks": dict(checks="points")}
 
 
@@ -51,6 +51,26 @@ def test_power_of_two_scales(form):
             ref = phi, g
         assert_close(phi * f, ref[0], 1e-12, f"{form} phi at 2^{e}")
         assert_close(g * f * f, ref[1], 1e-12, f"{form} grad at 2^{e}")
+
+
+@pytest.mark.parametrize("form", ["one-sided", "symmetric"])
+def test_power_of_two_charges(form):
+    # charges beyond 2^+-200 take the float64 form, as do all of a charge's pairs beside ordinary ones
+    s = W.uniform_gauss(N=389, d=(1.0, 1.5, 2.0), p=8, M=200, seed=74)
+    q = s.q.copy()
+    q[7::11] = 0.0
+    q[3] = 0.0
+    q[q != 0.0] -= q.sum() / np.count_nonzero(q)
+    ref = _run(s.x, q, s.d, pairs=form)
+    for e in (190, 240, -190, -240):
+        f = 2.0 ** e
+        phi, g = _run(s.x, q * f, s.d, pairs=form)
+        assert_close(phi / f, ref[0], 1e-12, f"{form} phi, charges 2^{e}")
+        assert_close(g / f, ref[1], 1e-12, f"{form} grad, charges 2^{e}")
+    q[3] = 1e-150
+    phi, g = _run(s.x, q, s.d, pairs=form)
+    assert_close(phi, ref[0], 1e-12, f"{form} phi, one tiny charge")
+    assert_close(g, ref[1], 1e-12, f"{form} grad, one tiny charge")
 
 
 @pytest.mark.parametrize("pairs", ["one-sided", "symmetric"])
