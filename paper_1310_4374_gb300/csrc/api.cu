@@ -238,7 +238,7 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
             one[0].shift0 = 0;
             one[0].n_img = n_img;
             one[0].fix = fixed_scale(pl.opt.d, pl.opt.K);
-            L.S = sym_partition(one, (int64_t)pl.num_sms * near64s_occupancy_ctas(), kTile64);
+            L.S = sym_partition(one, (int64_t)pl.num_sms * near64s_occupancy_ctas(L.n_tiles), kTile64);
             sym_bands(L, kTile64, pl.sym_band_bytes);
             L.sym = true;
         }

@@ -56,14 +56,16 @@ __host__ __device__ __forceinline__ double fixed_value(FixedDelta d, int k) {
 
 // The squared distance R 2^(64 - 2 s) units^2, R in [2^58, 2^62), of differences below 2^62 of which the
 // largest is at least kFixedNear 2^32: each is shifted until that one's leading bit is bit 61, and loses the
-// square of its low word, 3 units of R together.
+// square of its low word, 3 units of R together.  (Outside these bounds every function here gives some value
+// without meaning: the kernels compute it and throw it away.)
 struct FixedR2 {
     uint64_t R;
     int s;
 };
 __host__ __device__ __forceinline__ FixedR2 fixed_r2(FixedDelta x, FixedDelta y, FixedDelta z, uint32_t high) {
     FixedR2 r;
-    r.s = lead_zeros32(high) - 2;
+    const int s = lead_zeros32(high | kFixedNear) - 2;
+    r.s = s > 0 ? s : 0;
     const uint64_t a = x.a << r.s, b = y.a << r.s, c = z.a << r.s;
     const uint32_t ah = (uint32_t)(a >> 32), bh = (uint32_t)(b >> 32), ch = (uint32_t)(c >> 32);
     const uint64_t cross = (uint64_t)ah * (uint32_t)a + (uint64_t)bh * (uint32_t)b + (uint64_t)ch * (uint32_t)c;
@@ -71,7 +73,10 @@ __host__ __device__ __forceinline__ FixedR2 fixed_r2(FixedDelta x, FixedDelta y,
     return r;
 }
 // The float32 copy of R 2^-32 for the estimate of its inverse square root.
-__host__ __device__ __forceinline__ float fixed_estimate_arg(uint64_t R) { return (float)(uint32_t)(R >> 32); }
+__host__ __device__ __forceinline__ float fixed_estimate_arg(uint64_t R) {
+    const uint32_t h = (uint32_t)(R >> 32);
+    return (float)(h > 1u << 26 ? h : 1u << 26);
+}
 
 // mantissa M (leading one in bit 63 - z) times 2^(x - 1) with bit 52 as the unit, rounded
 __host__ __device__ __forceinline__ double fixed_assemble(uint64_t M, int z, int x) {
@@ -106,7 +111,7 @@ __host__ __device__ __forceinline__ FixedInverse fixed_inverse(FixedR2 r, int k,
     return v;
 }
 __host__ __device__ __forceinline__ double fixed_ri(FixedInverse v) {
-    const int z = lead_zeros32((uint32_t)(v.M >> 32));                 // 0..2
+    const int z = lead_zeros32((uint32_t)(v.M >> 32) | 0x20000000u);   // 0..2
     return fixed_assemble(v.M, z, v.x - z + 848);
 }
 // 1/r^3 = M3 2^(3 x - 584), M3 in [2^59, 2^62]

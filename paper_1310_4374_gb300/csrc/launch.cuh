@@ -37,7 +37,7 @@ cudaError_t launch_sym_reduce(const double* partial, int64_t n_valid, const Near
                               double* out_grad, cudaStream_t st, bool fp64 = false, bool accumulate = false);
 cudaError_t launch_near64s(const double4_32a* pk, const double* shifts, double* partial, const NearSymLaunch& S,
                            cudaStream_t st);
-int near64s_occupancy_ctas();
+int near64s_occupancy_ctas(int64_t n_tiles);
 int near32s_occupancy_ctas(int img_per_g, bool ff = false, bool refine = false);
 constexpr int kNear32Variants = 2;
 int near64_occupancy_ctas();

@@ -614,15 +614,7 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
         // the weight (1, -1 or 0) goes onto the charge's bits: no float64 operation
         const int w_and = w != 0.0 ? -1 : 0, w_xor = w < 0.0 ? (int)0x80000000 : 0;
         const int n_src = live ? kNearChunk : 0;
-#pragma unroll 2
-        for (int s = 0; s < n_src; ++s) {
-            const FixedSource Q = s_fix[s];
-            FixedPair v;                                          // x_i + p - y
-            const bool near = !fixed_pair<kGrad, false>(Q, f, Q.c, 0.0, S.fix, v);
-            if (__any_sync(0xffffffffu, near)) {
-                __syncwarp();
-                if (near) float64_pair<kGrad, false>(s_src[s], a.tgt[tile * kTile64 + tid], sh, Q.q, v);
-            }
+        auto step = [&](const FixedSource& Q, const FixedPair& v) {
             if (kGrad) {
                 acc[0] = fma(Q.q, v.ri, acc[0]);
                 acc[1 % NQ] = fma(v.ex, v.wa, acc[1 % NQ]);
@@ -631,6 +623,31 @@ __global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
             } else {
                 const double qw = __hiloint2double((__double2hiint(Q.q) & w_and) ^ w_xor, __double2loint(Q.q) & w_and);
                 acc[0] = fma(qw, v.ri, acc[0]);
+            }
+        };
+        for (int s0 = 0; s0 < n_src; s0 += 32) {
+            double acc0[NQ];
+#pragma unroll
+            for (int qi = 0; qi < NQ; ++qi) acc0[qi] = acc[qi];
+            bool near = false;
+#pragma unroll 4
+            for (int s = s0; s < s0 + 32; ++s) {
+                const FixedSource Q = s_fix[s];
+                FixedPair v;                                      // x_i + p - y
+                near |= !fixed_pair<kGrad, false>(Q, f, Q.c, 0.0, S.fix, v);
+                step(Q, v);
+            }
+            if (__any_sync(0xffffffffu, near)) {
+#pragma unroll
+                for (int qi = 0; qi < NQ; ++qi) acc[qi] = acc0[qi];
+#pragma unroll 1
+                for (int s = s0; s < s0 + 32; ++s) {
+                    const FixedSource Q = s_fix[s];
+                    FixedPair v;
+                    if (!fixed_pair<kGrad, false>(Q, f, Q.c, 0.0, S.fix, v))
+                        float64_pair<kGrad, false>(s_src[s], a.tgt[tile * kTile64 + tid], sh, Q.q, v);
+                    step(Q, v);
+                }
             }
         }
         ++u;

@@ -445,8 +445,8 @@ __device__ __forceinline__ FixedSource fixed_source(const double4_32a& v, int k)
 }
 
 // One pair for the float64 sums: 1/r, and with kField the difference s - t, the action q_s / r^3 and with
-// kMirror the reaction q_t / r^3.  false: the pair is left to the float64 form (near, coincident, or outside
-// the range).
+// kMirror the reaction q_t / r^3.  false: without meaning, the pair is left to the float64 form (near,
+// coincident, or outside the range).
 struct FixedPair {
     double ri, ex, ey, ez, wa, wb;
 };
@@ -455,7 +455,6 @@ __device__ __forceinline__ bool fixed_pair(const FixedSource& s, const FixedSpot
                                            FixedPair& o) {
     const FixedDelta dx = fixed_delta(s.at.x, t.x), dy = fixed_delta(s.at.y, t.y), dz = fixed_delta(s.at.z, t.z);
     const uint32_t high = (uint32_t)((dx.a | dy.a | dz.a) >> 32);
-    if (high - kFixedNear >= kFixedFar - kFixedNear) return false;
     const FixedR2 r = fixed_r2(dx, dy, dz, high);
     const FixedInverse v = fixed_inverse(r, k, __float_as_uint(rsqrt_mufu(fixed_estimate_arg(r.R))));
     o.ri = fixed_ri(v);
@@ -467,10 +466,12 @@ __device__ __forceinline__ bool fixed_pair(const FixedSource& s, const FixedSpot
         o.ey = fixed_value(dy, k);
         o.ez = fixed_value(dz, k);
     }
-    return true;
+    return high - kFixedNear < kFixedFar - kFixedNear;
 }
-// ... in float64.  Callers branch to it by a warp vote and a warp barrier, lest it be compiled into
-// predicated instructions, which would take the float64 pipe on or off.
+// ... in float64.  The kernels run a block of 32 sources in integers without a branch and, where a lane met
+// such a pair, go back to the sums before the block and run it again, each pair in its form: a vote at every
+// pair keeps a warp's pairs from overlapping, and it then takes four warps a scheduler to keep the float64
+// pipe at 92%.
 template <bool kField, bool kMirror>
 __device__ __forceinline__ void float64_pair(const double4_32a& s, const double4_32a& t, const double* sh, double q,
                                              FixedPair& o) {

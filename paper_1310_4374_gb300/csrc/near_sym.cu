@@ -859,9 +859,9 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) 
 //
 // Bound by the float64 pipe: 8 float64 operations per mirror pair, the multiply-adds of its eight sums; the
 // pair's geometry and its weights q/r^3 are integer work beside them (fixed64.cuh).  12 001 charges take
-// 28.1 ms; 34.7 with the two weights as float64 products, 64.0 with the differences, the squared distance and
-// the last steps of 1/r^3 in float64 too (18 operations).  A 16^3 lattice 3.61, 4.35, 7.98 ms; 1000 charges
-// 0.345, 0.411, 0.685 ms.
+// 27.6 ms; 34.7 with the two weights as float64 products, 64.0 with the differences, the squared distance and
+// the last steps of 1/r^3 in float64 too (18 operations).  A 16^3 lattice 3.38, 4.35, 7.98 ms; 1000 charges
+// 0.34, 0.41, 0.69 ms.
 // ---------------------------------------------------------------------------
 struct Near64SymArgs {
     const double4_32a* pk;   // charges (x, y, z, q), absolute, padded with far-away zero charges
@@ -938,16 +938,8 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
 #pragma unroll 1
         for (int g = 0; g < nb32; ++g) {
             double rp = 0.0, rx = 0.0, ry = 0.0, rz = 0.0;
-#pragma unroll 2
-            for (int k = 0; k < 32; ++k) {
-                const int s = 32 * g + ((lane + k) & 31);
-                const FixedSource Q = s_fix[s];
-                FixedPair v;                             // x_s + p - y
-                const bool near = !fixed_pair<true, true>(Q, f, tc, t.w, S.fix, v);
-                if (__any_sync(0xffffffffu, near)) {
-                    __syncwarp();
-                    if (near) float64_pair<true, true>(s_src[s], a.pk[(S.tile0 + ta) * kTile64 + tid], sh, Q.q, v);
-                }
+            const double acc0[4] = {acc[0], acc[1], acc[2], acc[3]};
+            auto step = [&](const FixedSource& Q, const FixedPair& v) {
                 acc[0] = fma(Q.q, v.ri, acc[0]);         // action
                 acc[1] = fma(v.ex, v.wa, acc[1]);
                 acc[2] = fma(v.ey, v.wa, acc[2]);
@@ -960,6 +952,28 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
                 rx = __shfl_sync(0xffffffffu, rx, up);
                 ry = __shfl_sync(0xffffffffu, ry, up);
                 rz = __shfl_sync(0xffffffffu, rz, up);
+            };
+            bool near = false;
+#pragma unroll 4
+            for (int k = 0; k < 32; ++k) {
+                const FixedSource Q = s_fix[32 * g + ((lane + k) & 31)];
+                FixedPair v;                             // x_s + p - y
+                near |= !fixed_pair<true, true>(Q, f, tc, t.w, S.fix, v);
+                step(Q, v);
+            }
+            if (__any_sync(0xffffffffu, near)) {
+#pragma unroll
+                for (int qi = 0; qi < 4; ++qi) acc[qi] = acc0[qi];
+                rp = rx = ry = rz = 0.0;
+#pragma unroll 1
+                for (int k = 0; k < 32; ++k) {
+                    const int s = 32 * g + ((lane + k) & 31);
+                    const FixedSource Q = s_fix[s];
+                    FixedPair v;
+                    if (!fixed_pair<true, true>(Q, f, tc, t.w, S.fix, v))
+                        float64_pair<true, true>(s_src[s], a.pk[(S.tile0 + ta) * kTile64 + tid], sh, Q.q, v);
+                    step(Q, v);
+                }
             }
             const int s = 32 * g + lane;                 // the lane holds source s's reaction
             s_re[warp][0][s] += rp;
@@ -1145,7 +1159,12 @@ cudaError_t launch_sym_reduce(const double* partial, int64_t n_valid, const Near
     return cudaGetLastError();
 }
 
-constexpr int kNear64sMinBlocks = 4;
+// Three resident CTAs, from kNear64sTiles tiles on four.  With the pairs of a warp overlapping, the fourth adds
+// 1% where the pair sum is all (12 001 charges 27.6 ms, 28.3 with three); below, the registers are better left
+// to a CTA of the check sums, which fill the integer pipes' idle slots (4096 charges 3.32 ms, 3.45 with four).
+constexpr int64_t kNear64sTiles = 48;
+using Near64sKernel = void (*)(Near64SymArgs);
+Near64sKernel near64s_instance(int64_t n_tiles) { return n_tiles >= kNear64sTiles ? k_near64s<4> : k_near64s<3>; }
 
 cudaError_t launch_near64s(const double4_32a* pk, const double* shifts, double* partial, const NearSymLaunch& S,
                            cudaStream_t st) {
@@ -1156,13 +1175,13 @@ cudaError_t launch_near64s(const double4_32a* pk, const double* shifts, double* 
     a.status = S.status; a.n_status = S.n_status; a.limit = sym_limit(S);
     const cudaError_t e = S.zeroed ? cudaSuccess : cudaMemsetAsync(S.counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    k_near64s<kNear64sMinBlocks><<<(unsigned)S.G, kThreads64, 0, st>>>(a);
+    near64s_instance(S.tab.one.n_tiles)<<<(unsigned)S.G, kThreads64, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-int near64s_occupancy_ctas() {
+int near64s_occupancy_ctas(int64_t n_tiles) {
     int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_near64s<kNear64sMinBlocks>, kThreads64, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, near64s_instance(n_tiles), kThreads64, 0);
     return nb < 1 ? 1 : nb;
 }
 

@@ -90,3 +90,13 @@ def test_near_pairs(pairs):
     assert np.all(np.abs(phi - ref["phi"]) <= 1e-12 * np.maximum(np.abs(ref["phi"]), np.abs(ref["phi"]).min() + 1.0))
     gn = np.linalg.norm(ref["grad"], axis=1)
     assert np.all(np.linalg.norm(g - ref["grad"], axis=1) <= 1e-12 * gn)
+
+
+@pytest.mark.parametrize("N", [47 * 128, 47 * 128 + 1, 48 * 128 + 127])
+def test_symmetric_at_the_fourth_cta(N):
+    # 47 and 48 tiles (three and four resident CTAs), full and ragged, against the one-sided kernel: the same
+    # terms in another order (float64 rounding of 27 N terms)
+    s = W.uniform_gauss(N=N, d=(1.0, 1.5, 2.0), p=8, M=200, seed=75)
+    a, b = _run(s.x, s.q, s.d, pairs="symmetric"), _run(s.x, s.q, s.d, pairs="one-sided")
+    assert_close(a[0], b[0], 1e-12, "phi")
+    assert_close(a[1], b[1], 1e-12, "grad")
