@@ -525,8 +525,9 @@ struct Near64Args {
 };
 
 
+// the potential in 80 registers: a CTA of it fits beside three of the symmetric kernel's
 template <bool kGrad>
-__global__ void __launch_bounds__(kThreads64) k_near64(Near64Args a) {
+__global__ void __launch_bounds__(kThreads64, kGrad ? 5 : 6) k_near64(Near64Args a) {
     __shared__ double4_32a s_src[kNearChunk];
     __shared__ FixedSource s_fix[kNearChunk];
     constexpr int NQ = kGrad ? 4 : 1;

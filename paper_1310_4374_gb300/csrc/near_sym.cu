@@ -859,9 +859,9 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) 
 //
 // Bound by the float64 pipe: 8 float64 operations per mirror pair, the multiply-adds of its eight sums; the
 // pair's geometry and its weights q/r^3 are integer work beside them (fixed64.cuh).  12 001 charges take
-// 27.6 ms; 34.7 with the two weights as float64 products, 64.0 with the differences, the squared distance and
-// the last steps of 1/r^3 in float64 too (18 operations).  A 16^3 lattice 3.38, 4.35, 7.98 ms; 1000 charges
-// 0.34, 0.41, 0.69 ms.
+// 27.7 ms; 34.7 with the two weights as float64 products, 64.0 with the differences, the squared distance and
+// the last steps of 1/r^3 in float64 too (18 operations).  A 16^3 lattice 3.43, 4.35, 7.98 ms; 1000 charges
+// called from Python 0.32, 0.41, 0.69 ms.
 // ---------------------------------------------------------------------------
 struct Near64SymArgs {
     const double4_32a* pk;   // charges (x, y, z, q), absolute, padded with far-away zero charges
@@ -919,22 +919,43 @@ __global__ void __launch_bounds__(kThreads64, kMinB) k_near64s(Near64SymArgs a) 
         const double* sh = a.shifts + 3 * (S.shift0 + im0 + im);
         const int sg = diag ? shift_sign(sh) : 1;
         if (sg < 0) continue;                    // a tile against itself: image -p by reaction
-        if (sg == 0) {                           // ... and its zero image one-sided
-            const double px = t.x - sh[0], py = t.y - sh[1], pz = t.z - sh[2];
-#pragma unroll 4
-            for (int s = 0; s < kNearChunk; ++s) {
-                const double4_32a Q = s_src[s];
-                const double ex = Q.x - px, ey = Q.y - py, ez = Q.z - pz;
-                const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
-                const double w = Q.w * rsqrt3_f64_k0(r2);    // K(0) = 0
-                acc[0] = fma(w, r2, acc[0]);
-                acc[1] = fma(ex, w, acc[1]);
-                acc[2] = fma(ey, w, acc[2]);
-                acc[3] = fma(ez, w, acc[3]);
+        const FixedSpot f = fixed_minus(tf, sh, S.fix);
+        // ... and its zero image one-sided, K(0) = 0: in float64 throughout (13 operations a pair) these blocks were
+        // the longest items of a small system (1000 charges 288 us, 265 so; 500 charges 133, 117)
+        if (sg == 0) {
+#pragma unroll 1
+            for (int g = 0; g < nb32; ++g) {
+                const double acc0[4] = {acc[0], acc[1], acc[2], acc[3]};
+                auto step = [&](double q, const FixedPair& v) {
+                    acc[0] = fma(q, v.ri, acc[0]);
+                    acc[1] = fma(v.ex, v.wa, acc[1]);
+                    acc[2] = fma(v.ey, v.wa, acc[2]);
+                    acc[3] = fma(v.ez, v.wa, acc[3]);
+                };
+                bool near = false;
+#pragma unroll 2
+                for (int s = 32 * g; s < 32 * g + 32; ++s) {
+                    FixedSource Q = s_fix[s];
+                    if (s == tid) {              // its values, finite, times 0
+                        Q.q = 0.0;
+                        fixed_charge(0.0, Q.c);
+                    }
+                    FixedPair v;
+                    near |= !fixed_pair<true, false>(Q, f, Q.c, 0.0, S.fix, v) && s != tid;
+                    step(Q.q, v);
+                }
+                if (!__any_sync(0xffffffffu, near)) continue;
+#pragma unroll
+                for (int qi = 0; qi < 4; ++qi) acc[qi] = acc0[qi];
+#pragma unroll 1
+                for (int s = 32 * g; s < 32 * g + 32; ++s) {
+                    FixedPair v;
+                    float64_pair<true, false>(s_src[s], t, sh, s_src[s].w, v);
+                    step(s_src[s].w, v);
+                }
             }
             continue;
         }
-        const FixedSpot f = fixed_minus(tf, sh, S.fix);
 #pragma unroll 1
         for (int g = 0; g < nb32; ++g) {
             double rp = 0.0, rx = 0.0, ry = 0.0, rz = 0.0;
@@ -1160,7 +1181,7 @@ cudaError_t launch_sym_reduce(const double* partial, int64_t n_valid, const Near
 }
 
 // Three resident CTAs, from kNear64sTiles tiles on four.  With the pairs of a warp overlapping, the fourth adds
-// 1% where the pair sum is all (12 001 charges 27.6 ms, 28.3 with three); below, the registers are better left
+// 1% where the pair sum is all (12 001 charges 27.7 ms, 28.3 with three); below, the registers are better left
 // to a CTA of the check sums, which fill the integer pipes' idle slots (4096 charges 3.32 ms, 3.45 with four).
 constexpr int64_t kNear64sTiles = 48;
 using Near64sKernel = void (*)(Near64SymArgs);
