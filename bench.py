@@ -43,8 +43,10 @@ FP32_OPS_PAIR_GRAD = 13    # FP32-pipe lane operations per potential+gradient pa
 # reactions added to the running sum)
 FP32_OPS_PAIR_SYM = 152 / 16
 FP32_OPS_PAIR_PHI = 7      # potential only (3 sub, 3 r^2, 1 fma)
-FP64_OPS_PAIR = 19         # float64 kernel, one-sided
-FP64_OPS_PAIR_SYM = 12     # float64 kernel, symmetric
+# float64 kernels, one-sided and symmetric: the four sums' multiply-adds per ordered pair; the pair's
+# geometry and weight are integer operations
+FP64_OPS_PAIR = 4
+FP64_OPS_PAIR_SYM = 4
 
 
 def workload_name(N=N_MAIN):
@@ -420,16 +422,13 @@ def fp64_leg(args):
         res[prec] = {"pairs_per_s": pairs / (ms * 1e-3), "ms_per_step": ms, "timed_steps": reps,
                      "near_charges_pairs_per_s": near_rate, "near_charges_ms": near_ms, "pair_kernel": kernel}
         if prec == "fp64":
-            # float64 lane operations per ordered pair: one-sided 3 offset, 3 r^2, 5 rsqrt
-            # refinement, 1 q/r, 1 sum, 2 weight, 3 field; symmetric per mirror pair 3 + 3 + 5
-            # + 1 (1/r^2) shared and 6 per direction, 24 for two ordered pairs
+            # float64 lane operations per ordered pair; the rest runs on the integer pipes
             ops = FP64_OPS_PAIR_SYM if kernel == "symmetric" else FP64_OPS_PAIR
             props = torch.cuda.get_device_properties(x.device)
             peak = props.multi_processor_count * 2 * float(measured_peaks().get("sm_max_mhz", 2070.0)) * 1e6
             res[prec]["roofline"] = {"bound": "alu", "kernel": "k_near64s" if kernel == "symmetric" else "k_near64",
-                                     "ops_per_pair": FP32_OPS_PAIR_ALG,
-                                     "achieved": FP32_OPS_PAIR_ALG * near_rate / 1e12, "peak": peak / 1e12,
-                                     "unit": "T FP64-pipe ops/s", "frac": FP32_OPS_PAIR_ALG * near_rate / peak,
+                                     "ops_per_pair": ops, "achieved": ops * near_rate / 1e12, "peak": peak / 1e12,
+                                     "unit": "T FP64-pipe ops/s", "frac": ops * near_rate / peak,
                                      "issue_frac": ops * near_rate / peak, "executed_ops_per_pair": ops,
                                      "peak_source": "SMs x 2 FP64 lanes x sm_max_mhz (nominal 1.25 TFLOP/s FP64; "
                                                     "1.90 DFMA/clk/SM measured)"}

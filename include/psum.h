@@ -216,7 +216,7 @@ int psum_eval(psum_plan_t plan, int64_t N, const double *x, const double *q,
               double *phi, double *grad, void *stream);
 
 /* psum_eval through a CUDA graph: the first call for a given (N, x, q, phi, grad) captures
-   the whole evaluation (about 25 kernels and memsets) on an internal stream and later calls
+   the whole evaluation (11 kernels and memsets up to 24320 charges) on an internal stream and later calls
    with the same arguments replay it on `stream`, which removes the per-kernel launch cost
    (it dominates below ~5000 charges).  The inputs may change between replays in the same
    buffers.  Results, status reporting (psum_sync) and asynchrony are those of psum_eval;

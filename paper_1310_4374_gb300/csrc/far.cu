@@ -1,10 +1,10 @@
 // Everything in algorithm "get" (Sec. 2.3.2) around the near-field sum:
-//   validation (Eq. 1: neutral box, positions inside it),
+//   validation (Eq. 1: neutral box, positions inside it), with the sort keys,
 //   the right-hand side f and the least-squares coefficients (steps 4-5, Eqs. 8-10),
 //   the constant C_1 from the zero-mean condition (step 6, Eqs. pfx3-pfx4, App. C),
-//   the far field and its gradient at the charges and the final sum (steps 7-8,
-//   Eqs. 1.6-1.9).
-// All of it runs in float64.
+//   the far field and its gradient at the charges and the final sum, with the pair sums'
+//   partial slots (steps 7-8, Eqs. 1.6-1.9).
+// All of it runs in float64 but the far field of FP32C plans, which is float32.
 #include "launch.cuh"
 #include "diffuse.cuh"
 #include "harmonics.cuh"

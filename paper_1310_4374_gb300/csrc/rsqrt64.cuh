@@ -1,6 +1,7 @@
 // Float64 1/r and 1/r^3 from a float32 estimate, with as few float64 operations as they need: the
 // float64 pipe (one warp instruction per scheduler in 64 cycles, conversions included) bounds the
-// float64 pair kernels, the integer and float32 pipes beside it are idle.
+// float64 pair kernels, the integer and float32 pipes beside it are idle.  The form of the pairs that the
+// integer coordinates leave out (fixed64.cuh).
 #pragma once
 
 #include <math.h>
