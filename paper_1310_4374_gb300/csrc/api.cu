@@ -181,7 +181,8 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
             one[0].n_img = n_img;
             one[0].tau2 = coincident_r2(pl.opt.d);
             const bool rf = refined_terms(pl);
-            L.S = sym_partition(one, (int64_t)pl.num_sms * near32s_occupancy_ctas(n_img, ffp, rf));
+            L.S = sym_partition(one, (int64_t)pl.num_sms * near32s_occupancy_ctas(n_img, ffp, rf),
+                                ffp ? kSymItemsPerCta : rf ? kSymLastItemsRefined : kSymLastItemsFast);
             L.S.G = (int64_t)pl.num_sms * near32s_occupancy_ctas(L.S.max_ipg, ffp, rf);
             sym_bands(L, kTile32, pl.sym_band_bytes);
             L.sym = true;
@@ -238,7 +239,8 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
             one[0].shift0 = 0;
             one[0].n_img = n_img;
             one[0].fix = fixed_scale(pl.opt.d, pl.opt.K);
-            L.S = sym_partition(one, (int64_t)pl.num_sms * near64s_occupancy_ctas(L.n_tiles), kTile64);
+            L.S = sym_partition(one, (int64_t)pl.num_sms * near64s_occupancy_ctas(L.n_tiles),
+                                kSymItemsPerCta, kTile64);
             sym_bands(L, kTile64, pl.sym_band_bytes);
             L.sym = true;
         }

@@ -603,6 +603,12 @@ struct NearSymLaunch {
 #define PSUM_SYM_ITEMS_PER_CTA 8
 #endif
 constexpr int kSymItemsPerCta = PSUM_SYM_ITEMS_PER_CTA;
+// The last step, to one image per group, stages a chunk, forms its offsets and passes its reaction sums on for
+// every image anew: a tenth of an item with the fast float32 terms.  They take it only below one item per
+// CTA (8000 charges 0.784 ms with one image a group, 0.737 with three; 12 000 1.600, 1.452; 16 000 2.722, 2.418), the
+// refined ones, whose images take longer, below four (8000 charges 1.150, 1.183; 12 000 2.432, 2.363; 16 000
+// 4.204, 3.990); float-float (12 000 charges 11.13, 11.17) and float64 by the rule above.
+constexpr int kSymLastItemsFast = 1, kSymLastItemsRefined = 4;
 // automatic choice (measured crossovers against the one-sided kernels): FP32C from 12 tiles of
 // 512 charges (5500 charges even), float-float from 6 (3000 even), float64 at every size (1.64x
 // at 1000 charges)
@@ -631,8 +637,8 @@ inline int64_t sym_band_width(int64_t n_tiles, size_t slot_bytes, size_t cap) {
 }
 
 // `sys` holds tile0, n_tiles, n_chunks, shift0 and n_img of every system; the rest is filled
-// here.  G is the number of resident CTAs.
-inline NearSymLaunch sym_partition(std::vector<SymSys>& sys, int64_t G, int tile = kTile32) {
+// here.  G is the number of resident CTAs, last_items the items per CTA below which each image is a group.
+inline NearSymLaunch sym_partition(std::vector<SymSys>& sys, int64_t G, int last_items, int tile = kTile32) {
     NearSymLaunch S;
     int64_t pairs = 0;
     int max_img = 1;
@@ -641,7 +647,7 @@ inline NearSymLaunch sym_partition(std::vector<SymSys>& sys, int64_t G, int tile
         max_img = s.n_img > max_img ? s.n_img : max_img;
     }
     int ng = 1;
-    while (ng < max_img && pairs * ng < kSymItemsPerCta * G) ng *= 3;
+    while (ng < max_img && pairs * ng < (3 * ng >= max_img ? last_items : kSymItemsPerCta) * G) ng *= 3;
     int64_t item = 0;
     size_t part = 0;
     for (SymSys& s : sys) {
