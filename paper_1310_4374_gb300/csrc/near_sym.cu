@@ -300,6 +300,49 @@ __device__ __forceinline__ void sym_ff_step(const float4* __restrict__ s_hi, con
     }
 }
 
+// The offsets of a staged chunk from the target groups of tile TA, and the units' classes, for nimg images
+// from im0 on: a thread per (image, group), the classes joined over the four groups (one thread an
+// image took its groups' 35 float64 operations four times over, 9000 cycles a chunk).
+__device__ __forceinline__ void chunk_offsets(const Near32SymArgs& a, int im0, int nimg, int64_t TA, int64_t chunk,
+                                              bool diag, float* s_delta, int* s_near) {
+    const double* so = a.org + 4 * chunk;
+    for (int e = threadIdx.x; e < nimg * kTgt32; e += kThreads32) {
+        const int im = e / kTgt32, k = e % kTgt32;
+        const double* sh = a.shifts + 3 * (im0 + im);
+        const double* to = a.org + 4 * (TA * kTgt32 + k);
+        const double D0 = (to[0] - so[0]) - sh[0], D1 = (to[1] - so[1]) - sh[1], D2 = (to[2] - so[2]) - sh[2];
+        float* dl = s_delta + 6 * e;
+        dl[0] = (float)D0; dl[1] = (float)D1; dl[2] = (float)D2;
+        dl[3] = (float)(D0 - (double)dl[0]); dl[4] = (float)(D1 - (double)dl[1]);
+        dl[5] = (float)(D2 - (double)dl[2]);
+        bool near;
+        if (a.ext) {
+            // the gap between the two bounding boxes bounds every pair distance from below
+            const float4 ht = a.ext[TA * kTgt32 + k], hs = a.ext[chunk];
+            const double g0 = fmax(0.0, fabs(D0) - ((double)ht.x + (double)hs.x));
+            const double g1 = fmax(0.0, fabs(D1) - ((double)ht.y + (double)hs.y));
+            const double g2 = fmax(0.0, fabs(D2) - ((double)ht.z + (double)hs.z));
+            const double gap = (kNearFactor - 1.0) * (to[3] + so[3]);
+            near = g0 * g0 + g1 * g1 + g2 * g2 <= gap * gap;
+        } else {
+            const double reach = kNearFactor * (to[3] + so[3]);
+            near = D0 * D0 + D1 * D1 + D2 * D2 <= reach * reach;
+        }
+        int nr = quad_or(near ? (k < 2 ? kUnitNear0 : kUnitNear1) : 0);
+        if (diag) {
+            const int sg = shift_sign(sh);
+            nr = sg < 0 ? kUnitMirrored : sg == 0 ? nr | kUnitSelf : nr;
+        }
+        if (k == 0) s_near[im] = nr;
+    }
+}
+// ... as a call: inlined into the refined kernel it takes three registers of the pair loop's (60 000 dipole charges
+// 53.2 ms, 52.3 with the call); the fast one is better inlined (1e5 charges 81.6 ms, 82.6 with the call).
+__device__ __noinline__ void chunk_offsets_call(const Near32SymArgs& a, int im0, int nimg, int64_t TA, int64_t chunk,
+                                                bool diag, float* s_delta, int* s_near) {
+    chunk_offsets(a, im0, nimg, TA, chunk, diag, s_delta, s_near);
+}
+
 template <int kMinB, bool kFF, bool kRefine = false>
 __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) {
     static_assert(!(kFF && kRefine), "float-float pairs need no refinement");
@@ -391,38 +434,10 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) 
         // alone are skipped (their reactions stay zero)
         const int nv = chunk == S.tile0 * kTgt32 + S.n_chunks - 1 && S.last_n > 0 ? S.last_n : kNearChunk;
         const int nb32 = (nv + 31) >> 5, nb64 = (nv + 63) >> 6;
-        const double* so = a.org + 4 * chunk;
-        // a thread per (image, target group), the classes joined over the four groups: one thread
-        // an image took its groups' 35 float64 operations four times over, 9000 cycles a chunk
-        for (int e = tid; e < nimg * kTgt32; e += kThreads32) {
-            const int im = e / kTgt32, k = e % kTgt32;
-            const double* sh = a.shifts + 3 * (S.shift0 + im0 + im);
-            const double* to = a.org + 4 * (TA * kTgt32 + k);
-            const double D0 = (to[0] - so[0]) - sh[0], D1 = (to[1] - so[1]) - sh[1], D2 = (to[2] - so[2]) - sh[2];
-            float* dl = s_delta + 6 * e;
-            dl[0] = (float)D0; dl[1] = (float)D1; dl[2] = (float)D2;
-            dl[3] = (float)(D0 - (double)dl[0]); dl[4] = (float)(D1 - (double)dl[1]);
-            dl[5] = (float)(D2 - (double)dl[2]);
-            bool near;
-            if (a.ext) {
-                // the gap between the two bounding boxes bounds every pair distance from below
-                const float4 ht = a.ext[TA * kTgt32 + k], hs = a.ext[chunk];
-                const double g0 = fmax(0.0, fabs(D0) - ((double)ht.x + (double)hs.x));
-                const double g1 = fmax(0.0, fabs(D1) - ((double)ht.y + (double)hs.y));
-                const double g2 = fmax(0.0, fabs(D2) - ((double)ht.z + (double)hs.z));
-                const double gap = (kNearFactor - 1.0) * (to[3] + so[3]);
-                near = g0 * g0 + g1 * g1 + g2 * g2 <= gap * gap;
-            } else {
-                const double reach = kNearFactor * (to[3] + so[3]);
-                near = D0 * D0 + D1 * D1 + D2 * D2 <= reach * reach;
-            }
-            int nr = quad_or(near ? (k < 2 ? kUnitNear0 : kUnitNear1) : 0);
-            if (diag) {
-                const int sg = shift_sign(sh);
-                nr = sg < 0 ? kUnitMirrored : sg == 0 ? nr | kUnitSelf : nr;
-            }
-            if (k == 0) s_near[im] = nr;
-        }
+        if constexpr (kRefine)
+            chunk_offsets_call(a, S.shift0 + im0, nimg, TA, chunk, diag, s_delta, s_near);
+        else
+            chunk_offsets(a, S.shift0 + im0, nimg, TA, chunk, diag, s_delta, s_near);
         const long long limit = a.inject ? (1LL << 12) : kCopySpinLimit;
         if (tid == 0 && !mbar_wait(&s_bar, phase, limit)) s_fail = 1;
         phase ^= 1u;
