@@ -573,9 +573,9 @@ __global__ void __launch_bounds__(kThreads64, kGrad ? 5 : 6) k_near64(Near64Args
             tf = fixed_spot(t, S.fix);
             // a class outside 0..n_cls-1 reads class 0: the index stays inside the tables
             tcls = (!kGrad && a.n_cls > 1 && t.w >= 0.0 && t.w < (double)a.n_cls) ? (int)t.w : 0;
-            // check points are distinct, so a warp of targets at the padding's place holds padding alone:
-            // it runs no pair (M = 200 fills 25 of 32 quarter warps of its two tiles, M = 400 25 of 32)
-            live = kGrad || __any_sync(0xffffffffu, !(t.x == 1.0e3 && t.y == 1.0e3 && t.z == 1.0e3));
+            // a warp of padding (kPadCheck) runs no pair: M = 200 fills 7 of the 8 warps of its two tiles,
+            // M = 400 13 of 16
+            live = kGrad || __any_sync(0xffffffffu, t.w >= 0.0);
 #pragma unroll
             for (int qi = 0; qi < NQ; ++qi) acc[qi] = 0.0;
             cur_tile = tile;

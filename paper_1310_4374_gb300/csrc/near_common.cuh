@@ -409,19 +409,17 @@ __device__ __forceinline__ double rsqrt3_f64_k0(double r2) {
     return r2f > 0.f ? ri3 : 0.0;
 }
 
-// A packed point in integer coordinates (fixed64.cuh).  The packs' padding (1e3, 1e3, 1e3), no charge, is
-// put at the origin: outside the range it would send every pair of its warp through the float64 form, as
-// kFixedOut does on purpose for a charge without integer form (x of a source, y of a target: both at once are
-// out of range too).
+// A packed point in integer coordinates (fixed64.cuh).  The packs' padding (pad64) lies in the box, inside every
+// range: outside, it would send every pair of its warp through the float64 form, as kFixedOut does on purpose for
+// a charge without integer form (x of a source, y of a target: both at once are out of range too).
 struct FixedSpot {
     long long x, y, z;
 };
 __device__ __forceinline__ FixedSpot fixed_spot(const double4_32a& v, int k) {
-    const bool pad = v.x == 1.0e3 && v.y == 1.0e3 && v.z == 1.0e3;
     FixedSpot f;
-    f.x = pad ? 0 : to_fixed(v.x, k);
-    f.y = pad ? 0 : to_fixed(v.y, k);
-    f.z = pad ? 0 : to_fixed(v.z, k);
+    f.x = to_fixed(v.x, k);
+    f.y = to_fixed(v.y, k);
+    f.z = to_fixed(v.z, k);
     return f;
 }
 __device__ __forceinline__ FixedSpot fixed_minus(const FixedSpot& a, const double* sh, int k) {

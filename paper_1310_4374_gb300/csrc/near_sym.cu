@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32s(Near32SymArgs a) 
 // called from Python 0.32, 0.41, 0.69 ms.
 // ---------------------------------------------------------------------------
 struct Near64SymArgs {
-    const double4_32a* pk;   // charges (x, y, z, q), absolute, padded with far-away zero charges
+    const double4_32a* pk;   // charges (x, y, z, q), absolute, padded with zero charges (pad64)
     const double* shifts;
     double* partial;         // per system [n_tiles][n_tiles * n_g][4][kTile64] from part0
     SymSysTable tab;

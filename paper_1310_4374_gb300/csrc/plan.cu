@@ -367,7 +367,7 @@ static int build_check_layers(Plan& pl, const double d[3]) {
         if ((s1 = upload(&pl.d_lc_gmask, gmask.data(), gmask.size()))) return s1;
         if ((s1 = upload(&pl.d_lc_sub, sub.data(), sub.size()))) return s1;
     } else {
-        std::vector<double4_32a> pk(slot.size(), make_double4_32a(1e3, 1e3, 1e3, 0.0));
+        std::vector<double4_32a> pk(slot.size(), pad64(kPadCheck));
         for (size_t i = 0; i < slot.size(); ++i)
             if (slot[i] >= 0)
                 pk[i] = make_double4_32a(pl.Y[3 * (size_t)slot[i]], pl.Y[3 * (size_t)slot[i] + 1],
@@ -583,7 +583,7 @@ int build_plan(const psum_opts& o, Plan& pl) {
         const int tile = kTile64;
         pl.check_tile = tile;
         pl.n_check_tiles = (pl.n_check + tile - 1) / tile;
-        std::vector<double4_32a> pk((size_t)pl.n_check_tiles * tile, make_double4_32a(1e3, 1e3, 1e3, 0.0));
+        std::vector<double4_32a> pk((size_t)pl.n_check_tiles * tile, pad64(kPadCheck));
         for (int j = 0; j < pl.n_check; ++j) {
             pk[j] = make_double4_32a(pts[3 * (size_t)j], pts[3 * (size_t)j + 1], pts[3 * (size_t)j + 2], 0.0);
             pos[j] = j;

@@ -28,6 +28,11 @@ constexpr int kTgt32 = 4;                 // targets per thread, FP32C kernel (2
 constexpr int kTile32 = kThreads32 * kTgt32;
 constexpr int kThreads64 = 128;           // threads per CTA, FP64 kernel
 constexpr int kTile64 = kThreads64;       // one target per thread
+// Padding of the float64 packs: a point at the box's centre, which a charge may share (every position in the box
+// is valid, so no position tells padding), hence told by index.  As a charge its 0 adds nothing; as a check target
+// its fourth component, a class or 0 for a check point, is kPadCheck.
+constexpr double kPadCheck = -1.0;
+__host__ __device__ __forceinline__ double4_32a pad64(double w) { return make_double4_32a(0.0, 0.0, 0.0, w); }
 constexpr int kMaxImages = 343;           // K <= 3 per axis; trimmed plans: images kept
 constexpr int kMaxDegree = 40;
 

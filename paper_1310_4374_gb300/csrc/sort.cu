@@ -302,7 +302,7 @@ __global__ void k_pack64(const double* __restrict__ x, const double* __restrict_
     if (s < n)
         pk[s] = make_double4_32a(x[3 * s], x[3 * s + 1], x[3 * s + 2], q ? q[s] : 0.0);
     else
-        pk[s] = make_double4_32a(1.0e3, 1.0e3, 1.0e3, 0.0);
+        pk[s] = pad64(0.0);
 }
 
 // batches: packed point s of group g = s / 128 holds charge grp_start[g] + s % 128 if
@@ -318,7 +318,7 @@ __global__ void k_pack64_groups(const double* __restrict__ x, const double* __re
         const int64_t i = grp_start[g] + k;
         pk[s] = make_double4_32a(x[3 * i], x[3 * i + 1], x[3 * i + 2], q[i]);
     } else {
-        pk[s] = make_double4_32a(1.0e3, 1.0e3, 1.0e3, 0.0);
+        pk[s] = pad64(0.0);
     }
 }
 
