@@ -406,7 +406,7 @@ __device__ __forceinline__ double rsqrt_f64_k0(double r2) {
 __device__ __forceinline__ double rsqrt3_f64_k0(double r2) {
     const float r2f = estimate_arg(r2);
     const double ri3 = rsqrt3_refined(r2, __float_as_uint(rsqrt_mufu(r2f)));
-    return r2f > 0.f ? ri3 : 0.0;
+    return r2f > 0.f ? ri3 : rsqrt3_below(r2);
 }
 
 // A packed point in integer coordinates (fixed64.cuh).  The packs' padding (pad64) lies in the box, inside every
@@ -470,6 +470,7 @@ __device__ __forceinline__ bool fixed_pair(const FixedSource& s, const FixedSpot
 // such a pair, go back to the sums before the block and run it again, each pair in its form: a vote at every
 // pair keeps a warp's pairs from overlapping, and it then takes four warps a scheduler to keep the float64
 // pipe at 92%.
+constexpr double kMaxDouble = 1.7976931348623157e308;
 template <bool kField, bool kMirror>
 __device__ __forceinline__ void float64_pair(const double4_32a& s, const double4_32a& t, const double* sh, double q,
                                              FixedPair& o) {
@@ -482,6 +483,11 @@ __device__ __forceinline__ void float64_pair(const double4_32a& s, const double4
         o.ri = ri3 * r2;
         o.wa = q * ri3;
         if (kMirror) o.wb = t.w * ri3;
+        if (o.ri > kMaxDouble) {         // rsqrt3_below: no charge (padding), no field
+            o.ri = kMaxDouble;
+            if (q == 0.0) o.wa = 0.0;
+            if (kMirror && t.w == 0.0) o.wb = 0.0;
+        }
     } else {
         o.ri = rsqrt_f64_k0(r2);
     }

@@ -404,14 +404,15 @@ inline float coincident_r2(const double d[3]) {
 
 // The exponent k of the float64 pair kernels' integer coordinates (fixed64.cuh): 2^(62-k) above every
 // coordinate difference y - x - p, y in the box or on the sphere around it (half diagonal R0), x in the
-// box, p an image of the block or of the layer next to it.  Outside 2^+-60 every pair is float64 throughout.
+// box, p an image of the block or of the layer next to it.  Every pair is float64 throughout below 2^-53 (so that
+// the integers hold no pair of the 2^-63 where rsqrt64.cuh's range ends, 2^-9 of the range) and above 2^60.
 inline int fixed_scale(const double d[3], const int K[3]) {
     double m = 0.0;
     for (int i = 0; i < 3; ++i) m = std::fmax(m, (K[i] + 2.0) * d[i]);
     m += 0.5 * std::sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
     int e;
     std::frexp(m * (1.0 + 1e-6), &e);
-    return e >= -60 && e <= 60 ? 62 - e : kNoFixed;
+    return e >= -53 && e <= 60 ? 62 - e : kNoFixed;
 }
 
 struct NearSys {

@@ -41,11 +41,16 @@ __host__ __device__ __forceinline__ uint32_t round_u32(float v) {
 }
 
 // The float32 copy of r2 for the estimate: the exponent rebiased (1023 -> 127) and the mantissa cut to
-// 23 bits, on the bits; r2 below 2^-126 counts as zero, which would need two distinct charges within
-// 1e-19 of each other.
+// 23 bits, on the bits; 0 below 2^-126, which would need two charges within 1e-19 of each other.
 __host__ __device__ __forceinline__ float estimate_arg(double r2) {
     const long long t = (f64_bits(r2) >> 29) - (896LL << 23);
     return f32_from(t >= 1LL << 23 ? (uint32_t)t : 0u);
+}
+// 1/r^3 where that copy is 0: charges within 2^-63.5 count as coincident, K(0) = 0; up to 2^-63 the pair is out of
+// the form's range, and an infinite field has the evaluation refused as not finite.
+__host__ __device__ __forceinline__ double rsqrt3_below(double r2) {
+    const long long t = (f64_bits(r2) >> 29) - (896LL << 23);
+    return f64_from(t > 0 && t < 1LL << 23 ? 0x7ffLL << 52 : 0LL);
 }
 // The magnitude of a float64 below 1 as float32, 20 mantissa bits; 0 below 2^-100.
 __host__ __device__ __forceinline__ float small_magnitude(double e) {
