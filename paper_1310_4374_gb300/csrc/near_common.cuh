@@ -100,9 +100,10 @@ __device__ __forceinline__ int shift_sign(const double* sh) {
                         : sh[1] != 0.0 ? (sh[1] > 0.0 ? 1 : -1) : sh[2] != 0.0 ? (sh[2] > 0.0 ? 1 : -1) : 0;
 }
 
-// the OR over four neighbouring lanes (all four active)
+// the OR over the lanes of a quad, all four of which arrive (a loop over items of four neighbouring threads): the
+// mask names them, so that they wait for each other wherever the warp has come apart
 __device__ __forceinline__ int quad_or(int v) {
-    const unsigned m = __activemask();
+    const unsigned m = quad_mask(threadIdx.x);
     v |= __shfl_xor_sync(m, v, 1);
     return v | __shfl_xor_sync(m, v, 2);
 }

@@ -105,6 +105,9 @@ __host__ __device__ __forceinline__ uint32_t curve_key(const double* p, const do
                          curve_cell(p[2], d[2], inv[2]));
 }
 
+// the four neighbouring lanes (0..3, 4..7, ...) of a thread's warp that hold it
+__host__ __device__ __forceinline__ unsigned quad_mask(int thread) { return 0xfu << (thread & 28); }
+
 // two-layer check points: flag in a group's class mask for a group of padding alone
 constexpr int kGroupEmpty = 1 << 30;
 
