@@ -544,7 +544,8 @@ int queue_forward(psum_plan_s* h, int64_t N, const double* x, const double* q, d
                 a.grad_acc = L.grad_n;
             }
         } else {
-            a.limit = L.n_tiles * L.Ln.max_contrib * 4 * tile;
+            const int64_t real = L.n_tiles * L.Ln.max_contrib * 4 * tile;
+            a.limit = h->debug_limit > 0 && h->debug_limit < real ? h->debug_limit : real;
         }
         a.status = L.eval_status;
         FarArgs f{ex, NE, eperm, pl.d_C, pl.d_Rbox, L.mean, zero_mean ? 1 : 0, o.p, 1.0 / pl.R0, phi, grad, pl.d_status};

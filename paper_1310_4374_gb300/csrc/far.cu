@@ -573,12 +573,32 @@ cudaError_t launch_constant(double* C, const double* Rbox, int P, const double* 
     return cudaGetLastError();
 }
 
+// Debug builds: a slot read refused inside the kernel before (debug_in_range) is known to all of it only when it
+// has ended, so it reaches the outputs and the plan's status here, as a refused write does in that kernel.
+#if PSUM_DEBUG_CHECKS
+__global__ void k_refused_reads(FarArgs f, const int* __restrict__ status) {
+    if (!(*status & kStatBounds)) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) atomicOr(f.plan_status, kStatBounds);
+    if (i >= f.n) return;
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    f.phi[i] = nan;
+    if (f.grad) f.grad[3 * i] = f.grad[3 * i + 1] = f.grad[3 * i + 2] = nan;
+}
+#endif
+static cudaError_t finish_sum_far(const FarArgs& f, const NearSlots& a, cudaStream_t st) {
+#if PSUM_DEBUG_CHECKS
+    k_refused_reads<<<(unsigned)((f.n + 255) / 256), 256, 0, st>>>(f, a.status);
+#endif
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sum_far32(const FarArgs& f, const NearSlots& a, const float* tab32, cudaStream_t st) {
     const int P = (f.p + 1) * (f.p + 1);
     const size_t smem = sizeof(double) * (kSlotWarps + 1) * 128 + sizeof(float) * (P + sh_tab_size(f.p));
     const auto kernel = f.grad ? k_sum_far32<true> : k_sum_far32<false>;
     kernel<<<(unsigned)((f.n + 31) / 32), 32 * (kSlotWarps + 1), smem, st>>>(f, a, tab32);
-    return cudaGetLastError();
+    return finish_sum_far(f, a, st);
 }
 
 cudaError_t launch_sum_far64(const FarArgs& f, const NearSlots& a, const double* tab64, const double* grad_tab,
@@ -591,7 +611,7 @@ cudaError_t launch_sum_far64(const FarArgs& f, const NearSlots& a, const double*
         if (e != cudaSuccess) return e;
     }
     kernel<<<(unsigned)((f.n + 31) / 32), 32 * (W + kSlotWarps), smem, st>>>(f, a, tab64, grad_tab);
-    return cudaGetLastError();
+    return finish_sum_far(f, a, st);
 }
 
 }  // namespace psum
