@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
         };
         // sources the unit's pair loops run over: the staged chunk, or for a unit that
         // straddles the ball its sources inside the ball, compacted (padded to whole blocks
-        // of 4 with far-away zero charges)
+        // of 4 with zero charges at the chunk's origin, as the pack does)
         const float4* uhi = s_hi;
         const float4* ulo = s_lo;
         int un = kNearChunk;
@@ -337,8 +337,8 @@ __global__ void __launch_bounds__(kThreads32, kMinB) k_near32(Near32Args a) {
             }
             const int padded = (total + kNearFold - 1) / kNearFold * kNearFold;
             if (tid >= total && tid < padded) {
-                s_hm[2 * tid] = make_float4(1.0e3f, 1.0e3f, 1.0e3f, 1.0e3f);
-                s_hm[2 * tid + 1] = make_float4(1.0e3f, 1.0e3f, 0.f, 0.f);
+                s_hm[2 * tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+                s_hm[2 * tid + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
                 s_hm[2 * kNearChunk + 2 * tid] = make_float4(0.f, 0.f, 0.f, 0.f);
                 s_hm[2 * kNearChunk + 2 * tid + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
             }

@@ -198,14 +198,14 @@ static int upload(T** dst, const T* src, size_t count) {
 }
 
 // Packs points for the float32 pair kernels: slot i of the pack holds point slot_pt[i]
-// (-1: padding far outside the box, never read back), 2 float4 of hi parts per slot
+// (-1: padding at the group's origin, its class outside the range), 2 float4 of hi parts per slot
 // followed by the same of lo parts, each an offset from its group's float64 origin (the
 // centre of the group's bounding box; 4 doubles per group with the radius about it).
 static void pack_groups32(const std::vector<double>& pts, const std::vector<int>& slot_pt, int ngroups,
                           std::vector<float4>& pk, std::vector<double>& org) {
     const size_t npk = 2 * (size_t)ngroups * kNearChunk;
     pk.assign(2 * npk, make_float4(0.f, 0.f, 0.f, 0.f));
-    for (size_t i = 0; i < npk; ++i) pk[i] = make_float4(1e3f, 1e3f, 1e3f, 1e3f);
+    for (size_t i = 1; i < npk; i += 2) pk[i] = make_float4(0.f, 0.f, 1e3f, 1e3f);
     org.assign(4 * (size_t)ngroups, 0.0);
     for (int g = 0; g < ngroups; ++g) {
         double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};

@@ -110,8 +110,9 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t* _
 // each point's offset from the origin is split into a float32 hi part and the float32
 // rounding remainder lo, packed two float4 each: (x,x,y,y),(z,z,q,q) and (xl,xl,yl,yl),(zl,zl,ql,ql)
 // (ql = q - float(q), read only by the float-float kernels).
-// Padding points (s >= n) get q = 0 and a far-away position.  `ext` (optional) receives each
-// group's bounding-box half extents about its origin.
+// Padding points (s >= n) get q = 0 and the origin: a far unit's targets all lie outside the group, off its
+// origin (any other place may be a charge's in some box: 1/0 there, times 0, is no number), and a near unit
+// takes K(0) = 0.  `ext` (optional) receives each group's bounding-box half extents about its origin.
 // With a group table (batches) group g covers the sorted positions
 // [grp_start[g], grp_start[g] + grp_count[g]); without one, [128 g, min(128 (g+1), n)).
 //
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(kPackThreads) k_pack32(const double* __restric
     double r2 = 0.0;
     const int64_t s = grp * kNearChunk + tid;
     {
-        float fx = 1.0e3f, fy = 1.0e3f, fz = 1.0e3f, fc = 0.f, lx = 0.f, ly = 0.f, lz = 0.f, lq = 0.f;
+        float fx = 0.f, fy = 0.f, fz = 0.f, fc = 0.f, lx = 0.f, ly = 0.f, lz = 0.f, lq = 0.f;
         if (ok) {
             const double rx = px[0] - o[0], ry = px[1] - o[1], rz = px[2] - o[2];
             r2 = rx * rx + ry * ry + rz * rz;
