@@ -337,11 +337,12 @@ int psum_check_form(psum_plan_t plan, int *form);
  * PSUM_NUM_STAGES durations (milliseconds) of the last evaluation:
  *   [0] validation, spatial sort and packing
  *   [1] near-field sum at the charges (potential and gradient)
- *   [2] the charges' reduction
+ *   [2] the charges' reduction of RBF plans; about 0 for spherical ones, whose far field adds up
+ *       the pair sums' partial results itself, in [4]
  *   [3] what is left of the check-point sums, the least squares, the box mean and C_1: those
  *       run on internal streams of the lowest priority from the end of [0] (the mean from its
  *       start), beside the charge sum, and fill the SMs it releases as it finishes
- *   [4] far field, combination and write-back
+ *   [4] the charges' partial sums (spherical plans), C_1, far field, combination and write-back
  * Returns PSUM_ERR_ARG if profiling is off. */
 #define PSUM_NUM_STAGES 5
 int psum_profile(psum_plan_t plan, int enable);
@@ -404,8 +405,8 @@ void psum_batch_destroy(psum_batch_t batch);
 int psum_debug_inject_timeout(psum_plan_t plan, int enable);
 
 /* Debug builds (the paper has no counterpart).  A library compiled with -DPSUM_DEBUG_CHECKS=1
-   range-checks every write and read of the pair kernels' partial sums against the buffer's size:
-   an access outside it is skipped and flagged, psum_sync returns PSUM_ERR_INTERNAL and the outputs
+   range-checks the writes and reads of an evaluation's partial sums against the buffer's size (the
+   float64 one-sided kernel's writes and the RBF plans' one-sided reduction are not checked): an access outside it is skipped and flagged, psum_sync returns PSUM_ERR_INTERNAL and the outputs
    are NaN, and the CUDA context stays usable (no trap).  psum_debug_checks() returns 1 in such a
    build, 0 otherwise.  psum_debug_bounds_limit is its test hook: the checks see the partial
    buffers as `doubles` long (0: their real size), so that a smaller value makes them fire without

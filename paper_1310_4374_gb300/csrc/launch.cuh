@@ -78,7 +78,7 @@ cudaError_t launch_pack64_groups(const double* x, const double* q, int64_t n_pts
 // far.cu
 int reduce_blocks(int64_t n, int num_sms);
 // validation of the charges (q) or of evaluation points (q null), with their curve keys where
-// `keys` is given; launch_constant finishes the charges' neutrality test
+// `keys` is given; launch_totals finishes the charges' neutrality test
 cudaError_t launch_prepare(const double* x, const double* q, int64_t n, const double d[3], double* partial, int nblk,
                            int* status, uint32_t* keys, cudaStream_t st);
 int mean_blocks(int64_t n, int num_sms);   // grid of launch_box_mean for n charges
@@ -133,8 +133,9 @@ cudaError_t launch_sum_far64(const FarArgs& f, const NearSlots& a, const double*
 int64_t sym_limit(const NearSymLaunch& S);   // doubles of the partial buffer as the debug checks see it
 constexpr int kSlotWarps = 8;
 
-// Debug builds (-DPSUM_DEBUG_CHECKS=1) check every write and read of the pair kernels'
-// partial sums against the buffer's size: an access outside it is skipped and flagged in the
+// Debug builds (-DPSUM_DEBUG_CHECKS=1) check the pair kernels' writes of their partial sums (the one-sided
+// float64 kernel's aside) and the symmetric reductions' and the far field's reads of them against the
+// buffer's size: an access outside it is skipped and flagged in the
 // launch's status words (kStatBounds, PSUM_ERR_INTERNAL at psum_sync) instead of faulting.
 __device__ __forceinline__ bool debug_in_range(int64_t off, int64_t n, int64_t limit, int* status, int n_status) {
 #if PSUM_DEBUG_CHECKS

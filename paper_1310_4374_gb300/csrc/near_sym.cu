@@ -1196,8 +1196,10 @@ cudaError_t launch_sym_reduce(const double* partial, int64_t n_valid, const Near
 }
 
 // Three resident CTAs, from kNear64sTiles tiles on four.  With the pairs of a warp overlapping, the fourth adds
-// 1% where the pair sum is all (12 001 charges 27.7 ms, 28.3 with three); below, the registers are better left
-// to a CTA of the check sums, which fill the integer pipes' idle slots (4096 charges 3.32 ms, 3.45 with four).
+// 1 to 2% where the pair sum is all; below, the registers are better left to a CTA of the check sums, which fill the
+// integer pipes' idle slots.  Evaluations with four against three: 8 tiles 1.04 to 1.09 times the time, 16 to 32
+// 1.01 to 1.03 (4096 charges 3.43 and 3.36 ms), 36 to 48 0.99 to 1.006 either way, 52 and 56 0.97 to 0.99, 64 to 80
+// 0.99 to 1.006, 94 0.98 to 0.99 (12 032 charges 27.5 and 28.0 ms): the line may lie anywhere from 36 to 51.
 constexpr int64_t kNear64sTiles = 48;
 using Near64sKernel = void (*)(Near64SymArgs);
 Near64sKernel near64s_instance(int64_t n_tiles) { return n_tiles >= kNear64sTiles ? k_near64s<4> : k_near64s<3>; }
