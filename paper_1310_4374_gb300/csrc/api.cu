@@ -152,6 +152,7 @@ size_t layout(Plan& pl, int64_t N, char* base, Layout& L, bool backward = false,
         if (g_cap > 0 && gmax > g_cap) gmax = g_cap;
         L.Ln = near_partition(L.n_tiles, L.n_chunks, n_img, gmax, ipc);
         L.Ln.tab.one.tau2 = coincident_r2(pl.opt.d);
+        L.Ln.two_per_sm = g_cap > 0 && gmax <= 2 * (int64_t)pl.num_sms;
         // check sums: the 2M points with the block's images, or the M points with their
         // class's two image layers
         const bool layers = pl.lc_tiles > 0;

@@ -733,6 +733,12 @@ size_t near32_dyn_smem(int n_img, bool trimmed, bool grad, int n_cls) {
     return head + (trimmed ? sizeof(float4) * 4 * kNearChunk : 0);   // compacted sources (hi, lo parts)
 }
 
+// A launch of at most two CTAs an SM, one work item each (the allocation-free entry): where the mean or the check
+// sums still hold part of an SM, its CTAs land four on an SM and leave others idle.  With 48 KB of dynamic beside 31 to
+// 37 KB of static shared memory no more than two fit.  FP32C, 14 000 charges 5.63 -> 3.03 ms, 18 000 7.8 to 8.5 -> 4.94,
+// 32 768 15.6 (29.3 without the mean condition -> 15.6); float-float, 10 000 charges 15.4 -> 12.5 ms.
+constexpr size_t kTwoPerSmSmem = 48 * 1024;
+
 cudaError_t launch_near32(bool grad, const float4* src_hi, const float4* src_lo, const double* src_org,
                           const float4* tgt_hi, const float4* tgt_lo, const double* tgt_org, const double* shifts,
                           double* partial, const NearPlanLaunch& L, cudaStream_t st, int variant,
@@ -765,7 +771,8 @@ cudaError_t launch_near32(bool grad, const float4* src_hi, const float4* src_lo,
     a.grp_sub = grp_sub;
     a.img_w = img_w;
     a.n_cls = n_cls;
-    const size_t smem = near32_dyn_smem(L.max_img, Rb > 0.0, grad, n_cls);
+    size_t smem = near32_dyn_smem(L.max_img, Rb > 0.0, grad, n_cls);
+    if (L.two_per_sm && smem < kTwoPerSmSmem) smem = kTwoPerSmSmem;
     if (!L.counter) return cudaErrorInvalidValue;
     const cudaError_t e = L.zeroed ? cudaSuccess : cudaMemsetAsync(L.counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;

@@ -512,6 +512,7 @@ struct NearPlanLaunch {
     int64_t W;                    // work items
     int* counter = nullptr;       // device int, zeroed by the launcher before each launch
     bool zeroed = false;          // ... unless the caller's own stream order has zeroed it already
+    bool two_per_sm = false;      // float32: CTAs held to two an SM (near.cu, kTwoPerSmSmem)
     int* status = nullptr;        // device error words the pair kernel may flag (kStatTimeout)
     int n_status = 0;
     int inject = 0;               // test hook: arm the chunk-copy barrier for bytes that never come
